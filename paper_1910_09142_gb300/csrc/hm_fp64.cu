@@ -23,6 +23,7 @@
 
 #include "hm_block.cuh"
 #include "hm_internal.h"
+#include "hm_transfer.cuh"
 
 namespace hm {
 
@@ -37,6 +38,14 @@ struct GemmSmem {
   double b[TK][TN + 1];
 };
 
+// Shared memory of the measurement, susceptibility and collapse kernels.
+struct TransferSh {
+  tr::Tabs tab;
+  double red[NT / 32 * 3];
+  double scal[2];
+  int32_t ival;
+};
+
 struct Shared {
   GemmSmem g;
   double red[NT / 32][4];
@@ -48,31 +57,6 @@ __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
-}
-
-// Block-wide sum of up to 3 values; result broadcast to every thread.
-__device__ void block_sum3(double& x, double& y, double& z, Shared& sh) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  x = warp_sum(x);
-  y = warp_sum(y);
-  z = warp_sum(z);
-  __syncthreads();
-  if (lane == 0) {
-    sh.red[warp][0] = x;
-    sh.red[warp][1] = y;
-    sh.red[warp][2] = z;
-  }
-  __syncthreads();
-  double a = 0, b = 0, c = 0;
-  for (int w = 0; w < NT / 32; ++w) {
-    a += sh.red[w][0];
-    b += sh.red[w][1];
-    c += sh.red[w][2];
-  }
-  x = a;
-  y = b;
-  z = c;
-  __syncthreads();
 }
 
 // C[M x N] = alpha op(A) op(B) (+ beta C), row-major.  TA: A stored K x M.
@@ -464,164 +448,12 @@ __global__ void __launch_bounds__(NT) evolve_fp64_kernel(BatchArg b, OutArg o) {
   }
 }
 
-// ---------------------------------------------------------------------------
-// Transfer matrices (steps 3 and 4).
-// ---------------------------------------------------------------------------
-
-// Eout[cr x cr] = sum_{s,t} O[s][t] A^{sT} Ein A^t   (O == nullptr: identity).
-// Z: cl x 3cr scratch.  Ein/Eout are row-major, bra index first.
-__device__ void cta_transfer(const double* Ein, const double* A, int cl, int cr, const double* O,
-                             double* Eout, double* Z, Shared& sh) {
-  if (threadIdx.x == 0) sh.scal[4] += 6.0 * cl * cl * cr + 6.0 * cl * cr * cr;
-  cta_gemm<false, false>(cl, 3 * cr, cl, 1.0, Ein, cl, A, 3 * cr, 0.0, Z, 3 * cr, sh.g);
-  if (O) {
-    for (int e = threadIdx.x; e < cl * cr; e += NT) {
-      const int i = e / cr, r = e % cr;
-      double* z = Z + (size_t)i * 3 * cr + r;
-      const double z0 = z[0], z1 = z[cr], z2 = z[2 * cr];
-      z[0] = O[0] * z0 + O[1] * z1 + O[2] * z2;
-      z[cr] = O[3] * z0 + O[4] * z1 + O[5] * z2;
-      z[2 * cr] = O[6] * z0 + O[7] * z1 + O[8] * z2;
-    }
-    __syncthreads();
-  }
-  cta_gemm<true, false>(cr, cr, 3 * cl, 1.0, A, cr, Z, cr, 0.0, Eout, cr, sh.g);
-}
-
-__device__ __constant__ double kSz[9] = {1, 0, 0, 0, 0, 0, 0, 0, -1};
-// S+ = sqrt(2) (|+1><0| + |0><-1|); S- its transpose (basis m = +1, 0, -1)
-__device__ __constant__ double kSp[9] = {0, 1.4142135623730951, 0, 0, 0, 1.4142135623730951, 0, 0, 0};
-__device__ __constant__ double kSm[9] = {0, 0, 0, 1.4142135623730951, 0, 0, 0, 1.4142135623730951, 0};
-// Right environment through one site: Rout[i, j] = sum_s A^s Rin A^{sT}
-// (Rin cr x cr, Rout cl x cl).  Y: 3cl x cr scratch.
-__device__ void cta_rtransfer(const double* Rin, const double* A, int cl, int cr, double* Rout, double* Y,
-                              Shared& sh) {
-  if (threadIdx.x == 0) sh.scal[4] += 12.0 * cl * cr * cr;
-  cta_gemm<false, false>(3 * cl, cr, cr, 1.0, A, cr, Rin, cr, 0.0, Y, cr, sh.g);
-  cta_gemm<false, true>(cl, cl, 3 * cr, 1.0, Y, 3 * cr, A, 3 * cr, 0.0, Rout, cl, sh.g);
-}
-
-// Charge blocks of the transfer matrices (Sec. II.C).  A bond's indices are
-// grouped by S^z charge, so a charge is one run [start, start + len) of the
-// bond.  For a state of definite total S^z an environment E[i, j] (bra i,
-// ket j) is nonzero only where q_i - q_j = D, its charge shift: 0 for the
-// plain environment, sigma for one S^+ inserted on a leg of sign sigma,
-// -sigma for S^-.  Dense-mode chains have every charge 0: one run, D = 0,
-// and these reduce to the plain dense transfers.
-__device__ void charge_run(const int16_t* q, int n, int Q, int* start, int* len) {
-  int lo = 0, hi = n;
-  while (lo < hi) {                       // first index with q >= Q
-    const int mid = (lo + hi) >> 1;
-    if (q[mid] < Q) lo = mid + 1;
-    else hi = mid;
-  }
-  int e = lo;
-  while (e < n && q[e] == Q) ++e;
-  *start = lo;
-  *len = e - lo;
-}
-
-// Left environment through site pos with operator O (nullptr: identity;
-// O[s][t] = <s|O|t>, nonzero only for m(s) - m(t) = dO):
-// Eout[i', j'] = sum_{s,t} O[s][t] sum_{i,j} A[i,s,i'] Ein[i,j] A[j,t,j'],
-// computed only on the charge blocks it can fill.  Ein has shift D; the
-// result has shift D + sigma dO (returned).  Z: scratch of cl x cr doubles.
-__device__ int cta_transfer_blk(const ChainDev* c, int pos, const double* Ein, int D, const double* O, int dO,
-                                double* Eout, double* Z, Shared& sh) {
-  const int cl = c->chi[pos], cr = c->chi[pos + 1];
-  const double* A = c->site[pos];
-  const int16_t* qL = c->qn + (size_t)pos * c->chi_cap;
-  const int16_t* qR = qL + c->chi_cap;
-  const int sg = c->sgn[pos];
-  const int D2 = D + sg * dO;
-  for (int e = threadIdx.x; e < cr * cr; e += NT) Eout[e] = 0.0;
-  __syncthreads();
-  double fl = 0.0;
-  for (int b0 = 0; b0 < cr;) {
-    int bs, bl;
-    charge_run(qR, cr, qR[b0], &bs, &bl);     // bra run of the right bond
-    const int Qb = qR[b0], Qk = Qb - D2;
-    b0 = bs + bl;
-    int ks, kl;
-    charge_run(qR, cr, Qk, &ks, &kl);         // ket run
-    if (kl == 0) continue;
-    for (int s1 = 0; s1 < 3; ++s1) {
-      int is, il;
-      charge_run(qL, cl, Qb - sg * (1 - s1), &is, &il);
-      if (il == 0) continue;
-      bool first = true;
-      for (int t1 = 0; t1 < 3; ++t1) {
-        const double w = O ? O[3 * s1 + t1] : (s1 == t1 ? 1.0 : 0.0);
-        if (w == 0.0) continue;
-        int js, jl;
-        charge_run(qL, cl, Qk - sg * (1 - t1), &js, &jl);
-        if (jl == 0) continue;
-        // Z (il x kl) (+)= w Ein[i-run, j-run] A[j-run, t1, k-run]
-        cta_gemm<false, false>(il, kl, jl, w, Ein + (size_t)is * cl + js, cl, A + (size_t)(3 * js + t1) * cr + ks,
-                               3 * cr, first ? 0.0 : 1.0, Z, kl, sh.g);
-        fl += 2.0 * il * jl * kl;
-        first = false;
-      }
-      if (first) continue;
-      // Eout[b-run, k-run] += A[i-run, s1, b-run]^T Z
-      cta_gemm<true, false>(bl, kl, il, 1.0, A + (size_t)(3 * is + s1) * cr + bs, 3 * cr, Z, kl, 1.0,
-                            Eout + (size_t)bs * cr + ks, cr, sh.g);
-      fl += 2.0 * il * bl * kl;
-    }
-  }
-  if (threadIdx.x == 0) sh.scal[4] += fl;
-  __syncthreads();
-  return D2;
-}
-
-// Plain right environment through site pos (shift 0):
-// Rout[i, j] = sum_s sum_{a,b} A[i,s,a] Rin[a,b] A[j,s,b], block by block.
-// Y: scratch of cl x cr doubles.
-__device__ void cta_rtransfer_blk(const ChainDev* c, int pos, const double* Rin, double* Rout, double* Y, Shared& sh) {
-  const int cl = c->chi[pos], cr = c->chi[pos + 1];
-  const double* A = c->site[pos];
-  const int16_t* qL = c->qn + (size_t)pos * c->chi_cap;
-  const int16_t* qR = qL + c->chi_cap;
-  const int sg = c->sgn[pos];
-  for (int e = threadIdx.x; e < cl * cl; e += NT) Rout[e] = 0.0;
-  __syncthreads();
-  double fl = 0.0;
-  for (int i0 = 0; i0 < cl;) {
-    int is, il;
-    charge_run(qL, cl, qL[i0], &is, &il);
-    const int Q = qL[i0];
-    i0 = is + il;
-    for (int s1 = 0; s1 < 3; ++s1) {
-      int as, al;
-      charge_run(qR, cr, Q + sg * (1 - s1), &as, &al);
-      if (al == 0) continue;
-      // Y (il x al) = A[i-run, s1, a-run] Rin[a-run, a-run]
-      cta_gemm<false, false>(il, al, al, 1.0, A + (size_t)(3 * is + s1) * cr + as, 3 * cr, Rin + (size_t)as * cr + as,
-                             cr, 0.0, Y, al, sh.g);
-      // Rout[i-run, i-run] += Y A[i-run, s1, a-run]^T
-      cta_gemm<false, true>(il, il, al, 1.0, Y, al, A + (size_t)(3 * is + s1) * cr + as, 3 * cr, 1.0,
-                            Rout + (size_t)is * cl + is, cl, sh.g);
-      fl += 2.0 * il * al * al + 2.0 * il * il * al;
-    }
-  }
-  if (threadIdx.x == 0) sh.scal[4] += fl;
-  __syncthreads();
-}
-
-// sum_{k,l} X[k, l] Y[k, l] over n entries, block-wide.
-__device__ double cta_dot(const double* X, const double* Y, int n, Shared& sh) {
-  double acc = 0.0, d1 = 0.0, d2 = 0.0;
-  for (int e = threadIdx.x; e < n; e += NT) acc = fma(X[e], Y[e], acc);
-  block_sum3(acc, d1, d2, sh);
-  return acc;
-}
-
 // Step 3 (Sec. I.C.1): <S_i.S_j> and <Sz_i Sz_j> on every measured bond.
 // Right environments are built explicitly from the last site (no reliance on
 // the canonical form), so <psi|psi> is the full contraction and every value
 // is divided by it.
 __global__ void __launch_bounds__(NT) measure_fp64_kernel(BatchArg b, OutArg o) {
-  __shared__ Shared sh;
+  __shared__ TransferSh sh;
   ChainDev* c = b.c[blockIdx.x];
   const int tid = threadIdx.x;
   double* out = o.obs + (size_t)blockIdx.x * o.n_obs;
@@ -636,10 +468,8 @@ __global__ void __launch_bounds__(NT) measure_fp64_kernel(BatchArg b, OutArg o) 
   double* Et = c->env_ws + 7 * cc;         // cc
   double* Rp[2] = {c->env_ws + 8 * cc, c->env_ws + 9 * cc};
   double* Rend = c->env_ws + 10 * cc;      // one cc slot per distinct measured end site
-  if (tid == 0) {
-    Rp[0][0] = 1.0;
-    sh.scal[4] = 0.0;
-  }
+  long long fma_n = 0;
+  if (tid == 0) Rp[0][0] = 1.0;
   __syncthreads();
   // right sweep: R(pos) = environment of sites >= pos; keep R(b + 1) per end b
   int rc = 0;
@@ -652,7 +482,7 @@ __global__ void __launch_bounds__(NT) measure_fp64_kernel(BatchArg b, OutArg o) 
       }
     }
     __syncthreads();
-    cta_rtransfer_blk(c, pos, Rp[rc], Rp[rc ^ 1], Z, sh);
+    tr::right_transfer<NT>(c, pos, Rp[rc], 0, tr::op_id(), Rp[rc ^ 1], Z, false, false, sh.tab, fma_n);
     rc ^= 1;
   }
   const double nrm = Rp[rc][0];            // <psi|psi>
@@ -666,9 +496,8 @@ __global__ void __launch_bounds__(NT) measure_fp64_kernel(BatchArg b, OutArg o) 
   // S_i.S_j is invariant.  Passes: (Sz Sz), (S+ S-), (S- S+); operator
   // charge shifts dO = 0, +1, -1 and -dO.
   const int frame = c->counters[2];
-  const double* ops1[3] = {kSz, kSp, kSm};
-  const double* ops2[3] = {kSz, kSm, kSp};
-  const int dop[3] = {0, 1, -1};
+  const tr::Op1 ops1[3] = {tr::op_sz(), tr::op_sp(), tr::op_sm()};
+  const tr::Op1 ops2[3] = {tr::op_sz(), tr::op_sm(), tr::op_sp()};
   int bi = 0;
   while (bi < c->n_meas) {
     const int a = c->meas_i[bi];
@@ -676,24 +505,26 @@ __global__ void __launch_bounds__(NT) measure_fp64_kernel(BatchArg b, OutArg o) 
     while (bend < c->n_meas && c->meas_i[bend] == a) ++bend;
     const int blast = c->meas_j[bend - 1];
     while (pos < a) {
-      cta_transfer_blk(c, pos, Lp[cur], 0, nullptr, 0, Lp[cur ^ 1], Z, sh);
+      tr::left_transfer<NT>(c, pos, Lp[cur], 0, tr::op_id(), Lp[cur ^ 1], Z, false, false, sh.tab, fma_n);
       cur ^= 1;
       ++pos;
     }
     double vals[3][8];   // up to 8 bonds per start site
     for (int o1 = 0; o1 < 3; ++o1) {
       int ec = 0;
-      int D = cta_transfer_blk(c, a, Lp[cur], 0, ops1[o1], dop[o1], Ep[ec], Z, sh);
+      int D = tr::left_transfer<NT>(c, a, Lp[cur], 0, ops1[o1], Ep[ec], Z, false, false, sh.tab, fma_n);
       for (int kk = a + 1; kk <= blast; ++kk) {
         for (int q = bi; q < bend; ++q) {
           if (c->meas_j[q] == kk) {
-            cta_transfer_blk(c, kk, Ep[ec], D, ops2[o1], -dop[o1], Et, Z, sh);
-            const int n2 = c->chi[kk + 1] * c->chi[kk + 1];
-            vals[o1][q - bi] = cta_dot(Et, Rend + (size_t)c->meas_slot[q] * cc, n2, sh);
+            const int D2 = tr::left_transfer<NT>(c, kk, Ep[ec], D, ops2[o1], Et, Z, false, false, sh.tab, fma_n);
+            // the right environment has shift 0: another shift closes to 0
+            vals[o1][q - bi] = D2 != 0 ? 0.0
+                                       : tr::block_dot<NT>(sh.tab, 0, Et, Rend + (size_t)c->meas_slot[q] * cc,
+                                                           c->chi[kk + 1], sh.red);
           }
         }
         if (kk < blast) {
-          D = cta_transfer_blk(c, kk, Ep[ec], D, nullptr, 0, Ep[ec ^ 1], Z, sh);
+          D = tr::left_transfer<NT>(c, kk, Ep[ec], D, tr::op_id(), Ep[ec ^ 1], Z, false, false, sh.tab, fma_n);
           ec ^= 1;
         }
       }
@@ -712,49 +543,8 @@ __global__ void __launch_bounds__(NT) measure_fp64_kernel(BatchArg b, OutArg o) 
   }
   if (tid == 0) {
     out[0] = E_est;
-    c->stats[ST_TRANSFER] += sh.scal[4];
+    c->stats[ST_TRANSFER] += 2.0 * (double)fma_n;
   }
-}
-
-// Right environment with an operator on this site, accumulated:
-// Rout <- acc * Rout + sum_{s,t} O[s][t] A^s Rin A^{tT}  (O == nullptr: identity;
-// bra index s first).  Rin cr x cr, Rout cl x cl, Y: 3cl x cr scratch.
-__device__ void cta_rtransfer_op(const double* Rin, const double* A, int cl, int cr, const double* O, double* Rout,
-                                 double* Y, double acc, Shared& sh) {
-  if (threadIdx.x == 0) sh.scal[4] += 12.0 * cl * cr * cr;
-  cta_gemm<false, false>(3 * cl, cr, cr, 1.0, A, cr, Rin, cr, 0.0, Y, cr, sh.g);
-  if (O) {
-    for (int e = threadIdx.x; e < cl * cr; e += NT) {
-      const int i = e / cr, r = e % cr;
-      double* y = Y + (size_t)i * 3 * cr + r;
-      const double y0 = y[0], y1 = y[cr], y2 = y[2 * cr];
-      y[0] = O[0] * y0 + O[3] * y1 + O[6] * y2;
-      y[cr] = O[1] * y0 + O[4] * y1 + O[7] * y2;
-      y[2 * cr] = O[2] * y0 + O[5] * y1 + O[8] * y2;
-    }
-    __syncthreads();
-  }
-  cta_gemm<false, true>(cl, cl, 3 * cr, 1.0, Y, 3 * cr, A, 3 * cr, acc, Rout, cl, sh.g);
-}
-
-// Left environment with an operator on this site, accumulated:
-// Eout <- acc * Eout + sum_{s,t} O[s][t] A^{sT} Ein A^t.
-__device__ void cta_transfer_acc(const double* Ein, const double* A, int cl, int cr, const double* O, double* Eout,
-                                 double* Z, double acc, Shared& sh) {
-  if (threadIdx.x == 0) sh.scal[4] += 6.0 * cl * cl * cr + 6.0 * cl * cr * cr;
-  cta_gemm<false, false>(cl, 3 * cr, cl, 1.0, Ein, cl, A, 3 * cr, 0.0, Z, 3 * cr, sh.g);
-  if (O) {
-    for (int e = threadIdx.x; e < cl * cr; e += NT) {
-      const int i = e / cr, r = e % cr;
-      double* z = Z + (size_t)i * 3 * cr + r;
-      const double z0 = z[0], z1 = z[cr], z2 = z[2 * cr];
-      z[0] = O[0] * z0 + O[1] * z1 + O[2] * z2;
-      z[cr] = O[3] * z0 + O[4] * z1 + O[5] * z2;
-      z[2 * cr] = O[6] * z0 + O[7] * z1 + O[8] * z2;
-    }
-    __syncthreads();
-  }
-  cta_gemm<true, false>(cr, cr, 3 * cl, 1.0, A, cr, Z, cr, acc, Eout, cr, sh.g);
 }
 
 // Uniform susceptibility (Eq. sus, Sec. II.A): the double sum
@@ -765,8 +555,12 @@ __device__ void cta_transfer_acc(const double* Ein, const double* A, int cl, int
 // (R(a+1)); a left sweep carries the mirrored sums L, L_z, L_+, L_- and
 // closes, at each region site a, O_a on L against the right sums (b > a)
 // and the left sums with O_a against R (b < a).  Linear in the chain length.
+// Charge blocks throughout: S^z leaves an environment's shift at 0, S^+ and
+// S^- move it by the sign of the physical legs.  A chain whose physical
+// positions hold legs of different signs (explicit op lists can leave it so)
+// mixes shifts in one sum and is contracted densely.
 __global__ void __launch_bounds__(NT) susceptibility_fp64_kernel(BatchArg b, OutArg o) {
-  __shared__ Shared sh;
+  __shared__ TransferSh sh;
   ChainDev* c = b.c[blockIdx.x];
   const int tid = threadIdx.x;
   double* out = o.obs + blockIdx.x;
@@ -789,21 +583,33 @@ __global__ void __launch_bounds__(NT) susceptibility_fp64_kernel(BatchArg b, Out
   double* Et = c->env_ws + 19 * cc;
   double* store = c->env_ws + 20 * cc;     // 4 cc per region site
   // right sums carry S^z, S^-, S^+ ; left sums carry S^z, S^+, S^-
-  const double* ropk[4] = {nullptr, kSz, kSm, kSp};
-  const double* lopk[4] = {nullptr, kSz, kSp, kSm};
+  const tr::Op1 ropk[4] = {tr::op_id(), tr::op_sz(), tr::op_sm(), tr::op_sp()};
+  const tr::Op1 lopk[4] = {tr::op_id(), tr::op_sz(), tr::op_sp(), tr::op_sm()};
+  // the one sign of the physical legs; dense when there is none
+  int leg = 0;
+  bool dense = false;
+  for (int pos = 0; pos < c->n_sites; ++pos) {
+    if (c->site_kind[pos] == SITE_ANC) continue;
+    if (leg == 0) leg = c->sgn[pos];
+    if (c->sgn[pos] != leg || leg == 0) dense = true;
+  }
+  if (dense) leg = 0;
+  // shifts of the right sums (bra minus ket charge) and of the left ones
+  const int rD[4] = {0, 0, leg, -leg};
+  const int lD[4] = {0, 0, leg, -leg};
+  long long fma_n = 0;
   if (tid == 0) {
     Rc[0][0] = 1.0;
     Rc[1][0] = Rc[2][0] = Rc[3][0] = 0.0;
     Lc[0][0] = 1.0;
     Lc[1][0] = Lc[2][0] = Lc[3][0] = 0.0;
-    sh.scal[4] = 0.0;
   }
   __syncthreads();
   const int n = c->n_sites;
   int amax = -1;
   for (int s2 = 0; s2 < c->n_region; ++s2) amax = max(amax, c->region[s2]);
   for (int pos = n - 1; pos >= 0; --pos) {
-    const int cl = c->chi[pos], cr = c->chi[pos + 1];
+    const int cr = c->chi[pos + 1];
     int slot = -1;
     for (int s2 = 0; s2 < c->n_region; ++s2)
       if (c->region[s2] == pos) slot = s2;
@@ -812,12 +618,10 @@ __global__ void __launch_bounds__(NT) susceptibility_fp64_kernel(BatchArg b, Out
         for (int e = tid; e < cr * cr; e += NT) store[(size_t)(4 * slot + qq) * cc + e] = Rc[qq][e];
       __syncthreads();
     }
-    const double* A = c->site[pos];
     const bool phys = c->site_kind[pos] != SITE_ANC;
-    cta_rtransfer_op(Rc[0], A, cl, cr, nullptr, Rn[0], Z, 0.0, sh);
-    for (int qq = 1; qq < 4; ++qq) {
-      cta_rtransfer_op(Rc[qq], A, cl, cr, nullptr, Rn[qq], Z, 0.0, sh);
-      if (phys) cta_rtransfer_op(Rc[0], A, cl, cr, ropk[qq], Rn[qq], Z, 1.0, sh);
+    for (int qq = 0; qq < 4; ++qq) {
+      tr::right_transfer<NT>(c, pos, Rc[qq], rD[qq], tr::op_id(), Rn[qq], Z, false, dense, sh.tab, fma_n);
+      if (qq > 0 && phys) tr::right_transfer<NT>(c, pos, Rc[0], 0, ropk[qq], Rn[qq], Z, true, dense, sh.tab, fma_n);
     }
     for (int qq = 0; qq < 4; ++qq) {
       double* t = Rc[qq];
@@ -828,8 +632,7 @@ __global__ void __launch_bounds__(NT) susceptibility_fp64_kernel(BatchArg b, Out
   const double nrm = Rc[0][0];             // <psi|psi>
   double total = 0.0;
   for (int pos = 0; pos <= amax; ++pos) {
-    const int cl = c->chi[pos], cr = c->chi[pos + 1];
-    const double* A = c->site[pos];
+    const int cr = c->chi[pos + 1];
     int slot = -1;
     for (int s2 = 0; s2 < c->n_region; ++s2)
       if (c->region[s2] == pos) slot = s2;
@@ -838,29 +641,22 @@ __global__ void __launch_bounds__(NT) susceptibility_fp64_kernel(BatchArg b, Out
       const double* Rz = R0 + cc;
       const double* Rm = R0 + 2 * cc;
       const double* Rp = R0 + 3 * cc;
-      const int n2 = cr * cr;
-      // b > a: O_a on L, closed against the right sums
-      cta_transfer_acc(Lc[0], A, cl, cr, kSz, Et, Z, 0.0, sh);
-      total += cta_dot(Et, Rz, n2, sh);
-      cta_transfer_acc(Lc[0], A, cl, cr, kSp, Et, Z, 0.0, sh);
-      total += 0.5 * cta_dot(Et, Rm, n2, sh);
-      cta_transfer_acc(Lc[0], A, cl, cr, kSm, Et, Z, 0.0, sh);
-      total += 0.5 * cta_dot(Et, Rp, n2, sh);
-      // b < a: left sums with O_a, closed against R
-      cta_transfer_acc(Lc[1], A, cl, cr, kSz, Et, Z, 0.0, sh);
-      total += cta_dot(Et, R0, n2, sh);
-      cta_transfer_acc(Lc[2], A, cl, cr, kSm, Et, Z, 0.0, sh);
-      total += 0.5 * cta_dot(Et, R0, n2, sh);
-      cta_transfer_acc(Lc[3], A, cl, cr, kSp, Et, Z, 0.0, sh);
-      total += 0.5 * cta_dot(Et, R0, n2, sh);
+      // b > a: O_a on L, closed against the right sums; b < a: the left sums
+      // with O_a, closed against R
+      const tr::Op1 oa[6] = {tr::op_sz(), tr::op_sp(), tr::op_sm(), tr::op_sz(), tr::op_sm(), tr::op_sp()};
+      const double* right[6] = {Rz, Rm, Rp, R0, R0, R0};
+      for (int u = 0; u < 6; ++u) {
+        const int from = u < 3 ? 0 : u - 2;
+        const int D = tr::left_transfer<NT>(c, pos, Lc[from], lD[from], oa[u], Et, Z, false, dense, sh.tab, fma_n);
+        total += (u % 3 == 0 ? 1.0 : 0.5) * tr::block_dot<NT>(sh.tab, D, Et, right[u], cr, sh.red);
+      }
       total += 2.0 * nrm;                  // b = a: S.S = s(s+1) = 2
     }
     if (pos == amax) break;
     const bool phys = c->site_kind[pos] != SITE_ANC;
-    cta_transfer_acc(Lc[0], A, cl, cr, nullptr, Ln[0], Z, 0.0, sh);
-    for (int qq = 1; qq < 4; ++qq) {
-      cta_transfer_acc(Lc[qq], A, cl, cr, nullptr, Ln[qq], Z, 0.0, sh);
-      if (phys) cta_transfer_acc(Lc[0], A, cl, cr, lopk[qq], Ln[qq], Z, 1.0, sh);
+    for (int qq = 0; qq < 4; ++qq) {
+      tr::left_transfer<NT>(c, pos, Lc[qq], lD[qq], tr::op_id(), Ln[qq], Z, false, dense, sh.tab, fma_n);
+      if (qq > 0 && phys) tr::left_transfer<NT>(c, pos, Lc[0], 0, lopk[qq], Ln[qq], Z, true, dense, sh.tab, fma_n);
     }
     for (int qq = 0; qq < 4; ++qq) {
       double* t = Lc[qq];
@@ -870,7 +666,7 @@ __global__ void __launch_bounds__(NT) susceptibility_fp64_kernel(BatchArg b, Out
   }
   if (tid == 0) {
     *out = total / nrm;
-    c->stats[ST_TRANSFER] += sh.scal[4];
+    c->stats[ST_TRANSFER] += 2.0 * (double)fma_n;
   }
 }
 
@@ -925,7 +721,7 @@ __device__ void basis_rows(const ChainDev* c, int basis, double B[9]) {
 // basis of sample n (Sec. I.C.1 step 4); cluster sites are traced out, which
 // turns the boundary vector into a density matrix (Eq. detailbalance1).
 __global__ void __launch_bounds__(NT) collapse_fp64_kernel(BatchArg b, OutArg o) {
-  __shared__ Shared sh;
+  __shared__ TransferSh sh;
   ChainDev* c = b.c[blockIdx.x];
   const int tid = threadIdx.x;
   if (*(volatile int32_t*)c->status != 0) return;
@@ -939,30 +735,26 @@ __global__ void __launch_bounds__(NT) collapse_fp64_kernel(BatchArg b, OutArg o)
   const int64_t cc = (int64_t)c->chi_cap * c->chi_cap;
   double* R[2] = {c->env_ws, c->env_ws + cc};
   double* X = c->env_ws + 2 * cc;      // cl x 3cr
-  double* At = c->env_ws + 5 * cc;     // cl x cr
   double* Y = c->env_ws + 6 * cc;      // cl x cr
+  long long fma_n = 0;
   int cur = 0;
   bool vec_mode = true;
-  if (tid == 0) {
-    R[0][0] = 1.0;                     // v = [1]
-    sh.scal[4] = 0.0;
-  }
+  if (tid == 0) R[0][0] = 1.0;           // v = [1]
   __syncthreads();
   int e_ord = 0;
   double logp = 0.0;
   for (int k = 0; k < c->n_sites; ++k) {
     const double* A = c->site[k];
     const int cl = c->chi[k], cr = c->chi[k + 1];
+    const int sg = c->sgn[k];
+    const int16_t* qL = c->qn + (size_t)k * c->chi_cap;
+    const int16_t* qR = qL + c->chi_cap;
+    tr::build_tabs<NT>(c, k, false, sh.tab);
     if (c->site_kind[k] == SITE_ENV) {
       double q[3] = {0.0, 0.0, 0.0};
+      // X[i, s, r] = sum_l rho[i, l] A[l, s, r]; a vector boundary is one row
+      tr::row_times_site<NT>(c, k, sh.tab, R[cur], vec_mode ? 1 : cl, X);
       if (vec_mode) {
-        // X[(s r)] = sum_l v[l] A[l, s, r]
-        for (int e = tid; e < 3 * cr; e += NT) {
-          double acc = 0.0;
-          for (int l = 0; l < cl; ++l) acc = fma(R[cur][l], A[(size_t)l * 3 * cr + e], acc);
-          X[e] = acc;
-        }
-        __syncthreads();
         for (int r = tid; r < cr; r += NT) {
           const double x0 = X[r], x1 = X[cr + r], x2 = X[2 * cr + r];
           for (int bb = 0; bb < 3; ++bb) {
@@ -971,21 +763,34 @@ __global__ void __launch_bounds__(NT) collapse_fp64_kernel(BatchArg b, OutArg o)
           }
         }
       } else {
-        cta_gemm<false, false>(cl, 3 * cr, cl, 1.0, R[cur], cl, A, 3 * cr, 0.0, X, 3 * cr, sh.g);
+        // q_b = sum_{s,t} B[b][s] B[b][t] G[s][t], G[s][t] = sum_{i,r} A[i,s,r] X[i,t,r]:
+        // an (i, r) whose charges allow no s is skipped, and the others cost one
+        // product per t instead of both basis rotations
+        double G[9] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
         for (int e = tid; e < cl * cr; e += NT) {
           const int i = e / cr, r = e % cr;
+          const int m = (qR[r] - qL[i]) * sg;            // m(s) of the one allowed s (sg = 0: all)
+          if (sg != 0 && (m < -1 || m > 1)) continue;
           const double* a = A + (size_t)i * 3 * cr + r;
           const double* x = X + (size_t)i * 3 * cr + r;
-          const double a0 = a[0], a1 = a[cr], a2 = a[2 * cr];
           const double x0 = x[0], x1 = x[cr], x2 = x[2 * cr];
-          for (int bb = 0; bb < 3; ++bb) {
-            const double at = B[3 * bb] * a0 + B[3 * bb + 1] * a1 + B[3 * bb + 2] * a2;
-            const double yt = B[3 * bb] * x0 + B[3 * bb + 1] * x1 + B[3 * bb + 2] * x2;
-            q[bb] = fma(at, yt, q[bb]);
+#pragma unroll
+          for (int s = 0; s < 3; ++s) {
+            if (sg != 0 && m != blk::mval(s)) continue;
+            const double as = a[s * cr];
+            G[3 * s] = fma(as, x0, G[3 * s]);
+            G[3 * s + 1] = fma(as, x1, G[3 * s + 1]);
+            G[3 * s + 2] = fma(as, x2, G[3 * s + 2]);
           }
         }
+#pragma unroll
+        for (int bb = 0; bb < 3; ++bb)
+#pragma unroll
+          for (int s = 0; s < 3; ++s)
+            q[bb] = fma(B[3 * bb + s], B[3 * bb] * G[3 * s] + B[3 * bb + 1] * G[3 * s + 1] + B[3 * bb + 2] * G[3 * s + 2],
+                        q[bb]);
       }
-      block_sum3(q[0], q[1], q[2], sh);
+      tr::block_sums<NT, 3>(q, sh.red);
       if (tid == 0) {
         const double tot = q[0] + q[1] + q[2];
         int pick = -1;
@@ -999,12 +804,12 @@ __global__ void __launch_bounds__(NT) collapse_fp64_kernel(BatchArg b, OutArg o)
           pick = choose3(p, u);
           if (pick >= 0) pb = p[pick];
         }
-        sh.ival[2] = pick;
+        sh.ival = pick;
         sh.scal[1] = pick >= 0 ? q[pick] : 0.0;
         if (pick >= 0) logp += log(pb);
       }
       __syncthreads();
-      const int pick = sh.ival[2];
+      const int pick = sh.ival;
       const double qb = sh.scal[1];
       if (pick < 0) {
         set_error(c, HM_ERR_NUMERIC, 100000 + k, o.ctx_err);
@@ -1023,14 +828,13 @@ __global__ void __launch_bounds__(NT) collapse_fp64_kernel(BatchArg b, OutArg o)
       } else {
         for (int e = tid; e < cl * cr; e += NT) {
           const int i = e / cr, r = e % cr;
-          const double* a = A + (size_t)i * 3 * cr + r;
           const double* x = X + (size_t)i * 3 * cr + r;
-          At[e] = b0 * a[0] + b1 * a[cr] + b2 * a[2 * cr];
           Y[e] = b0 * x[0] + b1 * x[cr] + b2 * x[2 * cr];
         }
         __syncthreads();
-        cta_gemm<true, false>(cr, cr, cl, 1.0 / qb, At, cr, Y, cr, 0.0, R[cur ^ 1], cr, sh.g);
-        if (tid == 0) sh.scal[4] += 6.0 * cl * cl * cr + 2.0 * cl * cr * cr;
+        const double bv[3] = {b0, b1, b2};
+        tr::site_times_rows<NT>(c, k, sh.tab, bv, 1.0 / qb, Y, 0, cr, R[cur ^ 1]);
+        if (tid == 0) fma_n += (cl + cr) * tr::site_entries(sh.tab, sg);
       }
       cur ^= 1;
       ++e_ord;
@@ -1042,7 +846,10 @@ __global__ void __launch_bounds__(NT) collapse_fp64_kernel(BatchArg b, OutArg o)
         cur ^= 1;
         vec_mode = false;
       }
-      cta_transfer(R[cur], A, cl, cr, nullptr, R[cur ^ 1], X, sh);
+      const double one[3] = {1.0, 1.0, 1.0};
+      tr::row_times_site<NT>(c, k, sh.tab, R[cur], cl, X);
+      tr::site_times_rows<NT>(c, k, sh.tab, one, 1.0, X, cr, 3 * cr, R[cur ^ 1]);
+      if (tid == 0) fma_n += (cl + cr) * tr::site_entries(sh.tab, sg);
       cur ^= 1;
     }
   }
@@ -1050,7 +857,7 @@ __global__ void __launch_bounds__(NT) collapse_fp64_kernel(BatchArg b, OutArg o)
     if (o.logp) o.logp[blockIdx.x] = logp;
     c->counters[0] = n_sample + 1;
     c->counters[1] = basis;
-    c->stats[ST_TRANSFER] += sh.scal[4];
+    c->stats[ST_TRANSFER] += 2.0 * (double)fma_n;
   }
 }
 
