@@ -29,6 +29,7 @@
 #pragma once
 
 #include <cstdint>
+#include <cstring>
 
 #include "hm_internal.h"
 
@@ -41,42 +42,129 @@ constexpr int kMaxBlocks = kWin;
 // m(s) of the local basis s = 0, 1, 2 (m = +1, 0, -1).
 __device__ __forceinline__ int mval(int s) { return 1 - s; }
 
-// One output block of a split.
+// One theta block of a split (a middle charge with rows and columns): per
+// local state the first index and the offset in the block's row and column
+// lists, and the charge's run of the middle bond.
+struct InRec {
+  int16_t rst[3], roff[4], cst[3], coff[4];
+  int16_t mst, mlen;
+};
+
+// One output block of a split.  Lengths and offsets are below 3 x 4096.
 struct BlockRec {
-  int32_t Q, mq, nq, trans;               // charge, rows (l a), columns (b r), W holds the transpose
-  int32_t q, p, svoff, pad;               // W is q x p column-major, q >= p; first slot in the value list
-  int32_t rst[3], rlen[3], roff[3];       // per a: first l, count, offset in the row list
-  int32_t cst[3], clen[3], coff[3];       // per b: first r, count, offset in the column list
+  int16_t Q, mq, nq, trans;               // charge, rows (l a), columns (b r), W holds the transpose
+  int16_t q, p;                           // W is q x p column-major, q >= p
+  int16_t rst[3], rlen[3], roff[3];       // per a: first l, count, offset in the row list
+  int16_t cst[3], clen[3], coff[3];       // per b: first r, count, offset in the column list
+  int32_t svoff;                          // first slot in the value list
   int64_t woff, voff;                     // offsets (elements) of the block's W and V
 };
 
-// Split metadata in the chain's meta workspace.
+// Split metadata in the chain's meta workspace (splits of more than kShBlk blocks).
 struct Meta {
-  int32_t tab[3][kWin][2];                // (start, length) of each charge's run: left, middle, right bond
-  int32_t qin[kWin];                      // middle charges with rows and columns (theta blocks)
+  InRec in[kWin];
   BlockRec b[kMaxBlocks];
 };
 
 static_assert(sizeof(Meta) <= kMetaBytes, "meta workspace of a chain");
 
+// Charge-run tables of the three bonds while a split is prepared: (start,
+// end) of each charge of the window.  12 KB of the CTA's scratch memory.
+struct PrepTab {
+  int32_t t[3][kWin][2];
+};
+
+// Records of the usual split (at most 11 blocks measured on the benchmark
+// ladder) stay in shared memory; a split with more keeps all of its records
+// in the meta workspace.
+constexpr int kShBlk = 14;
+
 // Shared scalars of a split (CTA shared memory).
 struct SplitSh {
   int32_t sk, sk1, osk, osk1;             // input and output leg signs of sites k, k+1
-  int32_t qbase, qtop, nin, nblk, ok;
-  int32_t mask[9];                        // per output (a b): input (s1 s2) of its conserved sector
+  int32_t qbase, qtop, nin, nblk, ok, P;  // P: singular values over all blocks
+  int32_t nt[9];                          // per output (a b): terms of its conserved sector
+  int16_t tt[9][9];                       // term: input 3 s1 + s2
+  double G[9][9];                         // term: coefficient
+  float gh[9][9], gl[9][9];               // the coefficient as a binary32 pair hi + lo
   int32_t kk;
   double nrm;
-  double G[81];
+  const InRec* in;
+  const BlockRec* b;
+  double k1;                              // multiply-adds of the theta blocks
+  InRec in_sh[kShBlk];
+  BlockRec b_sh[kShBlk];
 };
 
 struct Seg {
   int32_t start, len;
 };
 
-__device__ __forceinline__ Seg seg_of(const Meta* M, int bond, int qbase, int q) {
+__device__ __forceinline__ Seg seg_of(const PrepTab& T, int bond, int qbase, int q) {
   const int i = q - qbase;
   if (i < 0 || i >= kWin) return {0, 0};   // callers stay within [qbase, qtop + 3]
-  return {M->tab[bond][i][0], M->tab[bond][i][1]};
+  return {T.t[bond][i][0], T.t[bond][i][1] - T.t[bond][i][0]};
+}
+
+// The value of another lane of the warp.
+template <typename T>
+__device__ __forceinline__ T lane_value(T v, int src) {
+  return __shfl_xor_sync(0xffffffffu, v, (threadIdx.x & 31) ^ src);
+}
+
+// Exclusive sum over the lanes of a warp; *total gets the warp's sum.
+__device__ __forceinline__ int lane_prefix(int v, int* total) {
+  const int lane = threadIdx.x & 31;
+  int x = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = lane_value(x, lane >= o ? lane - o : lane);
+    if (lane >= o) x += y;
+  }
+  *total = lane_value(x, 31);
+  return x - v;
+}
+
+// binary32 <-> binary64 by integer instructions: GB300 converts to and from
+// 64-bit types on its binary64 pipe (2 a clock and SM).  Both equal the
+// conversion instruction for every input (zero and normal binary32 values
+// take the integer form, the rest the instruction).
+__device__ __forceinline__ double widen(float f) {
+  const unsigned u = __float_as_uint(f), e = (u >> 23) & 0xffu;
+  if ((u << 1) == 0u || (e != 0u && e != 255u)) {
+    const unsigned hi = (u << 1) == 0u ? u : (u & 0x80000000u) | ((e + 896u) << 20) | ((u >> 3) & 0xfffffu);
+    const unsigned long long b = ((unsigned long long)hi << 32) | (unsigned)(u << 29);
+    double d;
+    memcpy(&d, &b, 8);
+    return d;
+  }
+  return (double)f;
+}
+
+__device__ __forceinline__ float narrow(double d) {
+  unsigned long long b;
+  memcpy(&b, &d, 8);
+  const unsigned hi = (unsigned)(b >> 32), lo = (unsigned)b;
+  const unsigned e = (hi >> 20) & 0x7ffu;
+  if (e > 896u && e < 1151u) {
+    unsigned u = ((e - 896u) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+    const unsigned rest = lo << 3;                       // the bits below, round half to even
+    u += (rest > 0x80000000u || (rest == 0x80000000u && (u & 1u))) ? 1u : 0u;
+    return __uint_as_float((hi & 0x80000000u) | u);
+  }
+  if ((b << 1) == 0ull) return __uint_as_float(hi);
+  return (float)d;
+}
+
+template <typename T>
+__device__ __forceinline__ T from64(double d);
+template <>
+__device__ __forceinline__ double from64<double>(double d) {
+  return d;
+}
+template <>
+__device__ __forceinline__ float from64<float>(double d) {
+  return narrow(d);
 }
 
 // Marks a chain as having no usable charge structure from here on: every
@@ -94,8 +182,10 @@ __device__ void go_dense(ChainDev* c) {
 // Phase A: signs, charge-run tables of the three bonds, the middle charges
 // of the theta blocks and the output blocks with their workspace offsets.
 // Returns false if the chain had to switch to dense mode first (then call again).
+// One thread a candidate charge: a serial loop over them, each step a chain of
+// dependent loads, took as long as the blocks' arithmetic on small bonds.
 template <int NT>
-__device__ bool prepare(ChainDev* c, const OpDev& op, SplitSh& s) {
+__device__ bool prepare(ChainDev* c, const OpDev& op, SplitSh& s, PrepTab& T) {
   const int tid = threadIdx.x;
   const int k = op.k;
   const int chil = c->chi[k], chim = c->chi[k + 1], chir = c->chi[k + 2];
@@ -156,8 +246,8 @@ __device__ bool prepare(ChainDev* c, const OpDev& op, SplitSh& s) {
   const int qb = s.qbase;
   const int span = s.qtop - qb + 4;        // window entries any lookup of this split reaches
   for (int e = tid; e < 3 * span; e += NT) {
-    M->tab[e / span][e % span][0] = 0;
-    M->tab[e / span][e % span][1] = 0;
+    T.t[e / span][e % span][0] = 0;
+    T.t[e / span][e % span][1] = 0;
   }
   __syncthreads();
   const int nall = chil + chim + chir;
@@ -167,71 +257,124 @@ __device__ bool prepare(ChainDev* c, const OpDev& op, SplitSh& s) {
     if (e < chil) bond = 0, i = e, n = chil, q = qL;
     else if (e < chil + chim) bond = 1, i = e - chil, n = chim, q = qM;
     else bond = 2, i = e - chil - chim, n = chir, q = qR;
-    if (i == 0 || q[i] != q[i - 1]) {
-      int j = i + 1;
-      while (j < n && q[j] == q[i]) ++j;
-      M->tab[bond][q[i] - qb][0] = i;
-      M->tab[bond][q[i] - qb][1] = j - i;
-    }
+    const int Q = q[i];
+    if (i == 0 || q[i - 1] != Q) T.t[bond][Q - qb][0] = i;
+    if (i == n - 1 || q[i + 1] != Q) T.t[bond][Q - qb][1] = i + 1;
   }
-  for (int e = tid; e < 81; e += NT) s.G[e] = c->gates[(size_t)op.gate * 81 + e];
   __syncthreads();
-  if (tid < 9) {
-    const int a = tid / 3, b = tid % 3;
-    int msk = 0;
+  if (tid >= 32 && tid < 41) {
+    // conserved sector of the outputs (a b) of the gate, its coefficients also as binary32 pairs
+    const int o = tid - 32, a = o / 3, b = o % 3;
+    const double* g = c->gates + (size_t)op.gate * 81 + o * 9;
+    int n = 0;
     for (int u = 0; u < 9; ++u) {
-      const int s1 = u / 3, s2 = u % 3;
-      if (s.sk * mval(s1) + s.sk1 * mval(s2) == s.osk * mval(a) + s.osk1 * mval(b) && s.G[(3 * a + b) * 9 + u] != 0.0)
-        msk |= 1 << u;
+      const double x = g[u];
+      if (s.sk * mval(u / 3) + s.sk1 * mval(u % 3) == s.osk * mval(a) + s.osk1 * mval(b) && x != 0.0) {
+        s.tt[o][n] = (int16_t)u;
+        s.G[o][n] = x;
+        s.gh[o][n] = (float)x;
+        s.gl[o][n] = (float)(x - (double)(float)x);
+        ++n;
+      }
     }
-    s.mask[tid] = msk;
+    s.nt[o] = n;
   }
-  if (tid == 0) {
-    int nin = 0, nblk = 0;
+  if (tid < 32) {
+    // candidate charges [lowest - 2, highest + 2] of the three bonds, 32 at a time:
+    // records in ascending charge, offsets by sums over the lanes
+    const int cand = s.qtop - qb + 2;
+    int nin = 0, nblk = 0, svoff = 0;
     int64_t woff = 0, voff = 0;
-    int svoff = 0;
-    // candidate charges: [lowest - 2, highest + 2] of the three bonds
-    for (int i = 1; i <= s.qtop - qb + 2; ++i) {
-      const int Q = qb + i;
-      // theta block of middle charge Q: rows (l s1) and columns (s2 r) exist
-      int rows = 0, cols = 0;
-      for (int t = 0; t < 3; ++t) {
-        rows += seg_of(M, 0, qb, Q - s.sk * mval(t)).len;
-        cols += seg_of(M, 2, qb, Q + s.sk1 * mval(t)).len;
+    double k1 = 0.0;
+    bool shared = true;
+    for (int pass = 0; pass < 2; ++pass) {
+      // pass 0 counts, so that the records of one split are all in one place
+      nin = nblk = svoff = 0;
+      woff = voff = 0;
+      for (int i0 = 1; i0 <= cand; i0 += 32) {
+        const int i = i0 + tid, Q = qb + i;
+        InRec in;
+        BlockRec r;
+        int rows = 0, cols = 0, mq = 0, nq = 0;
+        for (int t = 0; t < 3; ++t) {
+          const Seg a = seg_of(T, 0, qb, Q - s.sk * mval(t)), b = seg_of(T, 2, qb, Q + s.sk1 * mval(t));
+          in.rst[t] = (int16_t)a.start, in.roff[t] = (int16_t)rows;
+          in.cst[t] = (int16_t)b.start, in.coff[t] = (int16_t)cols;
+          rows += a.len;
+          cols += b.len;
+          const Seg x = seg_of(T, 0, qb, Q - s.osk * mval(t)), y = seg_of(T, 2, qb, Q + s.osk1 * mval(t));
+          r.rst[t] = (int16_t)x.start, r.rlen[t] = (int16_t)x.len, r.roff[t] = (int16_t)mq;
+          r.cst[t] = (int16_t)y.start, r.clen[t] = (int16_t)y.len, r.coff[t] = (int16_t)nq;
+          mq += x.len;
+          nq += y.len;
+        }
+        const bool is_in = i <= cand && rows > 0 && cols > 0, is_out = i <= cand && mq > 0 && nq > 0;
+        const Seg mid = seg_of(T, 1, qb, Q);
+        in.roff[3] = (int16_t)rows, in.coff[3] = (int16_t)cols;
+        in.mst = (int16_t)mid.start, in.mlen = (int16_t)mid.len;
+        int n_in, n_out, n_sv;
+        const int at_in = lane_prefix(is_in ? 1 : 0, &n_in), at_out = lane_prefix(is_out ? 1 : 0, &n_out);
+        if (pass == 1) {
+          InRec* ri = shared ? s.in_sh : M->in;
+          BlockRec* ro = shared ? s.b_sh : M->b;
+          const int p = mq < nq ? mq : nq, q = mq < nq ? nq : mq;
+          const int at_sv = lane_prefix(is_out ? p : 0, &n_sv);
+          // W and V offsets, in elements: sums of up to 32 x 12288^2 in two halves
+          int lo_t, hi_t, vlo_t, vhi_t;
+          const int64_t w = is_out ? (int64_t)q * p : 0, v = is_out ? (int64_t)p * p : 0;
+          const int wl = lane_prefix((int)(w & 0xfffff), &lo_t), wh = lane_prefix((int)(w >> 20), &hi_t);
+          const int vl = lane_prefix((int)(v & 0xfffff), &vlo_t), vh = lane_prefix((int)(v >> 20), &vhi_t);
+          if (is_in) ri[nin + at_in] = in;
+          if (is_out) {
+            r.Q = (int16_t)Q;
+            r.mq = (int16_t)mq;
+            r.nq = (int16_t)nq;
+            r.trans = nq > mq;
+            r.q = (int16_t)q;
+            r.p = (int16_t)p;
+            r.svoff = svoff + at_sv;
+            r.woff = woff + wl + ((int64_t)wh << 20);
+            r.voff = voff + vl + ((int64_t)vh << 20);
+            ro[nblk + at_out] = r;
+          }
+          svoff += n_sv;
+          woff += lo_t + ((int64_t)hi_t << 20);
+          voff += vlo_t + ((int64_t)vhi_t << 20);
+        }
+        nin += n_in;
+        nblk += n_out;
       }
-      if (rows > 0 && cols > 0) M->qin[nin++] = Q;
-      // output block of new middle charge Q
-      BlockRec r;
-      int mq = 0, nq = 0;
-      for (int t = 0; t < 3; ++t) {
-        const Seg a = seg_of(M, 0, qb, Q - s.osk * mval(t));
-        const Seg b = seg_of(M, 2, qb, Q + s.osk1 * mval(t));
-        r.rst[t] = a.start, r.rlen[t] = a.len, r.roff[t] = mq;
-        r.cst[t] = b.start, r.clen[t] = b.len, r.coff[t] = nq;
-        mq += a.len;
-        nq += b.len;
-      }
-      if (mq == 0 || nq == 0) continue;
-      r.Q = Q;
-      r.mq = mq;
-      r.nq = nq;
-      r.trans = nq > mq;
-      r.q = r.trans ? nq : mq;
-      r.p = r.trans ? mq : nq;
-      r.svoff = svoff;
-      r.pad = 0;
-      r.woff = woff;
-      r.voff = voff;
-      woff += (int64_t)r.q * r.p;
-      voff += (int64_t)r.p * r.p;
-      svoff += r.p;
-      M->b[nblk++] = r;
+      shared = nin <= kShBlk && nblk <= kShBlk;
     }
-    s.nin = nin;
-    s.nblk = nblk;
+    __syncwarp();
+    if (tid == 0) {
+      s.nin = nin;
+      s.nblk = nblk;
+      s.P = svoff;
+      s.in = shared ? s.in_sh : M->in;
+      s.b = shared ? s.b_sh : M->b;
+      for (int i = 0; i < nin; ++i) k1 += (double)s.in[i].roff[3] * s.in[i].mlen * s.in[i].coff[3];
+      s.k1 = k1;
+    }
   }
   __syncthreads();
   return true;
+}
+
+// Calls f(e) for this lane's share of the n elements of one block: the
+// CTA's warps take chunks of 32 elements in turn over all blocks of a phase
+// (c0 counts the chunks so far), so that a phase over many small blocks keeps
+// every warp busy without a barrier or an idle warp between blocks.
+template <int NT, typename F>
+__device__ __forceinline__ void share(int n, int& c0, F&& f) {
+  constexpr int NW = NT / 32;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nch = (n + 31) >> 5;
+  for (int ch = (unsigned)(warp - c0) % NW; ch < nch; ch += NW) {
+    const int e = ch * 32 + lane;
+    if (e < n) f(e);
+  }
+  c0 += nch;
 }
 
 // Phase B: theta[(l s1), (s2 r)] = sum_m A_k[(l s1), m] A_{k+1}[m, (s2 r)] for
@@ -240,14 +383,71 @@ __device__ bool prepare(ChainDev* c, const OpDev& op, SplitSh& s) {
 // middle charge over that charge's run of the middle bond.  Entries of a
 // charge absent from the middle bond are written as 0.  A, B are binary64
 // site tensors; T is the accumulation and storage type of theta.
+//
+// Two forms.  Direct: a warp takes 4 rows x 32 columns of a block and reads
+// both operands through L1, all blocks at once, no barrier.  Binary64 always
+// takes it: its pipe (16 clocks a warp instruction) hides the two loads a
+// product costs, and a padded tile would be charged in full.  Binary32 takes it
+// while the split has at most kThetaDirect products; above, the CTA goes
+// through the blocks in TM x TN x TK tiles in shared memory, which convert and
+// load each operand once per tile instead of once per product.
+constexpr double kThetaDirect = 131072.0;
+
+template <int NT, typename T>
+__device__ void theta_direct(const ChainDev* c, int k, const SplitSh& s, T* __restrict__ theta) {
+  constexpr int R = 4;
+  const int chim = c->chi[k + 1], chir = c->chi[k + 2];
+  const int n = 3 * chir;
+  const double* __restrict__ A = c->site[k];
+  const double* __restrict__ B = c->site[k + 1];
+  int c0 = 0;
+  for (int bi = 0; bi < s.nin; ++bi) {
+    const InRec& r = s.in[bi];
+    const int Mv = r.roff[3], Nv = r.coff[3], K = r.mlen, mst = r.mst;
+    const int nu = (Nv + 31) >> 5;
+    // one element a lane: (row group, column), columns padded to whole warps
+    share<NT>(((Mv + R - 1) / R) * nu * 32, c0, [&](int e) {
+      const int g = e / (nu * 32), u = e - g * nu * 32;
+      const int uu = u < Nv ? u : Nv - 1;
+      const int t2 = uu >= r.coff[2] ? 2 : (uu >= r.coff[1] ? 1 : 0);
+      const int col = t2 * chir + r.cst[t2] + uu - r.coff[t2];
+      const double* b = B + (size_t)mst * n + col;
+      const double* a[R];
+      int row[R];
+      T acc[R];
+#pragma unroll
+      for (int x = 0; x < R; ++x) {
+        const int v = min(g * R + x, Mv - 1);
+        const int t = v >= r.roff[2] ? 2 : (v >= r.roff[1] ? 1 : 0);
+        row[x] = 3 * (r.rst[t] + v - r.roff[t]) + t;
+        a[x] = A + (size_t)row[x] * chim + mst;
+        acc[x] = T(0);
+      }
+      const int nr = min(R, Mv - g * R);
+#pragma unroll 4
+      for (int kk = 0; kk < K; ++kk) {
+        const T bv = from64<T>(b[(size_t)kk * n]);
+#pragma unroll
+        for (int x = 0; x < R; ++x)
+          if (x < nr) acc[x] = fma(from64<T>(a[x][kk]), bv, acc[x]);
+      }
+      if (u < Nv)
+#pragma unroll
+        for (int x = 0; x < R; ++x)
+          if (x < nr) theta[(size_t)row[x] * n + col] = acc[x];
+    });
+  }
+  __syncthreads();
+}
+
 template <int NT, int TM, int TN, int TK, typename T>
 __device__ void theta_blocks(const ChainDev* c, int k, const SplitSh& s, T* __restrict__ theta, T* smem) {
+  if (sizeof(T) == sizeof(double) || s.k1 <= kThetaDirect) return theta_direct<NT, T>(c, k, s, theta);
   const int tid = threadIdx.x;
   const int chim = c->chi[k + 1], chir = c->chi[k + 2];
   const int n = 3 * chir;
   const double* __restrict__ A = c->site[k];
   const double* __restrict__ B = c->site[k + 1];
-  const Meta* M = reinterpret_cast<const Meta*>(c->meta);
   // thread tile: rows ty + TY a (a < RA), columns tx + TX b (b < 4)
   constexpr int RB = 4, TX = TN / RB, TY = NT / TX, RA = TM / TY;
   static_assert(TN % RB == 0 && NT % TX == 0 && TM % TY == 0, "tile must split evenly over the CTA");
@@ -255,19 +455,8 @@ __device__ void theta_blocks(const ChainDev* c, int k, const SplitSh& s, T* __re
   T* sa = smem;                            // [TK][TM + 1]
   T* sb = smem + TK * (TM + 1);            // [TK][TN + 1]
   for (int bi = 0; bi < s.nin; ++bi) {
-    const int Q = M->qin[bi];
-    int rst[3], roff[4], cst[3], coff[4];
-    roff[0] = coff[0] = 0;
-    for (int t = 0; t < 3; ++t) {
-      const Seg a = seg_of(M, 0, s.qbase, Q - s.sk * mval(t));
-      const Seg b = seg_of(M, 2, s.qbase, Q + s.sk1 * mval(t));
-      rst[t] = a.start;
-      roff[t + 1] = roff[t] + a.len;
-      cst[t] = b.start;
-      coff[t + 1] = coff[t] + b.len;
-    }
-    const Seg mid = seg_of(M, 1, s.qbase, Q);
-    const int Mv = roff[3], Nv = coff[3], K = mid.len;
+    const InRec& r = s.in[bi];
+    const int Mv = r.roff[3], Nv = r.coff[3], K = r.mlen, mst = r.mst;
     for (int i0 = 0; i0 < Mv; i0 += TM) {
       for (int j0 = 0; j0 < Nv; j0 += TN) {
         T acc[RA][RB];
@@ -281,9 +470,9 @@ __device__ void theta_blocks(const ChainDev* c, int k, const SplitSh& s, T* __re
             const int v = i0 + ii, g = k0 + kk;
             T x = T(0);
             if (v < Mv && g < K) {
-              const int t = v >= roff[2] ? 2 : (v >= roff[1] ? 1 : 0);
-              const int l = rst[t] + v - roff[t];
-              x = (T)A[(size_t)(3 * l + t) * chim + mid.start + g];
+              const int t = v >= r.roff[2] ? 2 : (v >= r.roff[1] ? 1 : 0);
+              const int l = r.rst[t] + v - r.roff[t];
+              x = from64<T>(A[(size_t)(3 * l + t) * chim + mst + g]);
             }
             sa[kk * (TM + 1) + ii] = x;
           }
@@ -292,15 +481,15 @@ __device__ void theta_blocks(const ChainDev* c, int k, const SplitSh& s, T* __re
             const int u = j0 + jj, g = k0 + kk;
             T x = T(0);
             if (u < Nv && g < K) {
-              const int t = u >= coff[2] ? 2 : (u >= coff[1] ? 1 : 0);
-              const int r = cst[t] + u - coff[t];
-              x = (T)B[(size_t)(mid.start + g) * n + t * chir + r];
+              const int t = u >= r.coff[2] ? 2 : (u >= r.coff[1] ? 1 : 0);
+              x = from64<T>(B[(size_t)(mst + g) * n + t * chir + r.cst[t] + u - r.coff[t]]);
             }
             sb[kk * (TN + 1) + jj] = x;
           }
           __syncthreads();
+          const int kn = min(TK, K - k0);
 #pragma unroll 4
-          for (int kk = 0; kk < TK; ++kk) {
+          for (int kk = 0; kk < kn; ++kk) {
             T bv[RB];
 #pragma unroll
             for (int b = 0; b < RB; ++b) bv[b] = sb[kk * (TN + 1) + tx + TX * b];
@@ -317,14 +506,14 @@ __device__ void theta_blocks(const ChainDev* c, int k, const SplitSh& s, T* __re
         for (int a = 0; a < RA; ++a) {
           const int v = i0 + ty + TY * a;
           if (v >= Mv) continue;
-          const int t = v >= roff[2] ? 2 : (v >= roff[1] ? 1 : 0);
-          const int row = 3 * (rst[t] + v - roff[t]) + t;
+          const int t = v >= r.roff[2] ? 2 : (v >= r.roff[1] ? 1 : 0);
+          const int row = 3 * (r.rst[t] + v - r.roff[t]) + t;
 #pragma unroll
           for (int b = 0; b < RB; ++b) {
             const int u = j0 + tx + TX * b;
             if (u >= Nv) continue;
-            const int tt = u >= coff[2] ? 2 : (u >= coff[1] ? 1 : 0);
-            theta[(size_t)row * n + tt * chir + cst[tt] + u - coff[tt]] = acc[a][b];
+            const int tt = u >= r.coff[2] ? 2 : (u >= r.coff[1] ? 1 : 0);
+            theta[(size_t)row * n + tt * chir + r.cst[tt] + u - r.coff[tt]] = acc[a][b];
           }
         }
       }
@@ -333,45 +522,49 @@ __device__ void theta_blocks(const ChainDev* c, int k, const SplitSh& s, T* __re
   __syncthreads();
 }
 
-// Phase C input: block b of theta after the gate (Sec. I.A: the gate acts on
+// Phase C input: block r of theta after the gate (Sec. I.A: the gate acts on
 // the physical legs only), written column-major into W (q x p, leading
 // dimension ldw; the transpose when the block is wider than tall).  V = I.
+// c0: see share().  A binary32 theta takes each coefficient as a binary32 pair
+// (hi + lo): rounding the gate itself would repeat the same relative error at
+// every application of that gate and add up coherently over the evolution,
+// while the rounding of the products does not.  The pairs are split once per
+// split (prepare): split at every use they put four binary64 instructions
+// on each of the up to three terms of an entry.
 template <int NT, typename TT, typename TW>
 __device__ void gather_block(const ChainDev* c, int k, const SplitSh& s, const BlockRec& r,
-                             const TT* __restrict__ theta, TW* __restrict__ W, int ldw, TW* __restrict__ V, int ldv) {
+                             const TT* __restrict__ theta, TW* __restrict__ W, int ldw, TW* __restrict__ V, int ldv,
+                             int& c0) {
   const int chir = c->chi[k + 2];
   const int n = 3 * chir;
-  const int total = r.mq * r.nq;
-  for (int e = threadIdx.x; e < total; e += NT) {
-    const int v = e / r.nq, u = e % r.nq;              // u fastest: r runs contiguously in theta
+  const int nq = r.nq;
+  share<NT>(r.mq * nq, c0, [&](int e) {
+    const int v = e / nq, u = e - v * nq;              // u fastest: r runs contiguously in theta
     const int a = v >= r.roff[2] ? 2 : (v >= r.roff[1] ? 1 : 0);
     const int b = u >= r.coff[2] ? 2 : (u >= r.coff[1] ? 1 : 0);
-    const int l = r.rst[a] + v - r.roff[a];
-    const int rr = r.cst[b] + u - r.coff[b];
-    const int msk = s.mask[3 * a + b];
+    const int o = 3 * a + b;
+    const TT* th = theta + (size_t)(3 * (r.rst[a] + v - r.roff[a])) * n + r.cst[b] + u - r.coff[b];
+    const int nt = s.nt[o];
     TT x = TT(0), y = TT(0);
-#pragma unroll
-    for (int t = 0; t < 9; ++t) {
-      if (msk & (1 << t)) {
-        const int s1 = t / 3, s2 = t % 3;
-        const TT th = theta[(size_t)(3 * l + s1) * n + s2 * chir + rr];
-        const double g = s.G[(3 * a + b) * 9 + t];
-        const TT ghi = (TT)g;
-        x = fma(ghi, th, x);
-        // a binary32 theta takes each coefficient as a binary32 pair
-        // (hi + lo): rounding the gate itself would repeat the same relative
-        // error at every application of that gate and add up coherently over
-        // the evolution, while the rounding of the products does not
-        if (sizeof(TT) < sizeof(double)) y = fma((TT)(g - (double)ghi), th, y);
+    for (int t = 0; t < nt; ++t) {
+      const int in = s.tt[o][t];
+      const TT h = th[(size_t)(in / 3) * n + (in % 3) * chir];
+      if constexpr (sizeof(TT) < sizeof(double)) {
+        x = fma(s.gh[o][t], h, x);
+        y = fma(s.gl[o][t], h, y);
+      } else {
+        x = fma(s.G[o][t], h, x);
       }
     }
-    if (r.trans) W[(size_t)v * ldw + u] = (TW)(x + y);
-    else W[(size_t)u * ldw + v] = (TW)(x + y);
-  }
-  for (int e = threadIdx.x; e < r.p * r.p; e += NT) {
-    const int j = e / r.p, i = e % r.p;
+    if constexpr (sizeof(TT) < sizeof(double)) x += y;
+    if (r.trans) W[(size_t)v * ldw + u] = (TW)x;
+    else W[(size_t)u * ldw + v] = (TW)x;
+  });
+  const int p = r.p;
+  share<NT>(p * p, c0, [&](int e) {
+    const int j = e / p, i = e - j * p;
     V[(size_t)j * ldv + i] = (i == j) ? TW(1) : TW(0);
-  }
+  });
 }
 
 // Barrier of the nthreads threads (a multiple of 32) of a warp group; ids
@@ -874,86 +1067,158 @@ __device__ __forceinline__ double svd_count(double m, double n) {
   return 4.0 * M * M * N + 8.0 * M * N * N + 9.0 * N * N * N;
 }
 
+// Order-preserving integer key of a value >= 0 (compares on the integer
+// pipe; a binary64 compare is a binary64 instruction).
+__device__ __forceinline__ unsigned long long sort_key(double x) {
+  unsigned long long b;
+  memcpy(&b, &x, 8);
+  return b;
+}
+
+// Bytes of finish()'s scratch for P values.
+__device__ __forceinline__ size_t finish_bytes(int P) { return (size_t)P * (4 * sizeof(double) + 4 * sizeof(int32_t)); }
+
+// The truncation rule of trunc_rank on n sorted values by one warp: every
+// lane owns a run of values and sums it from its smallest value up, the
+// runs are joined by a suffix sum over the lanes.  Returns the kept count;
+// *kept and *tail get the kept and the discarded weight.
+__device__ inline int warp_trunc_rank(const double* s, int n, int chi_max, double cutoff, double* kept, double* tail) {
+  const int lane = threadIdx.x & 31;
+  const int per = (n + 31) / 32;
+  const int i0 = min(lane * per, n), i1 = min(i0 + per, n);
+  double own = 0.0;
+  for (int i = i1 - 1; i >= i0; --i) own = fma(s[i], s[i], own);
+  double suf = own;                        // sum over this lane and the later ones
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const double y = lane_value(suf, lane + o < 32 ? lane + o : lane);
+    if (lane + o < 32) suf += y;
+  }
+  const double total = lane_value(suf, 0);
+  double run = lane_value(suf, lane < 31 ? lane + 1 : 31);
+  if (lane == 31) run = 0.0;
+  // smallest kk >= 1 with sum_{q >= kk} s_q^2 <= cutoff total
+  int k = n;
+  const double bar = cutoff * total;
+  for (int i = i1 - 1; i >= i0; --i) {
+    // run = tail of kept count i + 1
+    if (run <= bar) k = min(k, i + 1);
+    run = fma(s[i], s[i], run);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) k = min(k, __shfl_xor_sync(0xffffffffu, k, o));
+  if (k > chi_max) k = chi_max;
+  while (k > 1 && k < n && s[k] >= s[k - 1] * (1.0 - 1e-8)) --k;
+  double a = 0.0, b = 0.0;
+  for (int i = lane; i < n; i += 32) {
+    if (i < k) a = fma(s[i], s[i], a);
+    else b = fma(s[i], s[i], b);
+  }
+  *kept = warp_sum64(a);
+  *tail = warp_sum64(b);
+  return k;
+}
+
 // Phase D: singular values of every block (column norms of its converged W,
 // binary64), one descending order over all blocks, the truncation rule,
 // renormalisation, then the new bond grouped by charge (ascending; by value
 // within a charge), the absorb into A_k and A_{k+1} (zeros outside the
 // blocks) and the new middle charges.  W and V hold every block's binary64
-// result; `scratch` (the theta buffer) holds 4 per-value arrays.
+// result.  scratch: finish_bytes(P) bytes; tiles: per warp 8 x 33 doubles of
+// shared memory (the transposition of the left factor).
+//
+// The binary64 pipe and dependent loads bound this phase, not its traffic: the
+// order compares integer keys, the truncation sums run over a warp, a kept
+// value's scales cost one divide each (not one per element), and the absorb
+// goes block by block, after a plain zero fill, instead of looking up each
+// element's block.
 template <int NT>
-__device__ void finish(ChainDev* c, const OpDev& op, int t, SplitSh& s, double* __restrict__ scratch,
+__device__ void finish(ChainDev* c, const OpDev& op, int t, SplitSh& s, char* __restrict__ scratch, double* tiles,
                        int32_t* ctx_err, int sweeps32, int sweeps64) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int nwarps = NT / 32;
+  constexpr int NW = NT / 32;
   const int k = op.k;
   const int chil = c->chi[k], chim = c->chi[k + 1], chir = c->chi[k + 2];
   const int m = 3 * chil, n = 3 * chir;
-  const Meta* M = reinterpret_cast<const Meta*>(c->meta);
-  const int nb = s.nblk;
-  const BlockRec& last = M->b[nb - 1];
-  const int P = last.svoff + last.p;                  // values over all blocks
-  double* sraw = scratch;                             // P: value of slot
-  int32_t* sblk = reinterpret_cast<int32_t*>(scratch + P);   // P: block of slot
-  double* tail = scratch + 2 * P;                     // P + 1
-  int32_t* newslot = reinterpret_cast<int32_t*>(scratch + 3 * P + 1);   // kk: slot of new index
+  const int nb = s.nblk, P = s.P;
+  double* sraw = reinterpret_cast<double*>(scratch);  // P: value of slot
+  double* sig = sraw + P;                             // P: sorted values
+  double* lsc = sig + P;                              // scales of the kept values in the left factor
+  double* rsc = lsc + P;                              // and in the right one
+  int32_t* sblk = reinterpret_cast<int32_t*>(rsc + P);   // block of slot
+  int32_t* perm = sblk + P;                           // slot of sorted value
+  int32_t* key = perm + P;                            // kept value: block, rank
+  int32_t* newslot = key + P;                         // slot of new index
   // column norms -> raw values, slot = svoff + column
-  for (int b = 0; b < nb; ++b) {
-    const BlockRec& r = M->b[b];
-    const double* Wb = c->W + r.woff;
-    for (int j = warp; j < r.p; j += nwarps) {
-      const double* cj = Wb + (size_t)j * r.q;
-      double s2 = 0.0;
-      for (int i = lane; i < r.q; i += 32) s2 = fma(cj[i], cj[i], s2);
-      s2 = warp_sum64(s2);
-      if (lane == 0) {
-        sraw[r.svoff + j] = sqrt(s2);
-        sblk[r.svoff + j] = b;
+  {
+    int c0 = 0;
+    for (int b = 0; b < nb; ++b) {
+      const BlockRec& r = s.b[b];
+      const double* Wb = c->W + r.woff;
+      for (int j = (unsigned)(warp - c0) % NW; j < r.p; j += NW) {
+        const double* cj = Wb + (size_t)j * r.q;
+        double s2 = 0.0;
+#pragma unroll 4
+        for (int i = lane; i < r.q; i += 32) s2 = fma(cj[i], cj[i], s2);
+        s2 = warp_sum64(s2);
+        if (lane == 0) {
+          sraw[r.svoff + j] = sqrt(s2);
+          sblk[r.svoff + j] = b;
+        }
       }
+      c0 += r.p;
     }
   }
   __syncthreads();
   // descending rank (ties by slot): sig[rank] = value, perm[rank] = slot
   for (int j = tid; j < P; j += NT) {
     const double sj = sraw[j];
+    const unsigned long long kj = sort_key(sj);
     int rank = 0;
-    for (int i = 0; i < P; ++i) {
-      const double si = sraw[i];
-      rank += (si > sj) || (si == sj && i < j);
-    }
-    c->sig[rank] = sj;
-    c->perm[rank] = j;
+#pragma unroll 8
+    for (int i = 0; i < j; ++i) rank += sort_key(sraw[i]) >= kj;
+#pragma unroll 8
+    for (int i = j + 1; i < P; ++i) rank += sort_key(sraw[i]) > kj;
+    sig[rank] = sj;
+    perm[rank] = j;
   }
   __syncthreads();
-  if (tid == 0) {
-    const double* sv = c->sig;
-    double total, nrm = 1.0;
+  if (warp == 0) {
+    double kept = 1.0, tail = 0.0, nrm = 1.0;
     int kk;
     if (!op.exact) {
-      kk = trunc_rank(sv, P, c->chi_max, c->cutoff, tail, &total);
+      kk = warp_trunc_rank(sig, P, c->chi_max, c->cutoff, &kept, &tail);
+      const double total = kept + tail;
       if (!(total > 0.0) || !isfinite(total)) kk = -1;
       else {
-        double kept = 0.0;
-        for (int i = 0; i < kk; ++i) kept += sv[i] * sv[i];
         nrm = 1.0 / sqrt(kept);
-        c->stats[ST_DISC] += tail[kk] / total;
+        tail /= total;
       }
     } else {
-      kk = 0;
-      while (kk < P && kk < chim && sv[kk] > 0.0) ++kk;
+      int pos = 0;                           // nonzero values
+      for (int i = lane; i < P; i += 32) pos += sort_key(sig[i]) != 0ull;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) pos += __shfl_xor_sync(0xffffffffu, pos, o);
+      kk = min(pos, chim);
       if (kk == 0) kk = -1;
     }
-    s.kk = kk;
-    s.nrm = nrm;
-    if (kk > 0) {
-      double svd = 0.0;
-      for (int b = 0; b < nb; ++b) svd += svd_count(M->b[b].mq, M->b[b].nq);
-      c->stats[ST_SVD] += svd;
-      c->stats[ST_SVD_DENSE] += svd_count(m, n);
-      c->stats[ST_SWEEPS] += sweeps32;
-      c->stats[ST_SWEEPS64] += sweeps64;
-      c->stats[ST_SPLITS] += 1.0;
-      c->stats[ST_BLOCKS] += nb;
-      if (kk > c->stats[ST_MAXCHI]) c->stats[ST_MAXCHI] = kk;
+    if (lane == 0) {
+      s.kk = kk;
+      s.nrm = nrm;
+      if (kk > 0) {
+        double svd = 0.0;
+        for (int b = 0; b < nb; ++b) svd += svd_count(s.b[b].mq, s.b[b].nq);
+        c->stats[ST_K1] += 2.0 * s.k1;
+        c->stats[ST_K2] += 2.0 * 81.0 * chil * chir;
+        c->stats[ST_SVD] += svd;
+        c->stats[ST_SVD_DENSE] += svd_count(m, n);
+        c->stats[ST_DISC] += tail;
+        c->stats[ST_SWEEPS] += sweeps32;
+        c->stats[ST_SWEEPS64] += sweeps64;
+        c->stats[ST_SPLITS] += 1.0;
+        c->stats[ST_BLOCKS] += nb;
+        if (kk > c->stats[ST_MAXCHI]) c->stats[ST_MAXCHI] = kk;
+      }
     }
   }
   __syncthreads();
@@ -966,68 +1231,86 @@ __device__ void finish(ChainDev* c, const OpDev& op, int t, SplitSh& s, double* 
     }
     return;
   }
+  double* __restrict__ Ak = c->site[k];
+  double* __restrict__ Ak1 = c->site[k + 1];
   // new position of kept rank i: kept values of lower-charge blocks first,
   // then by rank within the block
-  for (int i = tid; i < kk; i += NT) {
-    const int slot = c->perm[i];
-    const int b = sblk[slot];
-    int pos = 0;
-    for (int j = 0; j < kk; ++j) {
-      const int bj = sblk[c->perm[j]];
-      pos += (bj < b) || (bj == b && j < i);
-    }
-    newslot[pos] = slot;
+  for (int i = tid; i < kk; i += NT) key[i] = sblk[perm[i]] * 16384 + i;
+  // zeros everywhere (site slots are 256-byte aligned)
+  for (int h = 0; h < 2; ++h) {
+    double* A = h ? Ak1 : Ak;
+    const int tot = h ? kk * n : m * kk;
+    double2* A2 = reinterpret_cast<double2*>(A);
+    const double2 z = {0.0, 0.0};
+    for (int e = tid; e < tot / 2; e += NT) A2[e] = z;
+    if ((tot & 1) && tid == 0) A[tot - 1] = 0.0;
   }
   __syncthreads();
   const bool absorb_left = op.absorb == 0;
-  double* Ak = c->site[k];
-  double* Ak1 = c->site[k + 1];
-  // A_k[(l a), i]
-  for (int e = tid; e < m * kk; e += NT) {
-    const int row = e / kk, i = e % kk;
-    const int slot = newslot[i];
-    const BlockRec& r = M->b[sblk[slot]];
-    const int j = slot - r.svoff;
-    const int l = row / 3, a = row % 3;
-    double v = 0.0;
-    const int lo = l - r.rst[a];
-    if (lo >= 0 && lo < r.rlen[a]) {
-      const int rl = r.roff[a] + lo;
-      const double sg = sraw[slot];
-      if (!r.trans) {
-        const double w = c->W[r.woff + (size_t)j * r.q + rl];   // = U sigma
-        v = absorb_left ? w * nrm : w / sg;
-      } else {
-        const double u = c->V[r.voff + (size_t)j * r.p + rl];   // left vector
-        v = absorb_left ? u * sg * nrm : u;
-      }
-    }
-    Ak[e] = v;
-  }
-  // A_{k+1}[i, (b r)]
-  for (int e = tid; e < kk * n; e += NT) {
-    const int i = e / n, col = e % n;
-    const int slot = newslot[i];
-    const BlockRec& r = M->b[sblk[slot]];
-    const int j = slot - r.svoff;
-    const int b = col / chir, rr = col % chir;
-    double v = 0.0;
-    const int lo = rr - r.cst[b];
-    if (lo >= 0 && lo < r.clen[b]) {
-      const int cl = r.coff[b] + lo;
-      const double sg = sraw[slot];
-      if (!r.trans) {
-        const double u = c->V[r.voff + (size_t)j * r.p + cl];   // right vector
-        v = absorb_left ? u : u * sg * nrm;
-      } else {
-        const double w = c->W[r.woff + (size_t)j * r.q + cl];   // = V sigma
-        v = absorb_left ? w / sg : w * nrm;
-      }
-    }
-    Ak1[e] = v;
-  }
   int16_t* qM = c->qn + (size_t)(k + 1) * c->chi_cap;
-  for (int i = tid; i < kk; i += NT) qM[i] = (int16_t)M->b[sblk[newslot[i]]].Q;
+  for (int i = tid; i < kk; i += NT) {
+    const int ki = key[i];
+    int pos = 0;
+#pragma unroll 8
+    for (int j = 0; j < kk; ++j) pos += key[j] < ki;
+    const int slot = perm[i], b = sblk[slot];
+    newslot[pos] = slot;
+    qM[pos] = s.b[b].Q;
+    const double sg = sraw[slot];
+    // W column = U sigma (left) or V sigma (right, transposed block); V column a unit vector
+    const bool w_left = !s.b[b].trans;
+    const double unit = absorb_left ? (w_left ? 1.0 : sg * nrm) : (w_left ? sg * nrm : 1.0);   // V's side
+    const double wsc = absorb_left == w_left ? nrm : 1.0 / sg;
+    lsc[pos] = w_left ? wsc : unit;
+    rsc[pos] = w_left ? unit : wsc;
+  }
+  __syncthreads();
+  double* tile = tiles + warp * (8 * 33);
+  int c0 = 0, pos0 = 0;
+  for (int b = 0; b < nb; ++b) {
+    const BlockRec& r = s.b[b];
+    // kept values of this block: new indices [pos0, pos0 + kb)
+    int kb = 0;
+    while (pos0 + kb < kk && sblk[newslot[pos0 + kb]] == b) ++kb;
+    if (kb == 0) continue;
+    const double* L = r.trans ? c->V + r.voff : c->W + r.woff;
+    const double* Rf = r.trans ? c->W + r.woff : c->V + r.voff;
+    const int ldl = r.trans ? r.p : r.q, ldr = r.trans ? r.q : r.p;
+    const int mq = r.mq, nq = r.nq, sv = r.svoff;
+    // left factor A_k[(l a), i]: 32 rows x 8 kept values a warp, transposed in shared memory
+    const int tv = (mq + 31) >> 5, ti = (kb + 7) >> 3;
+    for (int x = (unsigned)(warp - c0) % NW; x < tv * ti; x += NW) {
+      const int v0 = (x % tv) * 32, j0 = (x / tv) * 8;
+      const int nv = min(32, mq - v0), nj = min(8, kb - j0);
+      __syncwarp();
+      if (lane < nv)
+#pragma unroll
+        for (int y = 0; y < 8; ++y)
+          if (y < nj) {
+            const int i = pos0 + j0 + y;
+            tile[y * 33 + lane] = L[(size_t)(newslot[i] - sv) * ldl + v0 + lane] * lsc[i];
+          }
+      __syncwarp();
+#pragma unroll
+      for (int y = 0; y < 8; ++y) {
+        const int vv = y * 4 + (lane >> 3), jj = lane & 7;
+        if (vv < nv && jj < nj) {
+          const int v = v0 + vv;
+          const int a = v >= r.roff[2] ? 2 : (v >= r.roff[1] ? 1 : 0);
+          Ak[(size_t)(3 * (r.rst[a] + v - r.roff[a]) + a) * kk + pos0 + j0 + jj] = tile[jj * 33 + vv];
+        }
+      }
+    }
+    c0 += tv * ti;
+    // right factor A_{k+1}[i, (b r)]
+    share<NT>(kb * nq, c0, [&](int e) {
+      const int i = pos0 + e / nq, u = e % nq;
+      const int bb = u >= r.coff[2] ? 2 : (u >= r.coff[1] ? 1 : 0);
+      Ak1[(size_t)i * n + bb * chir + r.cst[bb] + u - r.coff[bb]] =
+          Rf[(size_t)(newslot[i] - sv) * ldr + u] * rsc[i];
+    });
+    pos0 += kb;
+  }
   __syncthreads();
   if (tid == 0) {
     c->chi[k + 1] = kk;

@@ -46,6 +46,18 @@ struct TransferSh {
   int32_t ival;
 };
 
+// Shared memory of the evolve kernel: the charge-run tables of a split while
+// it is prepared, then the transposition tiles and the value lists of finish()
+// (more than 400 values use the theta buffer).
+constexpr int kTileDoubles = NT / 32 * 8 * 33;
+constexpr int kBufDoubles = kTileDoubles + 2496;
+struct EvolveSh {
+  double buf[kBufDoubles];
+  blk::SplitSh split;
+  blk::GroupSh gs;
+};
+static_assert(sizeof(blk::PrepTab) <= kBufDoubles * sizeof(double), "prepare's tables");
+
 struct Shared {
   GemmSmem g;
   double red[NT / 32][4];
@@ -390,19 +402,23 @@ __device__ void two_site_op(ChainDev* c, const OpDev op, int t, Shared& sh, int3
 // clock per SM on GB300) is the bound, and every warp of the CTA is needed
 // to hide the latency of the global-memory rotations (splitting the warps
 // over the blocks of a split measured 1.7x slower).
-__device__ void two_site_op_blocked(ChainDev* c, const OpDev op, int t, Shared& sh, blk::SplitSh& ss,
-                                    blk::GroupSh& gs, int32_t* ctx_err) {
-  if (!blk::prepare<NT>(c, op, ss)) blk::prepare<NT>(c, op, ss);
-  blk::theta_blocks<NT, TM, TN, TK, double>(c, op.k, ss, c->theta, &sh.g.a[0][0]);
-  const blk::Meta* M = reinterpret_cast<const blk::Meta*>(c->meta);
+__device__ void two_site_op_blocked(ChainDev* c, const OpDev op, int t, EvolveSh& sh, int32_t* ctx_err) {
+  blk::SplitSh& ss = sh.split;
+  blk::PrepTab& tab = *reinterpret_cast<blk::PrepTab*>(sh.buf);
+  if (!blk::prepare<NT>(c, op, ss, tab)) blk::prepare<NT>(c, op, ss, tab);
+  blk::theta_blocks<NT, TM, TN, TK, double>(c, op.k, ss, c->theta, sh.buf);
+  int c0 = 0;
+  for (int b = 0; b < ss.nblk; ++b) {
+    const blk::BlockRec& r = ss.b[b];
+    blk::gather_block<NT, double, double>(c, op.k, ss, r, c->theta, c->W + r.woff, r.q, c->V + r.voff, r.p, c0);
+  }
+  __syncthreads();
   int sweeps = 0;
   int64_t cost = -1;
   for (int b = 0; b < ss.nblk; ++b) {
-    const blk::BlockRec& r = M->b[b];
-    blk::gather_block<NT, double, double>(c, op.k, ss, r, c->theta, c->W + r.woff, r.q, c->V + r.voff, r.p);
-    __syncthreads();
+    const blk::BlockRec& r = ss.b[b];
     const int sw = blk::jacobi_group<double, double, 2>(c->W + r.woff, r.q, r.q, r.p, c->V + r.voff, r.p, c->sig,
-                                             threadIdx.x >> 5, NT / 32, 1, 0, gs, 1e-9, kMaxSweeps);
+                                             threadIdx.x >> 5, NT / 32, 1, 0, sh.gs, 1e-9, kMaxSweeps);
     if (sw < 0) {
       set_error(c, HM_ERR_NUMERIC, t, ctx_err);
       return;
@@ -411,28 +427,14 @@ __device__ void two_site_op_blocked(ChainDev* c, const OpDev op, int t, Shared& 
     if (cb > cost) cost = cb, sweeps = sw;
     __syncthreads();
   }
-  blk::finish<NT>(c, op, t, ss, c->theta, ctx_err, sweeps, 0);
-  if (threadIdx.x == 0 && ss.kk > 0) {
-    double k1 = 0.0;
-    for (int i = 0; i < ss.nin; ++i) {
-      const int Q = M->qin[i];
-      double rows = 0.0, cols = 0.0;
-      for (int u = 0; u < 3; ++u) {
-        rows += blk::seg_of(M, 0, ss.qbase, Q - ss.sk * blk::mval(u)).len;
-        cols += blk::seg_of(M, 2, ss.qbase, Q + ss.sk1 * blk::mval(u)).len;
-      }
-      k1 += 2.0 * rows * blk::seg_of(M, 1, ss.qbase, Q).len * cols;
-    }
-    c->stats[ST_K1] += k1;
-    c->stats[ST_K2] += 2.0 * 81.0 * c->chi[op.k] * c->chi[op.k + 2];
-  }
+  char* scratch = reinterpret_cast<char*>(sh.buf + kTileDoubles);
+  if (blk::finish_bytes(ss.P) > (kBufDoubles - kTileDoubles) * sizeof(double)) scratch = reinterpret_cast<char*>(c->theta);
+  blk::finish<NT>(c, op, t, ss, scratch, sh.buf, ctx_err, sweeps, 0);
   __syncthreads();
 }
 
 __global__ void __launch_bounds__(NT) evolve_fp64_kernel(BatchArg b, OutArg o) {
-  __shared__ Shared sh;
-  __shared__ blk::SplitSh ss;
-  __shared__ blk::GroupSh gs;
+  __shared__ EvolveSh sh;
   ChainDev* c = b.c[blockIdx.x];
   const OpDev* ops = b.ops_override ? b.ops_override : c->ops;
   const int n_ops = b.ops_override ? b.n_override : c->n_ops;
@@ -443,7 +445,7 @@ __global__ void __launch_bounds__(NT) evolve_fp64_kernel(BatchArg b, OutArg o) {
   for (int t = t0; t < t1; ++t) {
     if (*(volatile int32_t*)c->status != 0) return;
     __syncthreads();
-    two_site_op_blocked(c, ops[t], t, sh, ss, gs, o.ctx_err);
+    two_site_op_blocked(c, ops[t], t, sh, o.ctx_err);
     __syncthreads();
   }
 }

@@ -389,6 +389,8 @@ __device__ void promote_v(const float* V32, int ldv, int q, int p, double* W64, 
 // memory is at least this (and at least the staged fallback's plan).  Two
 // CTAs per SM share the SM's 228 KB.
 constexpr size_t kBlockSmem = kCtasPerSm == 1 ? 210 * 1024 : kPairBlockSmem;
+constexpr int kTileDoubles = NT / 32 * 8 * 33;   // finish()'s transposition tiles
+static_assert(sizeof(blk::PrepTab) <= kBlockSmem, "prepare's tables");
 
 // Stopping rule of the binary64 polish: a sweep whose largest rotation ratio
 // is below this leaves off-diagonals of order its square for the next sweep.
@@ -417,10 +419,10 @@ constexpr float kStop32 = 2e-4f, kStop32Polished = 1e-3f;
 __device__ void two_site_op_mixed(ChainDev* c, const OpDev op, int t, int bcols, int polish, float* smem, Scal& sc,
                                   blk::SplitSh& ss, blk::WaveSh& wv, blk::GroupSh& gs, int32_t* ctx_err) {
   const int tid = threadIdx.x, warp = tid >> 5;
-  if (!blk::prepare<NT>(c, op, ss)) blk::prepare<NT>(c, op, ss);
+  blk::PrepTab& tab = *reinterpret_cast<blk::PrepTab*>(smem);
+  if (!blk::prepare<NT>(c, op, ss, tab)) blk::prepare<NT>(c, op, ss, tab);
   float* theta = reinterpret_cast<float*>(c->theta);
   blk::theta_blocks<NT, GM, GN, GK, float>(c, op.k, ss, theta, smem);
-  const blk::Meta* M = reinterpret_cast<const blk::Meta*>(c->meta);
   int sw32 = 0, sw64 = 0;
   int64_t cost = -1;
   constexpr int64_t cap = (int64_t)(kBlockSmem / sizeof(float));
@@ -431,7 +433,7 @@ __device__ void two_site_op_mixed(ChainDev* c, const OpDev op, int t, int bcols,
       int64_t used = 0;
       int n = 0, p[15];
       while (b0 + n < ss.nblk && n < 15 && n < NT / 32) {
-        const blk::BlockRec& r = M->b[b0 + n];
+        const blk::BlockRec& r = ss.b[b0 + n];
         const int64_t need = (int64_t)r.p * (r.q | 1) + (int64_t)r.p * (r.p | 1) + r.p;
         if (used + need > cap) break;
         wv.off[n] = (int32_t)used;
@@ -446,10 +448,11 @@ __device__ void two_site_op_mixed(ChainDev* c, const OpDev op, int t, int bcols,
     __syncthreads();
     const int n = wv.n;
     if (n == 0) {
-      const blk::BlockRec& r = M->b[b0];
+      const blk::BlockRec& r = ss.b[b0];
       float* W32 = c->X;
       float* V32 = c->X + (size_t)r.q * r.p;
-      blk::gather_block<NT, float, float>(c, op.k, ss, r, theta, W32, r.q, V32, r.p);
+      int c0 = 0;
+      blk::gather_block<NT, float, float>(c, op.k, ss, r, theta, W32, r.q, V32, r.p, c0);
       __syncthreads();
       const int sw = cta_jacobi_f32(W32, r.q, r.p, V32, bcols, smem, sc, nullptr);
       if (sw < 0) {
@@ -474,16 +477,17 @@ __device__ void two_site_op_mixed(ChainDev* c, const OpDev op, int t, int bcols,
       b0 += 1;
       continue;
     }
+    int c0 = 0;
     for (int i = 0; i < n; ++i) {
-      const blk::BlockRec& r = M->b[b0 + i];
+      const blk::BlockRec& r = ss.b[b0 + i];
       float* W32 = smem + wv.off[i];
       float* V32 = W32 + (size_t)r.p * (r.q | 1);
-      blk::gather_block<NT, float, float>(c, op.k, ss, r, theta, W32, r.q | 1, V32, r.p | 1);
+      blk::gather_block<NT, float, float>(c, op.k, ss, r, theta, W32, r.q | 1, V32, r.p | 1, c0);
     }
     __syncthreads();
     const int g = blk::my_group(wv, warp);
     if (g >= 0) {
-      const blk::BlockRec& r = M->b[b0 + g];
+      const blk::BlockRec& r = ss.b[b0 + g];
       float* W32 = smem + wv.off[g];
       float* V32 = W32 + (size_t)r.p * (r.q | 1);
       const int sw = blk::jacobi_group<float>(W32, r.q, r.q | 1, r.p, V32, r.p | 1, V32 + (size_t)r.p * (r.p | 1),
@@ -493,7 +497,7 @@ __device__ void two_site_op_mixed(ChainDev* c, const OpDev op, int t, int bcols,
     }
     __syncthreads();
     for (int i = 0; i < n; ++i) {
-      const blk::BlockRec& r = M->b[b0 + i];
+      const blk::BlockRec& r = ss.b[b0 + i];
       const float* W32 = smem + wv.off[i];
       float* V32 = smem + wv.off[i] + (size_t)r.p * (r.q | 1);
       promote_w(W32, r.q | 1, V32, r.p | 1, r.q, r.p, c->W + r.woff, c->sig + r.svoff);
@@ -502,7 +506,7 @@ __device__ void two_site_op_mixed(ChainDev* c, const OpDev op, int t, int bcols,
     if (polish && g >= 0) {
       // binary64 polish by the same groups: W in binary64 (global), V stays
       // in shared memory in binary32; norms of block g in c->sig
-      const blk::BlockRec& r = M->b[b0 + g];
+      const blk::BlockRec& r = ss.b[b0 + g];
       float* V32 = smem + wv.off[g] + (size_t)r.p * (r.q | 1);
       const int s64 = blk::jacobi_group<double, float, 2>(c->W + r.woff, r.q, r.q, r.p, V32, r.p | 1, c->sig + r.svoff,
                                                        warp - wv.w0[g], wv.nw[g], g + 1, g, gs, kPolishStop,
@@ -511,7 +515,7 @@ __device__ void two_site_op_mixed(ChainDev* c, const OpDev op, int t, int bcols,
     }
     __syncthreads();
     for (int i = 0; i < n; ++i) {
-      const blk::BlockRec& r = M->b[b0 + i];
+      const blk::BlockRec& r = ss.b[b0 + i];
       const float* V32 = smem + wv.off[i] + (size_t)r.p * (r.q | 1);
       promote_v(V32, r.p | 1, r.q, r.p, c->W + r.woff, c->V + r.voff, c->sig + r.svoff, polish);
       __syncthreads();
@@ -522,28 +526,17 @@ __device__ void two_site_op_mixed(ChainDev* c, const OpDev op, int t, int bcols,
         set_error(c, HM_ERR_NUMERIC, t, ctx_err);
         return;
       }
-      const blk::BlockRec& r = M->b[b0 + i];
+      const blk::BlockRec& r = ss.b[b0 + i];
       const int64_t cb = (int64_t)r.q * r.p * r.p;
       if (cb > cost) cost = cb, sw32 = code % 1000, sw64 = code / 1000;
     }
     b0 += n;
     __syncthreads();
   }
-  blk::finish<NT>(c, op, t, ss, c->theta, ctx_err, sw32, sw64);
-  if (threadIdx.x == 0 && ss.kk > 0) {
-    double k1 = 0.0;
-    for (int i = 0; i < ss.nin; ++i) {
-      const int Q = M->qin[i];
-      double rows = 0.0, cols = 0.0;
-      for (int u = 0; u < 3; ++u) {
-        rows += blk::seg_of(M, 0, ss.qbase, Q - ss.sk * blk::mval(u)).len;
-        cols += blk::seg_of(M, 2, ss.qbase, Q + ss.sk1 * blk::mval(u)).len;
-      }
-      k1 += 2.0 * rows * blk::seg_of(M, 1, ss.qbase, Q).len * cols;
-    }
-    c->stats[ST_K1] += k1;
-    c->stats[ST_K2] += 2.0 * 81.0 * c->chi[op.k] * c->chi[op.k + 2];
-  }
+  double* tiles = reinterpret_cast<double*>(smem);
+  char* scratch = reinterpret_cast<char*>(tiles + kTileDoubles);
+  if (kTileDoubles * sizeof(double) + blk::finish_bytes(ss.P) > kBlockSmem) scratch = reinterpret_cast<char*>(c->theta);
+  blk::finish<NT>(c, op, t, ss, scratch, tiles, ctx_err, sw32, sw64);
   __syncthreads();
 }
 

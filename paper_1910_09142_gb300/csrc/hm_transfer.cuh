@@ -79,20 +79,7 @@ __device__ void build_tabs(const ChainDev* c, int pos, bool dense, Tabs& t) {
   __syncthreads();
 }
 
-// Calls f(e) for this lane's share of the n elements of one block: the
-// CTA's warps take chunks of 32 elements in turn over all blocks of a pass
-// (c0 counts the chunks so far).
-template <int NT, typename F>
-__device__ __forceinline__ void share(int n, int& c0, F&& f) {
-  constexpr int NW = NT / 32;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nch = (n + 31) >> 5;
-  for (int ch = (unsigned)(warp - c0) % NW; ch < nch; ch += NW) {
-    const int e = ch * 32 + lane;
-    if (e < n) f(e);
-  }
-  c0 += nch;
-}
+using blk::share;
 
 // Sum over k < n of x[k sx] y[k sy].
 __device__ __forceinline__ double dot_strided(const double* __restrict__ x, size_t sx, const double* __restrict__ y,
