@@ -1026,6 +1026,7 @@ struct WaveSh {
   int32_t b0, n;
   int32_t w0[15], nw[15], sw[15];
   int32_t off[15];                        // shared-memory offset (elements) of block i
+  int32_t koff[15];                       // scratch offset (elements) of block i (hm_refine.cuh)
 };
 
 // Index of this warp's group in the wave, or -1 (an idle warp).

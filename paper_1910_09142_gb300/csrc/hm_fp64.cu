@@ -20,9 +20,11 @@
 
 #include <cmath>
 #include <cstdint>
+#include <mutex>
 
 #include "hm_block.cuh"
 #include "hm_internal.h"
+#include "hm_refine.cuh"
 #include "hm_transfer.cuh"
 
 namespace hm {
@@ -46,17 +48,18 @@ struct TransferSh {
   int32_t ival;
 };
 
-// Shared memory of the evolve kernel: the charge-run tables of a split while
-// it is prepared, then the transposition tiles and the value lists of finish()
-// (more than 400 values use the theta buffer).
-constexpr int kTileDoubles = NT / 32 * 8 * 33;
-constexpr int kBufDoubles = kTileDoubles + 2496;
+// Dynamic shared memory of the evolve kernel: one CTA of 512 threads per SM,
+// or two of 256 (a batch with more chains than SMs).  In turn the charge-run
+// tables of a split, the decompositions of a wave of blocks, and finish()'s
+// transposition tiles and value lists.
+constexpr int kWideNT = 512;
+constexpr size_t kWideSmem = 204 * 1024, kPairSmem = 104 * 1024;
+static_assert(sizeof(blk::PrepTab) <= kPairSmem, "prepare's tables");
 struct EvolveSh {
-  double buf[kBufDoubles];
   blk::SplitSh split;
+  blk::WaveSh wave;
   blk::GroupSh gs;
 };
-static_assert(sizeof(blk::PrepTab) <= kBufDoubles * sizeof(double), "prepare's tables");
 
 struct Shared {
   GemmSmem g;
@@ -394,47 +397,180 @@ __device__ void two_site_op(ChainDev* c, const OpDev op, int t, Shared& sh, int3
   __syncthreads();
 }
 
+// Blocks of fewer columns go straight to the binary64 sweeps.
+constexpr int kPrecond = 12;
+// Stopping ratios: of the binary64 sweeps (the next sweep's off-diagonals
+// would be of order its square), and of the binary32 sweeps before them (what
+// they leave, ~1e-6, is binary32 resolution).
+constexpr double kStop64 = 1e-9;
+constexpr float kStopPre = 1e-3f;
+
+// Doubles of shared memory a block takes: W and V (odd leading dimensions), the
+// column norms.  The binary32 stage before it (W, V, norms) fits in W's part.
+__device__ __forceinline__ int64_t block_doubles(int q, int p) {
+  return (int64_t)p * max(q | 1, ((q | 1) + (p | 1) + 4) / 2) + (int64_t)p * (p | 1) + p;
+}
+
+// Decomposition of one block by the nw warps of a group: A (q x p, global) to W
+// = A V with orthogonal columns and orthonormal V, both in shared memory.
+//
+// What bounds it is the binary64 pipe: a Jacobi sweep costs 4.5 q p^2 of its
+// instructions, and from scratch it takes 7 to 10 sweeps.  The first ones only
+// look for the vectors, and binary32 does that 64 x faster: binary32 sweeps on
+// the rounded block give V to ~1e-6, two orthonormalisation steps V <- V - V (V^T V -
+// 1) / 2 make it orthonormal to binary64 (the first on split binary32 sums, the
+// second with p^3 / 2 binary64 products; both corrections are small enough to
+// be multiplied in binary32), W = A V is formed in binary64 (q p^2), and the
+// binary64 sweeps run from there under their own stopping rule, 2 or 3 of
+// them, the last mostly tests.  So nothing of the binary32 stage reaches the
+// result but the starting point.  KT: scratch, p ldk_of(p) floats (global).
+// Returns the binary64 sweeps, or -1.
+__device__ int decompose_block(const double* A, int q, int p, double* base, float* KT, int lw, int nw, int bar, int g,
+                               blk::GroupSh& gs) {
+  const int lane = threadIdx.x & 31, nthr = 32 * nw;
+  const int ldw = q | 1, ldv = p | 1;
+  double* W = base;
+  double* V = base + (block_doubles(q, p) - (int64_t)p * ldv - p);
+  double* nrm = V + (size_t)p * ldv;
+  int pre = 0;
+  if (p >= kPrecond) {
+    float* W32 = reinterpret_cast<float*>(base);
+    float* V32 = W32 + (size_t)p * ldw;
+    float* n32 = V32 + (size_t)p * ldv;
+    for (int j = lw; j < p; j += nw) {
+      for (int i = lane; i < q; i += 32) W32[(size_t)j * ldw + i] = blk::narrow(A[(size_t)j * q + i]);
+      for (int i = lane; i < p; i += 32) V32[(size_t)j * ldv + i] = i == j ? 1.0f : 0.0f;
+    }
+    blk::group_sync(bar, nthr);
+    pre = blk::jacobi_group<float>(W32, q, ldw, p, V32, ldv, n32, lw, nw, bar, g, gs, kStopPre, kMaxSweeps);
+    blk::group_sync(bar, nthr);
+    if (pre > 0) {
+      // V -> binary64, orthonormal
+      refine::unit_terms(V32, p, ldv, n32, KT, lw, nw);
+      blk::group_sync(bar, nthr);
+      refine::pair_terms<true>(V32, p, ldv, p, n32, n32, KT, lw, nw);
+      blk::group_sync(bar, nthr);
+      int x = 0;
+      refine::add_product<false>(V32, p, ldv, p, KT, V, ldv, lw, nw, x);
+      blk::group_sync(bar, nthr);
+      refine::ortho_terms64(V, p, ldv, KT, lw, nw);
+      blk::group_sync(bar, nthr);
+      x = 0;
+      refine::add_product<true>(V32, p, ldv, p, KT, V, ldv, lw, nw, x);
+      blk::group_sync(bar, nthr);
+      refine::product64(A, q, p, V, ldv, W, ldw, lw, nw);
+    }
+  }
+  if (pre <= 0) {
+    // a small block, or binary32 did not converge: from A and V = 1
+    for (int j = lw; j < p; j += nw) {
+      for (int i = lane; i < q; i += 32) W[(size_t)j * ldw + i] = A[(size_t)j * q + i];
+      for (int i = lane; i < p; i += 32) V[(size_t)j * ldv + i] = i == j ? 1.0 : 0.0;
+    }
+  }
+  blk::group_sync(bar, nthr);
+  return blk::jacobi_group<double, double, 2>(W, q, ldw, p, V, ldv, nrm, lw, nw, bar, g, gs, kStop64, kMaxSweeps);
+}
+
 // One two-site op of a chain, block by block in the S^z charge of the new
 // middle bond (Sec. II.C): theta by block GEMMs, the gate within its
-// conserved sectors, a binary64 one-sided Jacobi per block, then one
-// truncation over the union of the blocks' singular values (Sec. II).  The
-// blocks take the whole CTA in turn: the binary64 pipe (about 2 FMA per
-// clock per SM on GB300) is the bound, and every warp of the CTA is needed
-// to hide the latency of the global-memory rotations (splitting the warps
-// over the blocks of a split measured 1.7x slower).
-__device__ void two_site_op_blocked(ChainDev* c, const OpDev op, int t, EvolveSh& sh, int32_t* ctx_err) {
+// conserved sectors, the blocks' decompositions, then one truncation over the
+// union of the blocks' singular values (Sec. II).  The blocks of a split that
+// fit in shared memory together form a wave and are decomposed at once, each
+// by its own warp group; a block too large for shared memory takes the whole
+// CTA and works on global memory.
+template <int NTE>
+__device__ void two_site_op_blocked(ChainDev* c, const OpDev op, int t, double* buf, size_t buf_bytes, EvolveSh& sh,
+                                    int32_t* ctx_err) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   blk::SplitSh& ss = sh.split;
-  blk::PrepTab& tab = *reinterpret_cast<blk::PrepTab*>(sh.buf);
-  if (!blk::prepare<NT>(c, op, ss, tab)) blk::prepare<NT>(c, op, ss, tab);
-  blk::theta_blocks<NT, TM, TN, TK, double>(c, op.k, ss, c->theta, sh.buf);
-  int c0 = 0;
-  for (int b = 0; b < ss.nblk; ++b) {
-    const blk::BlockRec& r = ss.b[b];
-    blk::gather_block<NT, double, double>(c, op.k, ss, r, c->theta, c->W + r.woff, r.q, c->V + r.voff, r.p, c0);
+  blk::WaveSh& wv = sh.wave;
+  blk::PrepTab& tab = *reinterpret_cast<blk::PrepTab*>(buf);
+  if (!blk::prepare<NTE>(c, op, ss, tab)) blk::prepare<NTE>(c, op, ss, tab);
+  blk::theta_direct<NTE, double>(c, op.k, ss, c->theta);
+  {
+    int c0 = 0;
+    for (int b = 0; b < ss.nblk; ++b) {
+      const blk::BlockRec& r = ss.b[b];
+      blk::gather_block<NTE, double, double>(c, op.k, ss, r, c->theta, c->W + r.woff, r.q, c->V + r.voff, r.p, c0);
+    }
   }
   __syncthreads();
   int sweeps = 0;
   int64_t cost = -1;
-  for (int b = 0; b < ss.nblk; ++b) {
-    const blk::BlockRec& r = ss.b[b];
-    const int sw = blk::jacobi_group<double, double, 2>(c->W + r.woff, r.q, r.q, r.p, c->V + r.voff, r.p, c->sig,
-                                             threadIdx.x >> 5, NT / 32, 1, 0, sh.gs, 1e-9, kMaxSweeps);
-    if (sw < 0) {
-      set_error(c, HM_ERR_NUMERIC, t, ctx_err);
-      return;
+  const int64_t cap = (int64_t)(buf_bytes / sizeof(double));
+  for (int b0 = 0; b0 < ss.nblk;) {
+    if (tid == 0) {
+      int64_t used = 0;
+      int n = 0, koff = 0, p[15];
+      while (b0 + n < ss.nblk && n < 15 && n < NTE / 32) {
+        const blk::BlockRec& r = ss.b[b0 + n];
+        const int64_t need = block_doubles(r.q, r.p);
+        if (used + need > cap) break;
+        wv.off[n] = (int32_t)used;
+        wv.koff[n] = koff;
+        koff += r.p * refine::ldk_of(r.p);
+        p[n] = r.p;
+        used += need;
+        ++n;
+      }
+      wv.b0 = b0;
+      wv.n = n;
+      if (n > 0) blk::assign_warps(p, n, NTE / 32, wv.w0, wv.nw);
     }
-    const int64_t cb = (int64_t)r.q * r.p * r.p;   // sweeps of the costliest block
-    if (cb > cost) cost = cb, sweeps = sw;
+    __syncthreads();
+    const int n = wv.n;
+    if (n == 0) {
+      const blk::BlockRec& r = ss.b[b0];
+      const int sw = blk::jacobi_group<double, double, 2>(c->W + r.woff, r.q, r.q, r.p, c->V + r.voff, r.p, c->sig, warp,
+                                                          NTE / 32, 1, 0, sh.gs, kStop64, kMaxSweeps);
+      if (sw < 0) {
+        set_error(c, HM_ERR_NUMERIC, t, ctx_err);
+        return;
+      }
+      const int64_t cb = (int64_t)r.q * r.p * r.p;   // sweeps of the costliest block
+      if (cb > cost) cost = cb, sweeps = sw;
+      b0 += 1;
+      __syncthreads();
+      continue;
+    }
+    const int g = blk::my_group(wv, warp);
+    if (g >= 0) {
+      const blk::BlockRec& r = ss.b[b0 + g];
+      const int lw = warp - wv.w0[g], nw = wv.nw[g], q = r.q, p = r.p;
+      double* W = buf + wv.off[g];
+      // theta is free once every block is gathered: its buffer holds the K's
+      const int sw = decompose_block(c->W + r.woff, q, p, W, reinterpret_cast<float*>(c->theta) + wv.koff[g], lw, nw,
+                                     g + 1, g, sh.gs);
+      if (lw == 0 && lane == 0) wv.sw[g] = sw;
+      const double* V = W + (block_doubles(q, p) - (int64_t)p * (p | 1) - p);
+      for (int j = lw; j < p; j += nw) {
+        for (int i = lane; i < q; i += 32) c->W[r.woff + (size_t)j * q + i] = W[(size_t)j * (q | 1) + i];
+        for (int i = lane; i < p; i += 32) c->V[r.voff + (size_t)j * p + i] = V[(size_t)j * (p | 1) + i];
+      }
+    }
+    __syncthreads();
+    for (int i = 0; i < n; ++i) {
+      if (wv.sw[i] < 0) {
+        set_error(c, HM_ERR_NUMERIC, t, ctx_err);
+        return;
+      }
+      const blk::BlockRec& r = ss.b[b0 + i];
+      const int64_t cb = (int64_t)r.q * r.p * r.p;
+      if (cb > cost) cost = cb, sweeps = wv.sw[i];
+    }
+    b0 += n;
     __syncthreads();
   }
-  char* scratch = reinterpret_cast<char*>(sh.buf + kTileDoubles);
-  if (blk::finish_bytes(ss.P) > (kBufDoubles - kTileDoubles) * sizeof(double)) scratch = reinterpret_cast<char*>(c->theta);
-  blk::finish<NT>(c, op, t, ss, scratch, sh.buf, ctx_err, sweeps, 0);
+  constexpr int tiles = NTE / 32 * 8 * 33;
+  char* scratch = reinterpret_cast<char*>(buf + tiles);
+  if (tiles * sizeof(double) + blk::finish_bytes(ss.P) > buf_bytes) scratch = reinterpret_cast<char*>(c->theta);
+  blk::finish<NTE>(c, op, t, ss, scratch, buf, ctx_err, sweeps, 0);
   __syncthreads();
 }
 
-__global__ void __launch_bounds__(NT) evolve_fp64_kernel(BatchArg b, OutArg o) {
-  __shared__ EvolveSh sh;
+template <int NTE>
+__device__ void evolve_chain(const BatchArg& b, const OutArg& o, double* buf, size_t buf_bytes, EvolveSh& sh) {
   ChainDev* c = b.c[blockIdx.x];
   const OpDev* ops = b.ops_override ? b.ops_override : c->ops;
   const int n_ops = b.ops_override ? b.n_override : c->n_ops;
@@ -445,9 +581,21 @@ __global__ void __launch_bounds__(NT) evolve_fp64_kernel(BatchArg b, OutArg o) {
   for (int t = t0; t < t1; ++t) {
     if (*(volatile int32_t*)c->status != 0) return;
     __syncthreads();
-    two_site_op_blocked(c, ops[t], t, sh, o.ctx_err);
+    two_site_op_blocked<NTE>(c, ops[t], t, buf, buf_bytes, sh, o.ctx_err);
     __syncthreads();
   }
+}
+
+__global__ void __launch_bounds__(kWideNT, 1) evolve_fp64_wide_kernel(BatchArg b, OutArg o) {
+  extern __shared__ double dsm[];
+  __shared__ EvolveSh sh;
+  evolve_chain<kWideNT>(b, o, dsm, kWideSmem, sh);
+}
+
+__global__ void __launch_bounds__(NT, 2) evolve_fp64_pair_kernel(BatchArg b, OutArg o) {
+  extern __shared__ double dsm[];
+  __shared__ EvolveSh sh;
+  evolve_chain<NT>(b, o, dsm, kPairSmem, sh);
 }
 
 // Step 3 (Sec. I.C.1): <S_i.S_j> and <Sz_i Sz_j> on every measured bond.
@@ -948,7 +1096,29 @@ static int check_launch() {
 
 int launch_evolve_fp64(const BatchArg& b, const OutArg& o, void* stream) {
   if (b.n <= 0) return HM_OK;
-  evolve_fp64_kernel<<<b.n, NT, 0, (cudaStream_t)stream>>>(b, o);
+  // opt in to the dynamic shared memory once per device (a lock: serving
+  // workers may launch from several host threads)
+  static std::mutex mu;
+  static bool ready[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return HM_ERR_CUDA;
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    if (dev < 0 || dev >= 64 || !ready[dev]) {
+      if (cudaFuncSetAttribute(evolve_fp64_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWideSmem) !=
+              cudaSuccess ||
+          cudaFuncSetAttribute(evolve_fp64_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem) !=
+              cudaSuccess)
+        return HM_ERR_CUDA;
+      if (dev >= 0 && dev < 64) ready[dev] = true;
+    }
+  }
+  const int sms = device_sm_count();
+  if (sms > 0 && b.n > sms) {
+    evolve_fp64_pair_kernel<<<b.n, NT, kPairSmem, (cudaStream_t)stream>>>(b, o);
+  } else {
+    evolve_fp64_wide_kernel<<<b.n, kWideNT, kWideSmem, (cudaStream_t)stream>>>(b, o);
+  }
   return check_launch();
 }
 
@@ -1070,8 +1240,6 @@ two_site_static_kernel(double* scratch, const double* A, const double* B, int ch
 }  // namespace
 
 }  // namespace hm
-
-#include <mutex>
 
 namespace {
 

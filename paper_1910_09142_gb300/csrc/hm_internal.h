@@ -112,6 +112,8 @@ int launch_collapse_fp64(const BatchArg& b, const OutArg& o, void* stream);
 int launch_reset(const BatchArg& b, const OutArg& o, int draw_initial, void* stream);
 // Susceptibility double sum (Eq. sus), raw and unnormalised by beta: o.obs[i].
 int launch_susceptibility_fp64(const BatchArg& b, const OutArg& o, void* stream);
+// SMs of the current device, cached per device ordinal (0: unknown) (hm_mixed.cu).
+int device_sm_count();
 // Message returned by hm_last_error(NULL) (hm_api.cu).
 void set_global_error(const char* msg);
 

@@ -584,9 +584,10 @@ int launch_kernel(const BatchArg& b, const OutArg& o, int chi_cap, int polish, v
   return cudaGetLastError() == cudaSuccess ? HM_OK : HM_ERR_CUDA;
 }
 
+}  // namespace
+
 #if HM_MIXED_CTAS_PER_SM == 1
-// SMs of the current device (cached per device ordinal).
-int sm_count() {
+int device_sm_count() {
   static std::mutex mu;
   static int count[64] = {};
   int dev = 0;
@@ -598,15 +599,13 @@ int sm_count() {
 }
 #endif
 
-}  // namespace
-
 #if HM_MIXED_CTAS_PER_SM == 1
 // A batch with more chains than SMs whose charge blocks fit half an SM's
 // shared memory runs two chains per SM (hm_mixed_pair.cu): all of them are
 // resident at once, and each SM interleaves two independent CTAs.
 int launch_evolve_mixed(const BatchArg& b, const OutArg& o, int chi_cap, int polish, void* stream) {
   if (b.n <= 0) return HM_OK;
-  const int sms = sm_count();
+  const int sms = device_sm_count();
   if (chi_cap <= kPairChiCap && sms > 0 && b.n > sms) return launch_evolve_mixed_pair(b, o, chi_cap, polish, stream);
   return launch_kernel(b, o, chi_cap, polish, stream);
 }

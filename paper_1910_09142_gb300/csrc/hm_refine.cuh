@@ -1,0 +1,423 @@
+// Binary64-accurate finish of a block that the binary32 Jacobi sweeps have
+// diagonalised (HM_MIXED), without a binary64 sweep.
+//
+// After the sweeps W (q x p, binary32, shared memory) has columns that are
+// orthogonal to E ~ 1e-6 relative, and V its rotations.  A binary64 Jacobi
+// sweep on W takes 2.5 q p^2 instructions of the binary64 pipe (2 a clock and
+// SM): 1.2 M clocks at q = p = 100, a quarter of an evolution.  Its rotations
+// are tiny, so to first order they commute and the whole sweep is one product
+//   W' = W (I + K),  V' = V (I + K),  K_ij = -K_ji = tan of pair (i, j),
+// with K ~ 1e-6: a binary32 product K-wise gives W' to 1e-13 and leaves
+// off-diagonals of order E^2, as the sweep does.  What needs more than
+// binary32 is E itself.  W holds binary32 numbers, so a product of two of its
+// entries splits exactly into two binary32 numbers, and a sum against a
+// constant larger than every partial sum splits exactly too: dot2 below spends
+// seven binary32 instructions a term (64 x the rate of the binary64 pipe) and
+// returns the Gram entry to about 2^-45 of the columns' norms.
+//
+// Two columns of nearly the same norm have a large angle whatever their
+// overlap; their pairs (|b - a| < kNear max(a, b)) are left out of K and
+// rotated one after another in binary64 afterwards.  When too many pairs are near (an
+// exactly degenerate spectrum), or E is not small, the binary64 sweeps of
+// jacobi_group run on W' and V' as well.
+//
+// The columns of V come out of the sweeps up to ~1e-5 longer than 1 (a
+// binary32 rotation with a small angle has cosine exactly 1, so it stretches
+// both columns by sqrt(1 + t^2), always the same way).  Left in, that weights
+// each kept vector: a systematic energy error of ~2e-5 (measured).  The
+// rotations stay conformal and W = theta V holds column by column, so column
+// j of both factors is scaled by 1 / |v_j| = 1 + delta_j; delta is K's diagonal.
+#pragma once
+
+#include <cstdint>
+
+#include "hm_block.cuh"
+#include "hm_internal.h"
+
+namespace hm {
+namespace refine {
+
+// Relative gap of two squared column norms below which a pair is rotated
+// explicitly.  Outside it |t| < E / 0.02 ~ 1e-4, and the terms the first
+// order leaves out are below 1e-4 E.
+constexpr float kNear = 0.02f;
+
+// A value as an unevaluated binary32 sum.
+struct F2 {
+  float h, l;
+};
+
+// Sum of two F2 (Knuth's exact two-sum on the leading parts).
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+  const float s = a.h + b.h, bb = s - a.h;
+  const float e = (a.h - (s - bb)) + (b.h - bb);
+  return {s, e + a.l + b.l};
+}
+
+__device__ __forceinline__ F2 normal2(F2 a) {
+  const float s = a.h + a.l;
+  return {s, a.l - (s - a.h)};
+}
+
+// Running dot product: t = big + the products rounded to big's last bit, l =
+// everything below.  big > 2 |every partial sum|, so t + p, (t + p) - t and
+// p - ((t + p) - t) are exact splits (Dekker's fast two-sum).
+struct Dot2 {
+  float t, l;
+  __device__ __forceinline__ void start(float big) {
+    t = big;
+    l = 0.0f;
+  }
+  __device__ __forceinline__ void add(float x, float y) {
+    const float p = x * y;
+    const float e = fmaf(x, y, -p);
+    const float s = t + p;
+    l += p - (s - t);
+    l += e;
+    t = s;
+  }
+  __device__ __forceinline__ F2 get(float big) const { return {t - big, l}; }
+};
+
+// Power of two above 4 x (x > 0, normal).
+__device__ __forceinline__ float above(float x) {
+  return __uint_as_float((__float_as_uint(x) & 0x7f800000u) + (3u << 23));
+}
+
+// Shared-memory floats a block needs besides W and V: squared norms (high and
+// low part), delta.
+__device__ __forceinline__ int extra(int p) { return 3 * p; }
+
+// Leading dimension of K's transpose (four entries are loaded at once).
+__device__ __forceinline__ int ldk_of(int p) { return (p + 3) & ~3; }
+
+__device__ __forceinline__ bool near_pair(float a, float b) { return fabsf(b - a) < kNear * fmaxf(a, b); }
+
+// Squared norm of one column by a warp.
+__device__ __forceinline__ F2 warp_norm2(const float* x, int n) {
+  const int lane = threadIdx.x & 31;
+  float m = 0.0f;
+  for (int i = lane; i < n; i += 32) m = fmaf(x[i], x[i], m);
+  m = blk::warp_sum_t(m);
+  if (!(m > 0.0f)) return {0.0f, 0.0f};
+  const float big = above(m);
+  Dot2 d;
+  d.start(big);
+  for (int i = lane; i < n; i += 32) d.add(x[i], x[i]);
+  F2 s = d.get(big);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    s = add2(s, {__shfl_xor_sync(0xffffffffu, s.h, o), __shfl_xor_sync(0xffffffffu, s.l, o)});
+  return normal2(s);
+}
+
+// x' = x + (x delta + products with K): one column entry, binary64.
+__device__ __forceinline__ double corrected(float x, float corr) { return blk::widen(x) + blk::widen(corr); }
+
+// delta_j and the squared norms of the columns; KT: zeroed padding and the diagonal.
+__device__ inline void column_terms(const float* W, int q, int ldw, const float* V, int p, int ldv, float* ah, float* al,
+                             float* dl, float* KT, int lw, int nw) {
+  const int lane = threadIdx.x & 31;
+  const int ldk = ldk_of(p);
+  for (int j = lw; j < p; j += nw) {
+    const F2 a = warp_norm2(W + (size_t)j * ldw, q), v = warp_norm2(V + (size_t)j * ldv, p);
+    if (lane == 0) {
+      ah[j] = a.h;
+      al[j] = a.l;
+      // 1 / sqrt(1 + u) - 1 (u ~ 1e-5; a null column keeps its scale)
+      const float u = (v.h - 1.0f) + v.l;
+      const float d = v.h > 0.5f ? u * (-0.5f + u * (0.375f - 0.3125f * u)) : 0.0f;
+      dl[j] = d;
+      if (KT) KT[(size_t)j * ldk + j] = d;
+    }
+    if (KT && lane >= 1 && p + lane - 1 < ldk) KT[(size_t)j * ldk + p + lane - 1] = 0.0f;
+  }
+}
+
+// The diagonal of the orthonormalisation step, -1/2 of |v_j|^2 - 1, and the
+// squared norms (ah); KT: zeroed padding.
+__device__ inline void unit_terms(const float* V, int p, int ldv, float* ah, float* KT, int lw, int nw) {
+  const int lane = threadIdx.x & 31;
+  const int ldk = ldk_of(p);
+  for (int j = lw; j < p; j += nw) {
+    const F2 v = warp_norm2(V + (size_t)j * ldv, p);
+    if (lane == 0) {
+      ah[j] = v.h;
+      KT[(size_t)j * ldk + j] = -0.5f * ((v.h - 1.0f) + v.l);
+    }
+    if (lane >= 1 && p + lane - 1 < ldk) KT[(size_t)j * ldk + p + lane - 1] = 0.0f;
+  }
+}
+
+// K's off-diagonal entries: a warp takes four columns i against 32 columns j
+// (a lane each).  ORTHO = false: the rotations of W's columns.  ORTHO = true (al
+// unused): -1/2 of the overlaps of V's columns, the step that makes them
+// orthonormal.  Returns this lane's largest |E|.
+template <bool ORTHO>
+__device__ inline float pair_terms(const float* W, int q, int ldw, int p, const float* ah, const float* al, float* KT, int lw,
+                            int nw) {
+  constexpr int R = 4;
+  const int lane = threadIdx.x & 31;
+  const int ldk = ldk_of(p);
+  const int gi = (p + R - 1) / R;
+  float emax = 0.0f;
+  int x = 0;
+  for (int g = 0; g < gi; ++g) {
+    for (int j0 = (g * R) & ~31; j0 < p; j0 += 32, ++x) {
+      if (x % nw != lw) continue;
+      const int j = j0 + lane, jj = j < p ? j : p - 1;
+      const float b = ah[jj];
+      Dot2 d[R];
+      float big[R];
+      const float* xi[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int i = min(g * R + r, p - 1);
+        xi[r] = W + (size_t)i * ldw;
+        const float a = ah[i];
+        // |every partial sum| <= sqrt(a b)
+        big[r] = above(fmaxf(sqrtf(a) * sqrtf(b), 1e-36f));
+        d[r].start(big[r]);
+      }
+      const float* y = W + (size_t)jj * ldw;
+#pragma unroll 2
+      for (int k = 0; k < q; ++k) {
+        const float yk = y[k];
+#pragma unroll
+        for (int r = 0; r < R; ++r) d[r].add(xi[r][k], yk);
+      }
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int i = g * R + r;
+        if (i >= p || j >= p || j <= i) continue;
+        const float a = ah[i];
+        const F2 s = normal2(d[r].get(big[r]));
+        float t = 0.0f;
+        if (ORTHO) {
+          KT[(size_t)i * ldk + j] = KT[(size_t)j * ldk + i] = -0.5f * (s.h + s.l);
+          continue;
+        }
+        if (a > blk::kTiny32 && b > blk::kTiny32) {
+          emax = fmaxf(emax, fabsf(s.h) * (rsqrtf(a) * rsqrtf(b)));
+          // b - a exactly to binary32, then the rotation's tangent
+          if (s.h != 0.0f && !near_pair(a, b)) t = blk::jacobi_tangent32((b - a) + (al[j] - al[i]), s.h);
+        }
+        KT[(size_t)i * ldk + j] = -t;         // w_i' = w_i - t w_j
+        KT[(size_t)j * ldk + i] = t;          // w_j' = w_j + t w_i
+      }
+    }
+  }
+  return emax;
+}
+
+// out[:, j] = base[:, j] + X K[:, j], X n x p (shared, leading dimension ldx); base
+// = X, or out itself (ADD).  out: binary64 column-major, leading dimension
+// ldo.  A warp takes 128 rows x 4 columns; K comes four entries at a time, the
+// same for all lanes.  x: running task count (the tasks go round the warps).
+template <bool ADD>
+__device__ inline void add_product(const float* X, int n, int ldx, int p, const float* KT, double* out, int ldo,
+                                   int lw, int nw, int& x) {
+  const int lane = threadIdx.x & 31;
+  const int ldk = ldk_of(p);
+  for (int r0 = 0; r0 < n; r0 += 128) {
+    const int nu = min(4, (n - r0 + 31) >> 5);
+    for (int j0 = 0; j0 < p; j0 += 4, ++x) {
+      if (x % nw != lw) continue;
+      float acc[4][4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int y = 0; y < 4; ++y) acc[u][y] = 0.0f;
+      for (int i = 0; i < p; i += 4) {
+        float4 kv[4];
+#pragma unroll
+        for (int y = 0; y < 4; ++y) kv[y] = *reinterpret_cast<const float4*>(KT + (size_t)min(j0 + y, p - 1) * ldk + i);
+#pragma unroll
+        for (int z = 0; z < 4; ++z) {
+          const float* col = X + (size_t)min(i + z, p - 1) * ldx + r0 + lane;   // K's padding is 0
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (u < nu) {
+              const float w = r0 + lane + 32 * u < n ? col[32 * u] : 0.0f;
+#pragma unroll
+              for (int y = 0; y < 4; ++y) {
+                const float kz = z == 0 ? kv[y].x : (z == 1 ? kv[y].y : (z == 2 ? kv[y].z : kv[y].w));
+                acc[u][y] = fmaf(w, kz, acc[u][y]);
+              }
+            }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int r = r0 + lane + 32 * u;
+        if (u >= nu || r >= n) continue;
+#pragma unroll
+        for (int y = 0; y < 4; ++y)
+          if (j0 + y < p) {
+            double* o = out + (size_t)(j0 + y) * ldo + r;
+            *o = ADD ? *o + blk::widen(acc[u][y]) : corrected(X[(size_t)(j0 + y) * ldx + r], acc[u][y]);
+          }
+      }
+    }
+  }
+}
+
+// out[:, j] = (1 + delta_j) X[:, j].
+__device__ inline void scale_columns(const float* X, int n, int ldx, int p, const float* dl, double* out, int lw, int nw) {
+  const int lane = threadIdx.x & 31;
+  for (int j = lw; j < p; j += nw) {
+    const float d = dl[j];
+    for (int r = lane; r < n; r += 32) {
+      const float v = X[(size_t)j * ldx + r];
+      out[(size_t)j * n + r] = corrected(v, v * d);
+    }
+  }
+}
+
+// KT for the columns of a binary64 V that are orthonormal to binary32: -1/2 of
+// the overlaps minus 1, binary64 sums.  Same task split as pair_terms.
+__device__ inline void ortho_terms64(const double* V, int p, int ldv, float* KT, int lw, int nw) {
+  constexpr int R = 4;
+  const int lane = threadIdx.x & 31;
+  const int ldk = ldk_of(p);
+  int x = 0;
+  for (int g = 0; g < (p + R - 1) / R; ++g) {
+    for (int j0 = (g * R) & ~31; j0 < p; j0 += 32, ++x) {
+      if (x % nw != lw) continue;
+      const int j = j0 + lane, jj = j < p ? j : p - 1;
+      const double* y = V + (size_t)jj * ldv;
+      const double* xi[R];
+      double d[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        xi[r] = V + (size_t)min(g * R + r, p - 1) * ldv;
+        d[r] = 0.0;
+      }
+#pragma unroll 2
+      for (int k = 0; k < p; ++k) {
+        const double yk = y[k];
+#pragma unroll
+        for (int r = 0; r < R; ++r) d[r] = fma(xi[r][k], yk, d[r]);
+      }
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int i = g * R + r;
+        if (i >= p || j >= p || j < i) continue;
+        const float v = blk::narrow(-0.5 * (i == j ? d[r] - 1.0 : d[r]));
+        KT[(size_t)i * ldk + j] = v;
+        if (i != j) KT[(size_t)j * ldk + i] = v;
+      }
+    }
+  }
+}
+
+// out = A V: A q x p binary64 column-major (leading dimension q, global), V p x
+// p (shared, leading dimension ldv), out leading dimension ldo.  32 rows x 4
+// columns a warp.
+__device__ inline void product64(const double* __restrict__ A, int q, int p, const double* V, int ldv, double* out,
+                                 int ldo, int lw, int nw) {
+  const int lane = threadIdx.x & 31;
+  int x = 0;
+  for (int r0 = 0; r0 < q; r0 += 32) {
+    const int r = r0 + lane, rr = r < q ? r : q - 1;
+    for (int j0 = 0; j0 < p; j0 += 4, ++x) {
+      if (x % nw != lw) continue;
+      double acc[4] = {0.0, 0.0, 0.0, 0.0};
+      const double* a = A + rr;
+      const double* v[4];
+#pragma unroll
+      for (int y = 0; y < 4; ++y) v[y] = V + (size_t)min(j0 + y, p - 1) * ldv;
+      const int nj = min(4, p - j0);
+#pragma unroll 4
+      for (int i = 0; i < p; ++i) {
+        const double ai = a[(size_t)i * q];
+#pragma unroll
+        for (int y = 0; y < 4; ++y)
+          if (y < nj) acc[y] = fma(ai, v[y][i], acc[y]);
+      }
+      if (r < q)
+#pragma unroll
+        for (int y = 0; y < 4; ++y)
+          if (y < nj) out[(size_t)(j0 + y) * ldo + r] = acc[y];
+    }
+  }
+}
+
+// One binary64 rotation of columns i, j of W (q x p) and V (p x p) by a warp.
+__device__ inline void rotate64(double* W, int q, double* V, int p, int i, int j) {
+  const int lane = threadIdx.x & 31;
+  double* x = W + (size_t)i * q;
+  double* y = W + (size_t)j * q;
+  double a = 0.0, b = 0.0, g = 0.0;
+  for (int r = lane; r < q; r += 32) {
+    const double xr = x[r], yr = y[r];
+    a = fma(xr, xr, a);
+    b = fma(yr, yr, b);
+    g = fma(xr, yr, g);
+  }
+  a = blk::warp_sum64(a);
+  b = blk::warp_sum64(b);
+  g = blk::warp_sum64(g);
+  if (g == 0.0 || !(a > 0.0) || !(b > 0.0)) return;
+  const double t = blk::jacobi_tangent64(b - a, g);
+  const double cs = rsqrt(1.0 + t * t), sn = cs * t;
+  for (int r = lane; r < q; r += 32) {
+    const double xr = x[r], yr = y[r];
+    x[r] = cs * xr - sn * yr;
+    y[r] = sn * xr + cs * yr;
+  }
+  for (int r = lane; r < p; r += 32) {
+    const double xr = V[(size_t)i * p + r], yr = V[(size_t)j * p + r];
+    V[(size_t)i * p + r] = cs * xr - sn * yr;
+    V[(size_t)j * p + r] = sn * xr + cs * yr;
+  }
+  __syncwarp();
+}
+
+// Scales the columns of V to length 1 and those of W alike.  The explicit
+// rotations need it: V's columns overlap by the binary32 sweeps' ~1e-6, so a
+// large angle moves their lengths by as much (the first-order step's do not).
+__device__ inline void unit_columns(double* W, int q, double* V, int p, int lw, int nw) {
+  const int lane = threadIdx.x & 31;
+  for (int j = lw; j < p; j += nw) {
+    double s = 0.0;
+    for (int r = lane; r < p; r += 32) s = fma(V[(size_t)j * p + r], V[(size_t)j * p + r], s);
+    s = blk::warp_sum64(s);
+    if (fabs(s - 1.0) < 1e-13 || !(s > 0.5)) continue;
+    const double f = rsqrt(s);
+    for (int r = lane; r < p; r += 32) V[(size_t)j * p + r] *= f;
+    for (int r = lane; r < q; r += 32) W[(size_t)j * q + r] *= f;
+  }
+}
+
+// Rotates the near pairs in the order of their columns, one warp.  Columns
+// below binary32 resolution against the largest carry the rounding of theta
+// itself and are left as they are.  Returns the number found; stops (and the
+// caller sweeps) beyond `most`.
+__device__ inline int rotate_near(double* W, int q, double* V, int p, const float* ah, int most) {
+  const int lane = threadIdx.x & 31;
+  float top = 0.0f;
+  for (int j = lane; j < p; j += 32) top = fmaxf(top, ah[j]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+  const float floor = fmaxf(blk::kTiny32, top * 1.4e-14f);
+  int found = 0;
+  for (int i = 0; i + 1 < p; ++i) {
+    const float a = ah[i];
+    if (!(a > floor)) continue;
+    for (int j0 = i + 1; j0 < p; j0 += 32) {
+      const int j = j0 + lane;
+      const bool hit = j < p && ah[j] > floor && near_pair(a, ah[j]);
+      if (!__any_sync(0xffffffffu, hit)) continue;
+      for (int l = 0; l < 32; ++l) {
+        if (!blk::lane_value(hit ? 1 : 0, l)) continue;
+        if (++found > most) return found;
+        rotate64(W, q, V, p, i, j0 + l);
+      }
+    }
+  }
+  return found;
+}
+
+}  // namespace refine
+}  // namespace hm
