@@ -77,7 +77,10 @@ struct PrepTab {
 // Records of the usual split (at most 11 blocks measured on the benchmark
 // ladder) stay in shared memory; a split with more keeps all of its records
 // in the meta workspace.
-constexpr int kShBlk = 14;
+#ifndef HM_SH_BLK
+#define HM_SH_BLK 14
+#endif
+constexpr int kShBlk = HM_SH_BLK;
 
 // Shared scalars of a split (CTA shared memory).
 struct SplitSh {
@@ -391,7 +394,10 @@ __device__ __forceinline__ void share(int n, int& c0, F&& f) {
 // while the split has at most kThetaDirect products; above, the CTA goes
 // through the blocks in TM x TN x TK tiles in shared memory, which convert and
 // load each operand once per tile instead of once per product.
-constexpr double kThetaDirect = 131072.0;
+#ifndef HM_THETA_DIRECT
+#define HM_THETA_DIRECT 131072.0
+#endif
+constexpr double kThetaDirect = HM_THETA_DIRECT;
 
 template <int NT, typename T>
 __device__ void theta_direct(const ChainDev* c, int k, const SplitSh& s, T* __restrict__ theta) {
@@ -957,6 +963,248 @@ __device__ int jacobi_blocks(T* __restrict__ W, int q, int ldw, int p, TV* __res
   return -1;
 }
 
+// Two binary32 multiply-adds (products) in one instruction (sm_100 and later).
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+#if defined(__CUDA_ARCH__)
+  unsigned long long x, y, z, r;
+  memcpy(&x, &a, 8);
+  memcpy(&y, &b, 8);
+  memcpy(&z, &c, 8);
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(x), "l"(y), "l"(z));
+  float2 d;
+  memcpy(&d, &r, 8);
+  return d;
+#else
+  return {fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y)};
+#endif
+}
+
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+#if defined(__CUDA_ARCH__)
+  unsigned long long x, y, r;
+  memcpy(&x, &a, 8);
+  memcpy(&y, &b, 8);
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+  float2 d;
+  memcpy(&d, &r, 8);
+  return d;
+#else
+  return {a.x * b.x, a.y * b.y};
+#endif
+}
+
+// Leading dimension of a binary32 column for jacobi_regs: a multiple of four
+// (128-bit loads), an odd one (lanes that read the same rows of eight columns
+// hit different banks).
+__host__ __device__ __forceinline__ int ld4(int n) { return (((n + 3) >> 2) | 1) * 4; }
+
+// Rows 4 (sl + L u) .. + 3 of a column (n rows, padded with zeros to a multiple of 4).
+template <int U, int L>
+__device__ __forceinline__ void load_rows(const float* col, int n, int sl, bool ok, float2 (&x)[2 * U]) {
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int r = 4 * (sl + L * u);
+    float4 v = {0.0f, 0.0f, 0.0f, 0.0f};
+    if (ok && r < n) v = *reinterpret_cast<const float4*>(col + r);
+    x[2 * u] = {v.x, v.y};
+    x[2 * u + 1] = {v.z, v.w};
+  }
+}
+
+template <int U, int L>
+__device__ __forceinline__ void store_rows(float* col, int n, int sl, bool ok, const float2 (&x)[2 * U]) {
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int r = 4 * (sl + L * u);
+    if (ok && r < n)
+      *reinterpret_cast<float4*>(col + r) = {x[2 * u].x, x[2 * u].y, x[2 * u + 1].x, x[2 * u + 1].y};
+  }
+}
+
+// (x, y) <- (c x - s y, s x + c y).  Conformal whatever the rounding of c and s:
+// three shears by tan(angle / 2) and sin(angle) would take three operations
+// instead of four, but those two are rounded apart, and V's overlaps then
+// grew to 2e-6 (measured).
+template <int U, int L>
+__device__ __forceinline__ void rotate_rows(float2 (&x)[2 * U], float2 (&y)[2 * U], float c, float s, int n) {
+  const float2 cc = {c, c}, ss = {s, s}, ms = {-s, -s};
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    if (4 * L * u >= n) break;                  // warp-uniform
+#pragma unroll
+    for (int v = 2 * u; v < 2 * u + 2; ++v) {
+      const float2 a = x[v], b = y[v];
+      x[v] = fma2(cc, a, mul2(ms, b));
+      y[v] = fma2(cc, b, mul2(ss, a));
+    }
+  }
+}
+
+template <int U, int L>
+__device__ __forceinline__ void move_rows(float2 (&x)[2 * U], int n, int src) {
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    if (4 * L * u >= n) break;                  // warp-uniform
+#pragma unroll
+    for (int v = 2 * u; v < 2 * u + 2; ++v) {
+      x[v].x = lane_value(x[v].x, src);
+      x[v].y = lane_value(x[v].y, src);
+    }
+  }
+}
+
+// Block-ordered one-sided Jacobi as in jacobi_blocks, with super-columns of C
+// and a super-pair's 2 C columns of W and V in registers for its C sub-rounds
+// of cross pairs (L = 32 / C lanes a pair, q <= 4 L U; W and V 16-byte aligned,
+// leading dimensions multiples of 4).
+//
+// jacobi_blocks loads and stores every column of W and V once per rotation: 8 n
+// shared-memory words a pair against 9 n multiply-adds, and shared memory moves
+// 32 words a clock where the SM does 128 multiply-adds, so its traffic bounded
+// the sweeps of large blocks (82k clocks a sweep of a split against 107k at full
+// traffic, Lx = 16, chi = 200).  Here a column is loaded and stored once per
+// super-pair (128-bit accesses); lane group `sub` keeps column A + sub, and the
+// columns of the other super-column move on to the next group by shuffles.
+// What is left is the chain of a sub-round (dot product, reduction, angle,
+// rotation: ~300 clocks).  C = 4: eight pairs a sub-round (C = 8, 4 lanes a
+// pair) measured 3 % faster on blocks of up to 32 rows and 10 % slower above.
+// Lx = 9, 2W = 8, chi = 256, binary32, 152 chains: 269 ms a Markov step with
+// jacobi_blocks, 208 ms with this.
+template <int U, int C>
+__device__ int jacobi_regs(float* __restrict__ W, int q, int ldw, int p, float* __restrict__ V, int ldv,
+                           float* __restrict__ nrm, int lw, int nw, int bar, int g, GroupSh& gs, float stop,
+                           int max_sweeps) {
+  constexpr int L = 32 / C;
+  const int lane = threadIdx.x & 31;
+  const int sub = lane / L, sl = lane % L;
+  const int nthr = 32 * nw;
+  const float tol = sqrtf((float)q) * 1.1920928955078125e-07f;
+  const int ns = (p + C - 1) / C, ns2 = ns + (ns & 1), nsp = ns2 / 2;
+  const int next = ((sub + 1) & (C - 1)) * L + sl;   // the lane whose column this one takes next
+  for (int j = lw; j < p; j += nw) {                 // padding rows
+    if (q + lane < ((q + 3) & ~3)) W[(size_t)j * ldw + q + lane] = 0.0f;
+    if (p + lane < ((p + 3) & ~3)) V[(size_t)j * ldv + p + lane] = 0.0f;
+  }
+  for (int sweep = 1; sweep <= max_sweeps; ++sweep) {
+    for (int j = lw; j < p; j += nw) {
+      const float* cj = W + (size_t)j * ldw;
+      float s2 = 0.0f;
+      for (int i = lane; i < q; i += 32) s2 = fmaf(cj[i], cj[i], s2);
+      s2 = warp_sum_t(s2);
+      if (lane == 0) nrm[j] = s2;
+    }
+    if (lw == 0 && lane == 0) {
+      gs.flag[g] = 0;
+      gs.rbits[g] = 0u;
+    }
+    group_sync(bar, nthr);
+    float rmax = 0.0f;
+    int rot = 0;
+    for (int sr = 0; sr < ns2 - 1; ++sr) {
+      for (int sp = lw; sp < nsp; sp += nw) {                       // warp-uniform
+        const int m = ns2 - 1;             // (sr +- sp) mod m, as for the columns
+        int A, Bc;
+        if (sp == 0) {
+          A = sr;
+          Bc = m;
+        } else {
+          A = sr + sp;
+          if (A >= m) A -= m;
+          Bc = sr - sp;
+          if (Bc < 0) Bc += m;
+        }
+        const bool okA = A < ns, okB = Bc < ns;
+        if (sr == 0) {
+          // pairs inside A (the lower half of the groups) and inside B (the upper):
+          // the round robin of C columns
+          const int base = (sub < C / 2 ? A : Bc) * C, x = sub & (C / 2 - 1);
+          const bool ok = sub < C / 2 ? okA : okB;
+          for (int k = 0; k < C - 1; ++k) {
+            int a = base + (x == 0 ? k : (k + x) % (C - 1));
+            int b = base + (x == 0 ? C - 1 : (k + C - 1 - x) % (C - 1));
+            if (!ok || a >= p || b >= p) a = b = -1;
+            jacobi_pass<float, float, L, 4>(W, q, ldw, p, V, ldv, nrm, a, b, sl, tol, stop, rmax, rot);
+            __syncwarp();
+          }
+        }
+        if (okA && okB) {
+          const int a = A * C + sub;
+          int b = Bc * C + sub;
+          float2 xa[2 * U], xb[2 * U], va[2 * U], vb[2 * U];
+          load_rows<U, L>(W + (size_t)a * ldw, q, sl, a < p, xa);
+          load_rows<U, L>(W + (size_t)b * ldw, q, sl, b < p, xb);
+          load_rows<U, L>(V + (size_t)a * ldv, p, sl, a < p, va);
+          load_rows<U, L>(V + (size_t)b * ldv, p, sl, b < p, vb);
+          float na = a < p ? nrm[a] : 0.0f, nb = b < p ? nrm[b] : 0.0f;   // 0: no pair
+          int dirty = 0;
+#pragma unroll 1
+          for (int k = 0; k < C; ++k) {
+            float2 acc = {0.0f, 0.0f}, acc2 = {0.0f, 0.0f};
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              acc = fma2(xa[2 * u], xb[2 * u], acc);
+              acc2 = fma2(xa[2 * u + 1], xb[2 * u + 1], acc2);
+            }
+            float ga = (acc.x + acc2.x) + (acc.y + acc2.y);
+#pragma unroll
+            for (int o = L / 2; o > 0; o >>= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
+            // columns below kTiny32 are noise at binary32 resolution, and the
+            // fast reciprocal square root flushes subnormal inputs to 0
+            const float ratio = fabsf(ga) * (rsqrtf(fmaxf(na, kTiny32)) * rsqrtf(fmaxf(nb, kTiny32)));
+            const bool go = ga != 0.0f && na > kTiny32 && nb > kTiny32 && ratio > tol;
+            if (__any_sync(0xffffffffu, go)) {
+              float cs = 1.0f, sn = 0.0f;
+              if (go) {
+                rmax = fmaxf(rmax, ratio);
+                const float t = jacobi_tangent32(nb - na, ga);
+                cs = rsqrtf(1.0f + t * t);
+                sn = cs * t;
+                na -= t * ga;
+                nb += t * ga;
+              }
+              rotate_rows<U, L>(xa, xb, cs, sn, q);
+              rotate_rows<U, L>(va, vb, cs, sn, p);
+              dirty = 1;
+            }
+            if (k < C - 1) {
+              move_rows<U, L>(xb, q, next);
+              move_rows<U, L>(vb, p, next);
+              nb = lane_value(nb, next);
+            }
+          }
+          if (dirty) {
+            rot = 1;
+            b = Bc * C + ((sub + C - 1) & (C - 1));    // the column it holds after C - 1 moves
+            store_rows<U, L>(W + (size_t)a * ldw, q, sl, a < p, xa);
+            store_rows<U, L>(W + (size_t)b * ldw, q, sl, b < p, xb);
+            store_rows<U, L>(V + (size_t)a * ldv, p, sl, a < p, va);
+            store_rows<U, L>(V + (size_t)b * ldv, p, sl, b < p, vb);
+            if (sl == 0) {
+              if (a < p) nrm[a] = na;
+              if (b < p) nrm[b] = nb;
+            }
+          }
+          __syncwarp();
+        }
+      }
+      group_sync(bar, nthr);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
+    const int anyrot = __any_sync(0xffffffffu, rot);
+    if (lane == 0) {
+      if (anyrot) atomicMax(&gs.flag[g], 1);
+      atomicMax(&gs.rbits[g], __float_as_uint(rmax));
+    }
+    group_sync(bar, nthr);
+    const int any = gs.flag[g];
+    const float rm = __uint_as_float(gs.rbits[g]);
+    group_sync(bar, nthr);
+    if (!any || rm < stop) return sweep;
+  }
+  return -1;
+}
+
 // Lanes per pair from a latency model of one round: ceil(pairs / slots)
 // passes, each a fixed cost (reduction over log2 L lanes, the rotation
 // angle) plus the per-lane element work (about 3 q / L loads and FMAs).
@@ -973,8 +1221,11 @@ __device__ __forceinline__ int lanes_per_pair(int q, int p, int nw) {
   return best;
 }
 
-// One-sided Jacobi of one block by a warp group: the block ordering
-// (jacobi_blocks) for binary32 blocks of 16 columns or more, otherwise the
+constexpr int kRegsMin = 16;
+
+// One-sided Jacobi of one block by a warp group: the block ordering for
+// binary32 blocks of 16 columns or more (jacobi_regs up to 128 rows, where the
+// columns fit in registers, jacobi_blocks above), otherwise the
 // round-robin ordering with L lanes per pair from the latency model.
 // TV: element type of V.  A binary64 polish of a binary32 result may keep V
 // in binary32: V carries binary32 accuracy from the preconditioning sweeps
@@ -987,6 +1238,13 @@ template <typename T, typename TV = T, int B = 4>
 __device__ int jacobi_group(T* __restrict__ W, int q, int ldw, int p, TV* __restrict__ V, int ldv,
                             T* __restrict__ nrm, int lw, int nw, int bar, int g, GroupSh& gs, T stop, int max_sweeps) {
   if constexpr (sizeof(T) == sizeof(float)) {
+    const bool vec = ((ldw | ldv) & 3) == 0 && ((reinterpret_cast<uintptr_t>(W) | reinterpret_cast<uintptr_t>(V)) & 15) == 0;
+    if (p >= kRegsMin && vec) {
+      if (q <= 32) return jacobi_regs<1, 4>(W, q, ldw, p, V, ldv, nrm, lw, nw, bar, g, gs, stop, max_sweeps);
+      if (q <= 64) return jacobi_regs<2, 4>(W, q, ldw, p, V, ldv, nrm, lw, nw, bar, g, gs, stop, max_sweeps);
+      if (q <= 96) return jacobi_regs<3, 4>(W, q, ldw, p, V, ldv, nrm, lw, nw, bar, g, gs, stop, max_sweeps);
+      if (q <= 128) return jacobi_regs<4, 4>(W, q, ldw, p, V, ldv, nrm, lw, nw, bar, g, gs, stop, max_sweeps);
+    }
     if (p >= 16) return jacobi_blocks<T, TV, B>(W, q, ldw, p, V, ldv, nrm, lw, nw, bar, g, gs, stop, max_sweeps);
   }
   const int L = lanes_per_pair(q, p, nw);

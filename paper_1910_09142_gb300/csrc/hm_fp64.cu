@@ -405,11 +405,13 @@ constexpr int kPrecond = 12;
 constexpr double kStop64 = 1e-9;
 constexpr float kStopPre = 1e-3f;
 
-// Doubles of shared memory a block takes: W and V (odd leading dimensions), the
-// column norms.  The binary32 stage before it (W, V, norms) fits in W's part.
-__device__ __forceinline__ int64_t block_doubles(int q, int p) {
-  return (int64_t)p * max(q | 1, ((q | 1) + (p | 1) + 4) / 2) + (int64_t)p * (p | 1) + p;
+// Shared memory of a block, in doubles: W's part (W, leading dimension q | 1,
+// or the binary32 stage before it: W, V and their norms), V (leading dimension
+// p | 1), the column norms.
+__device__ __forceinline__ int w_doubles(int q, int p) {
+  return p * max(q | 1, (blk::ld4(q) + blk::ld4(p) + 2) / 2);
 }
+__device__ __forceinline__ int block_doubles(int q, int p) { return (w_doubles(q, p) + p * (p | 1) + p + 1) & ~1; }
 
 // Decomposition of one block by the nw warps of a group: A (q x p, global) to W
 // = A V with orthogonal columns and orthonormal V, both in shared memory.
@@ -430,33 +432,34 @@ __device__ int decompose_block(const double* A, int q, int p, double* base, floa
   const int lane = threadIdx.x & 31, nthr = 32 * nw;
   const int ldw = q | 1, ldv = p | 1;
   double* W = base;
-  double* V = base + (block_doubles(q, p) - (int64_t)p * ldv - p);
+  double* V = base + w_doubles(q, p);
   double* nrm = V + (size_t)p * ldv;
   int pre = 0;
   if (p >= kPrecond) {
+    const int lw4 = blk::ld4(q), lv4 = blk::ld4(p);
     float* W32 = reinterpret_cast<float*>(base);
-    float* V32 = W32 + (size_t)p * ldw;
-    float* n32 = V32 + (size_t)p * ldv;
+    float* V32 = W32 + (size_t)p * lw4;
+    float* n32 = V32 + (size_t)p * lv4;
     for (int j = lw; j < p; j += nw) {
-      for (int i = lane; i < q; i += 32) W32[(size_t)j * ldw + i] = blk::narrow(A[(size_t)j * q + i]);
-      for (int i = lane; i < p; i += 32) V32[(size_t)j * ldv + i] = i == j ? 1.0f : 0.0f;
+      for (int i = lane; i < q; i += 32) W32[(size_t)j * lw4 + i] = blk::narrow(A[(size_t)j * q + i]);
+      for (int i = lane; i < lv4; i += 32) V32[(size_t)j * lv4 + i] = i == j ? 1.0f : 0.0f;
     }
     blk::group_sync(bar, nthr);
-    pre = blk::jacobi_group<float>(W32, q, ldw, p, V32, ldv, n32, lw, nw, bar, g, gs, kStopPre, kMaxSweeps);
+    pre = blk::jacobi_group<float>(W32, q, lw4, p, V32, lv4, n32, lw, nw, bar, g, gs, kStopPre, kMaxSweeps);
     blk::group_sync(bar, nthr);
     if (pre > 0) {
       // V -> binary64, orthonormal
-      refine::unit_terms(V32, p, ldv, n32, KT, lw, nw);
+      refine::unit_terms(V32, p, lv4, n32, KT, lw, nw);
       blk::group_sync(bar, nthr);
-      refine::pair_terms<true>(V32, p, ldv, p, n32, n32, KT, lw, nw);
+      refine::pair_terms<true>(V32, p, lv4, p, n32, n32, KT, lw, nw);
       blk::group_sync(bar, nthr);
       int x = 0;
-      refine::add_product<false>(V32, p, ldv, p, KT, V, ldv, lw, nw, x);
+      refine::add_product<false>(V32, p, lv4, p, KT, V, ldv, lw, nw, x);
       blk::group_sync(bar, nthr);
       refine::ortho_terms64(V, p, ldv, KT, lw, nw);
       blk::group_sync(bar, nthr);
       x = 0;
-      refine::add_product<true>(V32, p, ldv, p, KT, V, ldv, lw, nw, x);
+      refine::add_product<true>(V32, p, lv4, p, KT, V, ldv, lw, nw, x);
       blk::group_sync(bar, nthr);
       refine::product64(A, q, p, V, ldv, W, ldw, lw, nw);
     }
@@ -543,7 +546,7 @@ __device__ void two_site_op_blocked(ChainDev* c, const OpDev op, int t, double* 
       const int sw = decompose_block(c->W + r.woff, q, p, W, reinterpret_cast<float*>(c->theta) + wv.koff[g], lw, nw,
                                      g + 1, g, sh.gs);
       if (lw == 0 && lane == 0) wv.sw[g] = sw;
-      const double* V = W + (block_doubles(q, p) - (int64_t)p * (p | 1) - p);
+      const double* V = W + w_doubles(q, p);
       for (int j = lw; j < p; j += nw) {
         for (int i = lane; i < q; i += 32) c->W[r.woff + (size_t)j * q + i] = W[(size_t)j * (q | 1) + i];
         for (int i = lane; i < p; i += 32) c->V[r.voff + (size_t)j * p + i] = V[(size_t)j * (p | 1) + i];

@@ -4,9 +4,10 @@
 // 1.2 TFLOP/s on 152 SMs), so this path forms the two-site tensor and applies
 // the 9x9 gate in binary32 and runs the one-sided Jacobi sweeps of every
 // charge block (Sec. II.C, hm_block.cuh) in binary32.  HM_MIXED then finishes
-// each block with one binary64 sweep (the singular values and left vectors
-// become binary64-accurate for that tensor); HM_MIXED32 stops at the binary32
-// sweeps.  The truncation weights (Sec. II), the renormalisation of the kept
+// each block so that the singular values and left vectors become
+// binary64-accurate for that tensor (hm_refine.cuh: one first-order sweep as a
+// product, binary64 rotations where that does not hold); HM_MIXED32 stops at
+// the binary32 sweeps.  The truncation weights (Sec. II), the renormalisation of the kept
 // singular values and the stored site tensors stay binary64.  Measurement
 // and collapse (steps 3-4) are the binary64 kernels of hm_fp64.cu.
 //
@@ -26,6 +27,7 @@
 
 #include "hm_block.cuh"
 #include "hm_internal.h"
+#include "hm_refine.cuh"
 
 namespace hm {
 
@@ -405,6 +407,61 @@ constexpr double kPolishStop = 1e-5;
 // kPolishStop, so one binary64 sweep still ends the polish.
 constexpr float kStop32 = 2e-4f, kStop32Polished = 1e-3f;
 
+// From a block's binary32 result (W32, V32 in shared memory, followed by
+// refine::extra floats) to its binary64 W and V (global memory), by the nw
+// warps of its group.  polish: the binary64-accurate finish of hm_refine.cuh;
+// otherwise only the unit-column scales.  K: scratch for the block's K.  Returns
+// the polish passes (1, or the binary64 sweeps it fell back on), -1 when
+// those did not converge.
+__device__ int refine_block(ChainDev* c, const blk::BlockRec& r, float* W32, float* V32, float* K,
+                            int polish, int lw, int nw, int bar, int g, blk::GroupSh& gs) {
+  const int q = r.q, p = r.p, ldw = blk::ld4(q), ldv = blk::ld4(p);
+  float* ah = V32 + (size_t)p * ldv;
+  float* al = ah + p;
+  float* dl = al + p;
+  double* W64 = c->W + r.woff;
+  double* V64 = c->V + r.voff;
+  const int nthr = 32 * nw;
+  blk::group_sync(bar, nthr);                 // the sweeps' last reads of the norms
+  refine::column_terms(W32, q, ldw, V32, p, ldv, ah, al, dl, polish ? K : nullptr, lw, nw);
+  if (lw == 0 && (threadIdx.x & 31) == 0) {
+    gs.flag[g] = 0;
+    gs.rbits[g] = 0u;
+  }
+  blk::group_sync(bar, nthr);
+  if (!polish) {
+    refine::scale_columns(W32, q, ldw, p, dl, W64, lw, nw);
+    refine::scale_columns(V32, p, ldv, p, dl, V64, lw, nw);
+    return 0;
+  }
+  float e = refine::pair_terms<false>(W32, q, ldw, p, ah, al, K, lw, nw);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) e = fmaxf(e, __shfl_xor_sync(0xffffffffu, e, o));
+  if ((threadIdx.x & 31) == 0) atomicMax(&gs.rbits[g], __float_as_uint(e));
+  blk::group_sync(bar, nthr);                 // K and its largest entry are complete
+  int x = 0;
+  refine::add_product<false>(W32, q, ldw, p, K, W64, q, lw, nw, x);
+  refine::add_product<false>(V32, p, ldv, p, K, V64, p, lw, nw, x);
+  blk::group_sync(bar, nthr);
+  if (lw == 0) {
+    const int found = refine::rotate_near(W64, q, V64, p, ah, 2 * p);
+    if ((threadIdx.x & 31) == 0)
+      gs.flag[g] = found > 2 * p || __uint_as_float(gs.rbits[g]) >= (float)kPolishStop ? 2 : (found > 0 ? 1 : 0);
+  }
+  blk::group_sync(bar, nthr);
+  const int more = gs.flag[g];
+  if (more == 0) return 1;
+  blk::group_sync(bar, nthr);                 // every warp has read the flag
+  int s64 = 1;
+  if (more == 2) {
+    s64 = blk::jacobi_group<double, double, 2>(W64, q, q, p, V64, p, c->sig + r.svoff, lw, nw, bar, g, gs, kPolishStop,
+                                               kMaxSweeps);
+    blk::group_sync(bar, nthr);
+  }
+  refine::unit_columns(W64, q, V64, p, lw, nw);
+  return s64;
+}
+
 // One two-site op (step 2 of Sec. I.C.1) in charge blocks (Sec. II.C):
 // theta and the gate in binary32 (operands rounded from the binary64 site
 // tensors, binary32 accumulation, gate coefficients as binary32 pairs); the
@@ -431,12 +488,15 @@ __device__ void two_site_op_mixed(ChainDev* c, const OpDev op, int t, int bcols,
       // as many consecutive blocks as fit in shared memory (at most 15 and
       // one warp each); a block that does not fit alone takes the global path
       int64_t used = 0;
-      int n = 0, p[15];
+      int n = 0, koff = 0, p[15];
       while (b0 + n < ss.nblk && n < 15 && n < NT / 32) {
         const blk::BlockRec& r = ss.b[b0 + n];
-        const int64_t need = (int64_t)r.p * (r.q | 1) + (int64_t)r.p * (r.p | 1) + r.p;
+        const int64_t need = (int64_t)r.p * blk::ld4(r.q) + (int64_t)r.p * blk::ld4(r.p) +
+                             blk::ld4(refine::extra(r.p));
         if (used + need > cap) break;
         wv.off[n] = (int32_t)used;
+        wv.koff[n] = koff;
+        koff += r.p * refine::ldk_of(r.p);
         p[n] = r.p;
         used += need;
         ++n;
@@ -481,45 +541,23 @@ __device__ void two_site_op_mixed(ChainDev* c, const OpDev op, int t, int bcols,
     for (int i = 0; i < n; ++i) {
       const blk::BlockRec& r = ss.b[b0 + i];
       float* W32 = smem + wv.off[i];
-      float* V32 = W32 + (size_t)r.p * (r.q | 1);
-      blk::gather_block<NT, float, float>(c, op.k, ss, r, theta, W32, r.q | 1, V32, r.p | 1, c0);
+      float* V32 = W32 + (size_t)r.p * blk::ld4(r.q);
+      blk::gather_block<NT, float, float>(c, op.k, ss, r, theta, W32, blk::ld4(r.q), V32, blk::ld4(r.p), c0);
     }
     __syncthreads();
     const int g = blk::my_group(wv, warp);
     if (g >= 0) {
       const blk::BlockRec& r = ss.b[b0 + g];
       float* W32 = smem + wv.off[g];
-      float* V32 = W32 + (size_t)r.p * (r.q | 1);
-      const int sw = blk::jacobi_group<float>(W32, r.q, r.q | 1, r.p, V32, r.p | 1, V32 + (size_t)r.p * (r.p | 1),
+      float* V32 = W32 + (size_t)r.p * blk::ld4(r.q);
+      const int sw = blk::jacobi_group<float>(W32, r.q, blk::ld4(r.q), r.p, V32, blk::ld4(r.p), V32 + (size_t)r.p * blk::ld4(r.p),
                                               warp - wv.w0[g], wv.nw[g], g + 1, g, gs,
                                               polish ? kStop32Polished : kStop32, kMaxSweeps);
-      if (warp == wv.w0[g] && (tid & 31) == 0) wv.sw[g] = sw;
+      const int s64 = sw < 0 ? 0 : refine_block(c, r, W32, V32, c->X + wv.koff[g], polish, warp - wv.w0[g], wv.nw[g],
+                                                g + 1, g, gs);
+      if (warp == wv.w0[g] && (tid & 31) == 0) wv.sw[g] = sw < 0 || s64 < 0 ? -1 : sw + 1000 * s64;
     }
     __syncthreads();
-    for (int i = 0; i < n; ++i) {
-      const blk::BlockRec& r = ss.b[b0 + i];
-      const float* W32 = smem + wv.off[i];
-      float* V32 = smem + wv.off[i] + (size_t)r.p * (r.q | 1);
-      promote_w(W32, r.q | 1, V32, r.p | 1, r.q, r.p, c->W + r.woff, c->sig + r.svoff);
-      __syncthreads();
-    }
-    if (polish && g >= 0) {
-      // binary64 polish by the same groups: W in binary64 (global), V stays
-      // in shared memory in binary32; norms of block g in c->sig
-      const blk::BlockRec& r = ss.b[b0 + g];
-      float* V32 = smem + wv.off[g] + (size_t)r.p * (r.q | 1);
-      const int s64 = blk::jacobi_group<double, float, 2>(c->W + r.woff, r.q, r.q, r.p, V32, r.p | 1, c->sig + r.svoff,
-                                                       warp - wv.w0[g], wv.nw[g], g + 1, g, gs, kPolishStop,
-                                                       kMaxSweeps);
-      if (warp == wv.w0[g] && (tid & 31) == 0) wv.sw[g] = wv.sw[g] < 0 ? -1 : (s64 < 0 ? -1 : wv.sw[g] + 1000 * s64);
-    }
-    __syncthreads();
-    for (int i = 0; i < n; ++i) {
-      const blk::BlockRec& r = ss.b[b0 + i];
-      const float* V32 = smem + wv.off[i] + (size_t)r.p * (r.q | 1);
-      promote_v(V32, r.p | 1, r.q, r.p, c->W + r.woff, c->V + r.voff, c->sig + r.svoff, polish);
-      __syncthreads();
-    }
     for (int i = 0; i < n; ++i) {
       const int code = wv.sw[i];
       if (code < 0) {

@@ -13,7 +13,9 @@
 // entries splits exactly into two binary32 numbers, and a sum against a
 // constant larger than every partial sum splits exactly too: dot2 below spends
 // seven binary32 instructions a term (64 x the rate of the binary64 pipe) and
-// returns the Gram entry to about 2^-45 of the columns' norms.
+// returns the Gram entry to about 2^-45 of the columns' norms.  Measured on Lx =
+// 16, 2W = 8, chi = 256 (256 chains, beta = 0.3): the evolution 1043 -> 800 ms,
+// sweep, promotion to binary64 and the scales together 37 -> about 15 % of it.
 //
 // Two columns of nearly the same norm have a large angle whatever their
 // overlap; their pairs (|b - a| < kNear max(a, b)) are left out of K and
@@ -114,8 +116,9 @@ __device__ __forceinline__ F2 warp_norm2(const float* x, int n) {
 // x' = x + (x delta + products with K): one column entry, binary64.
 __device__ __forceinline__ double corrected(float x, float corr) { return blk::widen(x) + blk::widen(corr); }
 
-// delta_j and the squared norms of the columns; KT: zeroed padding and the diagonal.
-__device__ inline void column_terms(const float* W, int q, int ldw, const float* V, int p, int ldv, float* ah, float* al,
+// delta_j and the squared norms of the columns; KT: zeroed padding and the
+// diagonal; W: zeroed rows up to a multiple of four.
+__device__ inline void column_terms(float* W, int q, int ldw, const float* V, int p, int ldv, float* ah, float* al,
                              float* dl, float* KT, int lw, int nw) {
   const int lane = threadIdx.x & 31;
   const int ldk = ldk_of(p);
@@ -131,6 +134,7 @@ __device__ inline void column_terms(const float* W, int q, int ldw, const float*
       if (KT) KT[(size_t)j * ldk + j] = d;
     }
     if (KT && lane >= 1 && p + lane - 1 < ldk) KT[(size_t)j * ldk + p + lane - 1] = 0.0f;
+    if (q + lane < ((q + 3) & ~3)) W[(size_t)j * ldw + q + lane] = 0.0f;   // pair_terms reads rows in fours
   }
 }
 
@@ -180,11 +184,17 @@ __device__ inline float pair_terms(const float* W, int q, int ldw, int p, const 
         d[r].start(big[r]);
       }
       const float* y = W + (size_t)jj * ldw;
-#pragma unroll 2
-      for (int k = 0; k < q; ++k) {
-        const float yk = y[k];
+      // rows in fours (128-bit loads; the rows from q on are zeros)
+      for (int k = 0; k < q; k += 4) {
+        const float4 yv = *reinterpret_cast<const float4*>(y + k);
 #pragma unroll
-        for (int r = 0; r < R; ++r) d[r].add(xi[r][k], yk);
+        for (int r = 0; r < R; ++r) {
+          const float4 xv = *reinterpret_cast<const float4*>(xi[r] + k);
+          d[r].add(xv.x, yv.x);
+          d[r].add(xv.y, yv.y);
+          d[r].add(xv.z, yv.z);
+          d[r].add(xv.w, yv.w);
+        }
       }
 #pragma unroll
       for (int r = 0; r < R; ++r) {
