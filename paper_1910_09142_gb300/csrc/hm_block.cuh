@@ -103,6 +103,22 @@ struct Seg {
   int32_t start, len;
 };
 
+// The CTAs that work on one chain together (a thread-block cluster), or one.
+struct Team {
+  int rank, size;
+};
+
+// Barrier of the team's threads; orders their accesses to global memory.
+__device__ __forceinline__ void team_sync(const Team& tm) {
+#if defined(__CUDA_ARCH__)
+  if (tm.size > 1) {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+    return;
+  }
+#endif
+  __syncthreads();
+}
+
 __device__ __forceinline__ Seg seg_of(const PrepTab& T, int bond, int qbase, int q) {
   const int i = q - qbase;
   if (i < 0 || i >= kWin) return {0, 0};   // callers stay within [qbase, qtop + 3]
@@ -188,7 +204,7 @@ __device__ void go_dense(ChainDev* c) {
 // One thread a candidate charge: a serial loop over them, each step a chain of
 // dependent loads, took as long as the blocks' arithmetic on small bonds.
 template <int NT>
-__device__ bool prepare(ChainDev* c, const OpDev& op, SplitSh& s, PrepTab& T) {
+__device__ bool prepare(ChainDev* c, const OpDev& op, SplitSh& s, PrepTab& T, const Team& tm) {
   const int tid = threadIdx.x;
   const int k = op.k;
   const int chil = c->chi[k], chim = c->chi[k + 1], chir = c->chi[k + 2];
@@ -241,9 +257,12 @@ __device__ bool prepare(ChainDev* c, const OpDev& op, SplitSh& s, PrepTab& T) {
   }
   __syncthreads();
   if (!s.ok) {
-    __syncthreads();
+    // every CTA of the team reads the same labels and comes here, or none does
+    team_sync(tm);
     if (c->counters[3]) return true;      // already dense: every charge is 0, cannot fail again
-    go_dense<NT>(c);
+    team_sync(tm);                        // every CTA has read the mark
+    if (tm.rank == 0) go_dense<NT>(c);
+    team_sync(tm);
     return false;
   }
   const int qb = s.qbase;
@@ -318,6 +337,7 @@ __device__ bool prepare(ChainDev* c, const OpDev& op, SplitSh& s, PrepTab& T) {
         int n_in, n_out, n_sv;
         const int at_in = lane_prefix(is_in ? 1 : 0, &n_in), at_out = lane_prefix(is_out ? 1 : 0, &n_out);
         if (pass == 1) {
+          // a team's CTAs write the same records
           InRec* ri = shared ? s.in_sh : M->in;
           BlockRec* ro = shared ? s.b_sh : M->b;
           const int p = mq < nq ? mq : nq, q = mq < nq ? nq : mq;
@@ -380,6 +400,20 @@ __device__ __forceinline__ void share(int n, int& c0, F&& f) {
   c0 += nch;
 }
 
+// The same over all CTAs of a team.
+template <int NT, typename F>
+__device__ __forceinline__ void share(const Team& tm, int n, int& c0, F&& f) {
+  const int lane = threadIdx.x & 31;
+  const unsigned nw = NT / 32 * tm.size;           // a power of two
+  const int warp = (threadIdx.x >> 5) + NT / 32 * tm.rank;
+  const int nch = (n + 31) >> 5;
+  for (int ch = (unsigned)(warp - c0) & (nw - 1); ch < nch; ch += nw) {
+    const int e = ch * 32 + lane;
+    if (e < n) f(e);
+  }
+  c0 += nch;
+}
+
 // Phase B: theta[(l s1), (s2 r)] = sum_m A_k[(l s1), m] A_{k+1}[m, (s2 r)] for
 // every entry whose row charge q(l) + sigma_k m(s1) and column charge
 // q(r) - sigma_{k+1} m(s2) agree (Sec. I.A two-site tensor), one GEMM per
@@ -400,19 +434,19 @@ __device__ __forceinline__ void share(int n, int& c0, F&& f) {
 constexpr double kThetaDirect = HM_THETA_DIRECT;
 
 template <int NT, typename T>
-__device__ void theta_direct(const ChainDev* c, int k, const SplitSh& s, T* __restrict__ theta) {
+__device__ void theta_direct(const ChainDev* c, int k, const SplitSh& s, T* __restrict__ theta, const Team& tm) {
   constexpr int R = 4;
   const int chim = c->chi[k + 1], chir = c->chi[k + 2];
   const int n = 3 * chir;
-  const double* __restrict__ A = c->site[k];
-  const double* __restrict__ B = c->site[k + 1];
+  const double* A = c->site[k];
+  const double* B = c->site[k + 1];
   int c0 = 0;
   for (int bi = 0; bi < s.nin; ++bi) {
     const InRec& r = s.in[bi];
     const int Mv = r.roff[3], Nv = r.coff[3], K = r.mlen, mst = r.mst;
     const int nu = (Nv + 31) >> 5;
     // one element a lane: (row group, column), columns padded to whole warps
-    share<NT>(((Mv + R - 1) / R) * nu * 32, c0, [&](int e) {
+    share<NT>(tm, ((Mv + R - 1) / R) * nu * 32, c0, [&](int e) {
       const int g = e / (nu * 32), u = e - g * nu * 32;
       const int uu = u < Nv ? u : Nv - 1;
       const int t2 = uu >= r.coff[2] ? 2 : (uu >= r.coff[1] ? 1 : 0);
@@ -443,28 +477,31 @@ __device__ void theta_direct(const ChainDev* c, int k, const SplitSh& s, T* __re
           if (x < nr) theta[(size_t)row[x] * n + col] = acc[x];
     });
   }
-  __syncthreads();
+  team_sync(tm);
 }
 
 template <int NT, int TM, int TN, int TK, typename T>
-__device__ void theta_blocks(const ChainDev* c, int k, const SplitSh& s, T* __restrict__ theta, T* smem) {
-  if (sizeof(T) == sizeof(double) || s.k1 <= kThetaDirect) return theta_direct<NT, T>(c, k, s, theta);
+__device__ void theta_blocks(const ChainDev* c, int k, const SplitSh& s, T* __restrict__ theta, T* smem,
+                             const Team& tm) {
+  if (sizeof(T) == sizeof(double) || s.k1 <= kThetaDirect) return theta_direct<NT, T>(c, k, s, theta, tm);
   const int tid = threadIdx.x;
   const int chim = c->chi[k + 1], chir = c->chi[k + 2];
   const int n = 3 * chir;
-  const double* __restrict__ A = c->site[k];
-  const double* __restrict__ B = c->site[k + 1];
+  const double* A = c->site[k];
+  const double* B = c->site[k + 1];
   // thread tile: rows ty + TY a (a < RA), columns tx + TX b (b < 4)
   constexpr int RB = 4, TX = TN / RB, TY = NT / TX, RA = TM / TY;
   static_assert(TN % RB == 0 && NT % TX == 0 && TM % TY == 0, "tile must split evenly over the CTA");
   const int tx = tid % TX, ty = tid / TX;
   T* sa = smem;                            // [TK][TM + 1]
   T* sb = smem + TK * (TM + 1);            // [TK][TN + 1]
+  int tile = 0;
   for (int bi = 0; bi < s.nin; ++bi) {
     const InRec& r = s.in[bi];
     const int Mv = r.roff[3], Nv = r.coff[3], K = r.mlen, mst = r.mst;
     for (int i0 = 0; i0 < Mv; i0 += TM) {
       for (int j0 = 0; j0 < Nv; j0 += TN) {
+        if (tile++ % tm.size != tm.rank) continue;        // tiles go round the team
         T acc[RA][RB];
 #pragma unroll
         for (int a = 0; a < RA; ++a)
@@ -525,7 +562,7 @@ __device__ void theta_blocks(const ChainDev* c, int k, const SplitSh& s, T* __re
       }
     }
   }
-  __syncthreads();
+  team_sync(tm);
 }
 
 // Phase C input: block r of theta after the gate (Sec. I.A: the gate acts on
@@ -539,8 +576,7 @@ __device__ void theta_blocks(const ChainDev* c, int k, const SplitSh& s, T* __re
 // on each of the up to three terms of an entry.
 template <int NT, typename TT, typename TW>
 __device__ void gather_block(const ChainDev* c, int k, const SplitSh& s, const BlockRec& r,
-                             const TT* __restrict__ theta, TW* __restrict__ W, int ldw, TW* __restrict__ V, int ldv,
-                             int& c0) {
+                             const TT* theta, TW* W, int ldw, TW* V, int ldv, int& c0) {
   const int chir = c->chi[k + 2];
   const int n = 3 * chir;
   const int nq = r.nq;
@@ -1205,28 +1241,14 @@ __device__ int jacobi_regs(float* __restrict__ W, int q, int ldw, int p, float* 
   return -1;
 }
 
-// Lanes per pair from a latency model of one round: ceil(pairs / slots)
-// passes, each a fixed cost (reduction over log2 L lanes, the rotation
-// angle) plus the per-lane element work (about 3 q / L loads and FMAs).
-__device__ __forceinline__ int lanes_per_pair(int q, int p, int nw) {
-  int best = 32;
-  long long bt = -1;
-  for (int L = 32; L >= 8; L >>= 1) {
-    const int slots = nw * (32 / L);
-    const int passes = ((p + 1) / 2 + slots - 1) / slots;
-    const int lg = L == 32 ? 5 : (L == 16 ? 4 : 3);
-    const long long tcost = (long long)passes * (150 + 25 * lg + 12 * ((q + L - 1) / L));
-    if (bt < 0 || tcost < bt) bt = tcost, best = L;
-  }
-  return best;
-}
-
 constexpr int kRegsMin = 16;
 
 // One-sided Jacobi of one block by a warp group: the block ordering for
 // binary32 blocks of 16 columns or more (jacobi_regs up to 128 rows, where the
 // columns fit in registers, jacobi_blocks above), otherwise the
-// round-robin ordering with L lanes per pair from the latency model.
+// round-robin ordering with 8 lanes a pair.  Neither depends on the number of
+// warps, nor does anything else a block goes through, so a chain's results are
+// the same bits whatever batch or team it runs in.
 // TV: element type of V.  A binary64 polish of a binary32 result may keep V
 // in binary32: V carries binary32 accuracy from the preconditioning sweeps
 // anyway, and the polish's rotations are tiny (angles ~1e-6).
@@ -1247,10 +1269,7 @@ __device__ int jacobi_group(T* __restrict__ W, int q, int ldw, int p, TV* __rest
     }
     if (p >= 16) return jacobi_blocks<T, TV, B>(W, q, ldw, p, V, ldv, nrm, lw, nw, bar, g, gs, stop, max_sweeps);
   }
-  const int L = lanes_per_pair(q, p, nw);
-  if (L == 8) return jacobi_lanes<T, TV, 8, B>(W, q, ldw, p, V, ldv, nrm, lw, nw, bar, g, gs, stop, max_sweeps);
-  if (L == 16) return jacobi_lanes<T, TV, 16, B>(W, q, ldw, p, V, ldv, nrm, lw, nw, bar, g, gs, stop, max_sweeps);
-  return jacobi_lanes<T, TV, 32, B>(W, q, ldw, p, V, ldv, nrm, lw, nw, bar, g, gs, stop, max_sweeps);
+  return jacobi_lanes<T, TV, 8, B>(W, q, ldw, p, V, ldv, nrm, lw, nw, bar, g, gs, stop, max_sweeps);
 }
 
 // Warp groups for one wave of charge blocks: every block gets at least one
@@ -1278,14 +1297,51 @@ __device__ inline void assign_warps(const int* p, int nblk, int nwarps, int* w0,
   for (int b = 0; b < nblk; ++b) w0[b] = w, w += nw[b];
 }
 
-// One wave of a split's charge blocks: blocks [b0, b0 + n) decomposed at
+// Blocks a team shares out one by one; a split with more stays with rank 0.
+constexpr int kTeamBlk = 64;
+
+// One wave of the blocks a CTA owns: its blocks [b0, b0 + n) decomposed at
 // once, block i by warps [w0[i], w0[i] + nw[i]) (barrier id i + 1).
 struct WaveSh {
+  int32_t nown;                           // blocks of this CTA
+  int32_t all;                            // it has them all (own unused)
+  int16_t own[kTeamBlk];
   int32_t b0, n;
   int32_t w0[15], nw[15], sw[15];
   int32_t off[15];                        // shared-memory offset (elements) of block i
-  int32_t koff[15];                       // scratch offset (elements) of block i (hm_refine.cuh)
 };
+
+__device__ __forceinline__ int own_block(const WaveSh& wv, int i) { return wv.all ? i : wv.own[i]; }
+
+// Shares the blocks of a split out over the team: the costliest block still
+// unassigned goes to the CTA with the least work (q p^2).  Every CTA computes
+// the same assignment.  One thread.  fits(q, p): the block can be decomposed
+// in shared memory; a split with one that cannot stays with rank 0, whose
+// scratch is then the whole buffer.
+template <typename F>
+__device__ inline void own_blocks(const SplitSh& s, const Team& tm, WaveSh& wv, F&& fits) {
+  bool alone = tm.size == 1 || s.nblk > kTeamBlk;
+  for (int b = 0; b < s.nblk && !alone; ++b) alone = !fits(s.b[b].q, s.b[b].p);
+  wv.all = alone;
+  wv.nown = alone && tm.rank == 0 ? s.nblk : 0;
+  if (alone) return;
+  int load[16];
+  for (int r = 0; r < tm.size; ++r) load[r] = 0;
+  unsigned long long done = 0;
+  for (int t = 0; t < s.nblk; ++t) {
+    int best = -1, bc = -1;
+    for (int b = 0; b < s.nblk; ++b) {
+      const int cost = (int)s.b[b].p * s.b[b].p + 64;     // a sweep is p rounds of p / 2 pairs
+      if (!((done >> b) & 1ull) && cost > bc) bc = cost, best = b;
+    }
+    done |= 1ull << best;
+    int to = 0;
+    for (int r = 1; r < tm.size; ++r)
+      if (load[r] < load[to]) to = r;
+    load[to] += bc;
+    if (to == tm.rank) wv.own[wv.nown++] = (int16_t)best;
+  }
+}
 
 // Index of this warp's group in the wave, or -1 (an idle warp).
 __device__ __forceinline__ int my_group(const WaveSh& wv, int warp) {
@@ -1392,8 +1448,8 @@ __device__ inline int warp_trunc_rank(const double* s, int n, int chi_max, doubl
 // goes block by block, after a plain zero fill, instead of looking up each
 // element's block.
 template <int NT>
-__device__ void finish(ChainDev* c, const OpDev& op, int t, SplitSh& s, char* __restrict__ scratch, double* tiles,
-                       int32_t* ctx_err, int sweeps32, int sweeps64) {
+__device__ void finish(ChainDev* c, const OpDev& op, int t, SplitSh& s, const WaveSh& wv, const Team& tm,
+                       char* __restrict__ scratch, double* tiles, int32_t* ctx_err, int sweeps32, int sweeps64) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int NW = NT / 32;
   const int k = op.k;
@@ -1408,26 +1464,28 @@ __device__ void finish(ChainDev* c, const OpDev& op, int t, SplitSh& s, char* __
   int32_t* perm = sblk + P;                           // slot of sorted value
   int32_t* key = perm + P;                            // kept value: block, rank
   int32_t* newslot = key + P;                         // slot of new index
-  // column norms -> raw values, slot = svoff + column
+  // column norms of this CTA's blocks -> raw values, slot = svoff + column
   {
     int c0 = 0;
-    for (int b = 0; b < nb; ++b) {
-      const BlockRec& r = s.b[b];
+    for (int i = 0; i < wv.nown; ++i) {
+      const BlockRec& r = s.b[own_block(wv, i)];
       const double* Wb = c->W + r.woff;
       for (int j = (unsigned)(warp - c0) % NW; j < r.p; j += NW) {
         const double* cj = Wb + (size_t)j * r.q;
         double s2 = 0.0;
 #pragma unroll 4
-        for (int i = lane; i < r.q; i += 32) s2 = fma(cj[i], cj[i], s2);
+        for (int e = lane; e < r.q; e += 32) s2 = fma(cj[e], cj[e], s2);
         s2 = warp_sum64(s2);
-        if (lane == 0) {
-          sraw[r.svoff + j] = sqrt(s2);
-          sblk[r.svoff + j] = b;
-        }
+        if (lane == 0) c->sig[r.svoff + j] = sqrt(s2);
       }
       c0 += r.p;
     }
   }
+  team_sync(tm);                          // every block's W, V and values are there
+  if (*(volatile int32_t*)c->status != 0) return;   // a decomposition failed (the same answer in every CTA)
+  for (int j = tid; j < P; j += NT) sraw[j] = c->sig[j];
+  for (int b = warp; b < nb; b += NW)
+    for (int j = lane; j < s.b[b].p; j += 32) sblk[s.b[b].svoff + j] = b;
   __syncthreads();
   // descending rank (ties by slot): sig[rank] = value, perm[rank] = slot
   for (int j = tid; j < P; j += NT) {
@@ -1464,7 +1522,7 @@ __device__ void finish(ChainDev* c, const OpDev& op, int t, SplitSh& s, char* __
     if (lane == 0) {
       s.kk = kk;
       s.nrm = nrm;
-      if (kk > 0) {
+      if (kk > 0 && tm.rank == 0) {
         double svd = 0.0;
         for (int b = 0; b < nb; ++b) svd += svd_count(s.b[b].mq, s.b[b].nq);
         c->stats[ST_K1] += 2.0 * s.k1;
@@ -1484,7 +1542,7 @@ __device__ void finish(ChainDev* c, const OpDev& op, int t, SplitSh& s, char* __
   const int kk = s.kk;
   const double nrm = s.nrm;
   if (kk <= 0) {
-    if (tid == 0) {
+    if (tid == 0 && tm.rank == 0) {
       if (atomicCAS(c->status, 0, HM_ERR_NUMERIC) == 0) *c->err_where = t;
       if (ctx_err) atomicCAS(ctx_err, 0, HM_ERR_NUMERIC);
     }
@@ -1501,10 +1559,10 @@ __device__ void finish(ChainDev* c, const OpDev& op, int t, SplitSh& s, char* __
     const int tot = h ? kk * n : m * kk;
     double2* A2 = reinterpret_cast<double2*>(A);
     const double2 z = {0.0, 0.0};
-    for (int e = tid; e < tot / 2; e += NT) A2[e] = z;
-    if ((tot & 1) && tid == 0) A[tot - 1] = 0.0;
+    for (int e = tid + NT * tm.rank; e < tot / 2; e += NT * tm.size) A2[e] = z;
+    if ((tot & 1) && tid == 0 && tm.rank == 0) A[tot - 1] = 0.0;
   }
-  __syncthreads();
+  team_sync(tm);
   const bool absorb_left = op.absorb == 0;
   int16_t* qM = c->qn + (size_t)(k + 1) * c->chi_cap;
   for (int i = tid; i < kk; i += NT) {
@@ -1514,7 +1572,7 @@ __device__ void finish(ChainDev* c, const OpDev& op, int t, SplitSh& s, char* __
     for (int j = 0; j < kk; ++j) pos += key[j] < ki;
     const int slot = perm[i], b = sblk[slot];
     newslot[pos] = slot;
-    qM[pos] = s.b[b].Q;
+    if (tm.rank == 0) qM[pos] = s.b[b].Q;
     const double sg = sraw[slot];
     // W column = U sigma (left) or V sigma (right, transposed block); V column a unit vector
     const bool w_left = !s.b[b].trans;
@@ -1538,7 +1596,7 @@ __device__ void finish(ChainDev* c, const OpDev& op, int t, SplitSh& s, char* __
     const int mq = r.mq, nq = r.nq, sv = r.svoff;
     // left factor A_k[(l a), i]: 32 rows x 8 kept values a warp, transposed in shared memory
     const int tv = (mq + 31) >> 5, ti = (kb + 7) >> 3;
-    for (int x = (unsigned)(warp - c0) % NW; x < tv * ti; x += NW) {
+    for (int x = (unsigned)(warp + NW * tm.rank - c0) & (NW * tm.size - 1); x < tv * ti; x += NW * tm.size) {
       const int v0 = (x % tv) * 32, j0 = (x / tv) * 8;
       const int nv = min(32, mq - v0), nj = min(8, kb - j0);
       __syncwarp();
@@ -1562,7 +1620,7 @@ __device__ void finish(ChainDev* c, const OpDev& op, int t, SplitSh& s, char* __
     }
     c0 += tv * ti;
     // right factor A_{k+1}[i, (b r)]
-    share<NT>(kb * nq, c0, [&](int e) {
+    share<NT>(tm, kb * nq, c0, [&](int e) {
       const int i = pos0 + e / nq, u = e % nq;
       const int bb = u >= r.coff[2] ? 2 : (u >= r.coff[1] ? 1 : 0);
       Ak1[(size_t)i * n + bb * chir + r.cst[bb] + u - r.coff[bb]] =
@@ -1570,8 +1628,9 @@ __device__ void finish(ChainDev* c, const OpDev& op, int t, SplitSh& s, char* __
     });
     pos0 += kb;
   }
-  __syncthreads();
-  if (tid == 0) {
+  // chi, the signs and qM are read by the split's records only: the barrier
+  // at the op's end orders them before the next op
+  if (tid == 0 && tm.rank == 0) {
     c->chi[k + 1] = kk;
     c->sgn[k] = s.osk;
     c->sgn[k + 1] = s.osk1;

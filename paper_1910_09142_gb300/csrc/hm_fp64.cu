@@ -25,6 +25,7 @@
 #include "hm_block.cuh"
 #include "hm_internal.h"
 #include "hm_refine.cuh"
+#include "hm_team.h"
 #include "hm_transfer.cuh"
 
 namespace hm {
@@ -484,35 +485,37 @@ __device__ int decompose_block(const double* A, int q, int p, double* base, floa
 // CTA and works on global memory.
 template <int NTE>
 __device__ void two_site_op_blocked(ChainDev* c, const OpDev op, int t, double* buf, size_t buf_bytes, EvolveSh& sh,
-                                    int32_t* ctx_err) {
+                                    const blk::Team& tm, int32_t* ctx_err) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   blk::SplitSh& ss = sh.split;
   blk::WaveSh& wv = sh.wave;
   blk::PrepTab& tab = *reinterpret_cast<blk::PrepTab*>(buf);
-  if (!blk::prepare<NTE>(c, op, ss, tab)) blk::prepare<NTE>(c, op, ss, tab);
-  blk::theta_direct<NTE, double>(c, op.k, ss, c->theta);
+  if (!blk::prepare<NTE>(c, op, ss, tab, tm)) blk::prepare<NTE>(c, op, ss, tab, tm);
+  blk::theta_direct<NTE, double>(c, op.k, ss, c->theta, tm);
+  const int64_t cap = (int64_t)(buf_bytes / sizeof(double));
+  if (tid == 0) blk::own_blocks(ss, tm, wv, [&](int q, int p) { return block_doubles(q, p) <= cap; });
+  __syncthreads();
+  const int nown = wv.nown;
   {
     int c0 = 0;
-    for (int b = 0; b < ss.nblk; ++b) {
-      const blk::BlockRec& r = ss.b[b];
+    for (int i = 0; i < nown; ++i) {
+      const blk::BlockRec& r = ss.b[blk::own_block(wv, i)];
       blk::gather_block<NTE, double, double>(c, op.k, ss, r, c->theta, c->W + r.woff, r.q, c->V + r.voff, r.p, c0);
     }
   }
   __syncthreads();
   int sweeps = 0;
   int64_t cost = -1;
-  const int64_t cap = (int64_t)(buf_bytes / sizeof(double));
-  for (int b0 = 0; b0 < ss.nblk;) {
+  bool failed = false;
+  for (int b0 = 0; b0 < nown && !failed;) {
     if (tid == 0) {
       int64_t used = 0;
-      int n = 0, koff = 0, p[15];
-      while (b0 + n < ss.nblk && n < 15 && n < NTE / 32) {
-        const blk::BlockRec& r = ss.b[b0 + n];
+      int n = 0, p[15];
+      while (b0 + n < nown && n < 15 && n < NTE / 32) {
+        const blk::BlockRec& r = ss.b[blk::own_block(wv, b0 + n)];
         const int64_t need = block_doubles(r.q, r.p);
         if (used + need > cap) break;
         wv.off[n] = (int32_t)used;
-        wv.koff[n] = koff;
-        koff += r.p * refine::ldk_of(r.p);
         p[n] = r.p;
         used += need;
         ++n;
@@ -524,12 +527,13 @@ __device__ void two_site_op_blocked(ChainDev* c, const OpDev op, int t, double* 
     __syncthreads();
     const int n = wv.n;
     if (n == 0) {
-      const blk::BlockRec& r = ss.b[b0];
+      const blk::BlockRec& r = ss.b[blk::own_block(wv, b0)];
       const int sw = blk::jacobi_group<double, double, 2>(c->W + r.woff, r.q, r.q, r.p, c->V + r.voff, r.p, c->sig, warp,
                                                           NTE / 32, 1, 0, sh.gs, kStop64, kMaxSweeps);
       if (sw < 0) {
         set_error(c, HM_ERR_NUMERIC, t, ctx_err);
-        return;
+        failed = true;
+        break;
       }
       const int64_t cb = (int64_t)r.q * r.p * r.p;   // sweeps of the costliest block
       if (cb > cost) cost = cb, sweeps = sw;
@@ -539,12 +543,14 @@ __device__ void two_site_op_blocked(ChainDev* c, const OpDev op, int t, double* 
     }
     const int g = blk::my_group(wv, warp);
     if (g >= 0) {
-      const blk::BlockRec& r = ss.b[b0 + g];
+      const int ib = blk::own_block(wv, b0 + g);
+      const blk::BlockRec& r = ss.b[ib];
       const int lw = warp - wv.w0[g], nw = wv.nw[g], q = r.q, p = r.p;
       double* W = buf + wv.off[g];
-      // theta is free once every block is gathered: its buffer holds the K's
-      const int sw = decompose_block(c->W + r.woff, q, p, W, reinterpret_cast<float*>(c->theta) + wv.koff[g], lw, nw,
-                                     g + 1, g, sh.gs);
+      // the transfer workspace is free during an evolution: it holds the K's
+      const int sw = decompose_block(c->W + r.woff, q, p, W,
+                                     reinterpret_cast<float*>(c->env_ws) + refine::k_offset(ss, ib), lw, nw, g + 1, g,
+                                     sh.gs);
       if (lw == 0 && lane == 0) wv.sw[g] = sw;
       const double* V = W + w_doubles(q, p);
       for (int j = lw; j < p; j += nw) {
@@ -556,49 +562,55 @@ __device__ void two_site_op_blocked(ChainDev* c, const OpDev op, int t, double* 
     for (int i = 0; i < n; ++i) {
       if (wv.sw[i] < 0) {
         set_error(c, HM_ERR_NUMERIC, t, ctx_err);
-        return;
+        failed = true;
+        break;
       }
-      const blk::BlockRec& r = ss.b[b0 + i];
+      const blk::BlockRec& r = ss.b[blk::own_block(wv, b0 + i)];
       const int64_t cb = (int64_t)r.q * r.p * r.p;
       if (cb > cost) cost = cb, sweeps = wv.sw[i];
     }
     b0 += n;
     __syncthreads();
   }
+  // a failed decomposition ends in finish(), behind the team's barrier
+  __syncthreads();
   constexpr int tiles = NTE / 32 * 8 * 33;
   char* scratch = reinterpret_cast<char*>(buf + tiles);
-  if (tiles * sizeof(double) + blk::finish_bytes(ss.P) > buf_bytes) scratch = reinterpret_cast<char*>(c->theta);
-  blk::finish<NTE>(c, op, t, ss, scratch, buf, ctx_err, sweeps, 0);
-  __syncthreads();
+  const size_t need = blk::finish_bytes(ss.P);
+  if (tiles * sizeof(double) + need > buf_bytes) scratch = reinterpret_cast<char*>(c->theta) + tm.rank * need;
+  blk::finish<NTE>(c, op, t, ss, wv, tm, scratch, buf, ctx_err, sweeps, 0);
 }
 
+// team: CTAs of a cluster that share one chain (1: no cluster).
 template <int NTE>
-__device__ void evolve_chain(const BatchArg& b, const OutArg& o, double* buf, size_t buf_bytes, EvolveSh& sh) {
-  ChainDev* c = b.c[blockIdx.x];
+__device__ void evolve_chain(const BatchArg& b, const OutArg& o, double* buf, size_t buf_bytes, EvolveSh& sh, int team) {
+  const blk::Team tm = {(int)blockIdx.x % team, team};
+  ChainDev* c = b.c[blockIdx.x / team];
   const OpDev* ops = b.ops_override ? b.ops_override : c->ops;
   const int n_ops = b.ops_override ? b.n_override : c->n_ops;
   const int t0 = b.budget > 0 ? c->counters[4] : b.t0;
   const int t1 = b.budget > 0 ? min(t0 + b.budget, n_ops) : (b.t1 < n_ops ? b.t1 : n_ops);
-  __syncthreads();                                           // every thread has read the cursor
-  if (b.budget > 0 && threadIdx.x == 0) c->counters[4] = t1;
+  blk::team_sync(tm);                                        // every thread has read the cursor
+  if (b.budget > 0 && threadIdx.x == 0 && tm.rank == 0) c->counters[4] = t1;
   for (int t = t0; t < t1; ++t) {
+    // the team agrees: a CTA sets the status only behind a barrier of the op
     if (*(volatile int32_t*)c->status != 0) return;
     __syncthreads();
-    two_site_op_blocked<NTE>(c, ops[t], t, buf, buf_bytes, sh, o.ctx_err);
-    __syncthreads();
+    two_site_op_blocked<NTE>(c, ops[t], t, buf, buf_bytes, sh, tm, o.ctx_err);
+    blk::team_sync(tm);
   }
 }
 
-__global__ void __launch_bounds__(kWideNT, 1) evolve_fp64_wide_kernel(BatchArg b, OutArg o) {
+__global__ void __launch_bounds__(kWideNT, 1) evolve_fp64_wide_kernel(BatchArg b, OutArg o, int team) {
   extern __shared__ double dsm[];
   __shared__ EvolveSh sh;
-  evolve_chain<kWideNT>(b, o, dsm, kWideSmem, sh);
+  evolve_chain<kWideNT>(b, o, dsm, kWideSmem, sh, team);
 }
 
 __global__ void __launch_bounds__(NT, 2) evolve_fp64_pair_kernel(BatchArg b, OutArg o) {
   extern __shared__ double dsm[];
   __shared__ EvolveSh sh;
-  evolve_chain<NT>(b, o, dsm, kPairSmem, sh);
+  evolve_chain<NT>(b, o, dsm, kPairSmem, sh, 1);
 }
 
 // Step 3 (Sec. I.C.1): <S_i.S_j> and <Sz_i Sz_j> on every measured bond.
@@ -1120,7 +1132,11 @@ int launch_evolve_fp64(const BatchArg& b, const OutArg& o, void* stream) {
   if (sms > 0 && b.n > sms) {
     evolve_fp64_pair_kernel<<<b.n, NT, kPairSmem, (cudaStream_t)stream>>>(b, o);
   } else {
-    evolve_fp64_wide_kernel<<<b.n, kWideNT, kWideSmem, (cudaStream_t)stream>>>(b, o);
+#if !defined(HM_HOST_EMULATION)
+    const int team = team_size((const void*)evolve_fp64_wide_kernel, kWideNT, kWideSmem, b.n);
+    if (team > 1) return launch_team(evolve_fp64_wide_kernel, b, o, team, kWideNT, kWideSmem, stream, team);
+#endif
+    evolve_fp64_wide_kernel<<<b.n, kWideNT, kWideSmem, (cudaStream_t)stream>>>(b, o, 1);
   }
   return check_launch();
 }

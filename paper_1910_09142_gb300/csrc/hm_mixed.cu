@@ -28,6 +28,7 @@
 #include "hm_block.cuh"
 #include "hm_internal.h"
 #include "hm_refine.cuh"
+#include "hm_team.h"
 
 namespace hm {
 
@@ -462,6 +463,11 @@ __device__ int refine_block(ChainDev* c, const blk::BlockRec& r, float* W32, flo
   return s64;
 }
 
+// Shared-memory floats of one block: W, V and the finish's terms.
+__device__ __forceinline__ int64_t block_floats(int q, int p) {
+  return (int64_t)p * blk::ld4(q) + (int64_t)p * blk::ld4(p) + blk::ld4(refine::extra(p));
+}
+
 // One two-site op (step 2 of Sec. I.C.1) in charge blocks (Sec. II.C):
 // theta and the gate in binary32 (operands rounded from the binary64 site
 // tensors, binary32 accumulation, gate coefficients as binary32 pairs); the
@@ -474,29 +480,31 @@ __device__ int refine_block(ChainDev* c, const blk::BlockRec& r, float* W32, flo
 // global memory.  Then the truncation rule (Sec. II), renormalisation and
 // absorb in binary64.
 __device__ void two_site_op_mixed(ChainDev* c, const OpDev op, int t, int bcols, int polish, float* smem, Scal& sc,
-                                  blk::SplitSh& ss, blk::WaveSh& wv, blk::GroupSh& gs, int32_t* ctx_err) {
+                                  blk::SplitSh& ss, blk::WaveSh& wv, blk::GroupSh& gs, const blk::Team& tm,
+                                  int32_t* ctx_err) {
   const int tid = threadIdx.x, warp = tid >> 5;
   blk::PrepTab& tab = *reinterpret_cast<blk::PrepTab*>(smem);
-  if (!blk::prepare<NT>(c, op, ss, tab)) blk::prepare<NT>(c, op, ss, tab);
+  if (!blk::prepare<NT>(c, op, ss, tab, tm)) blk::prepare<NT>(c, op, ss, tab, tm);
   float* theta = reinterpret_cast<float*>(c->theta);
-  blk::theta_blocks<NT, GM, GN, GK, float>(c, op.k, ss, theta, smem);
+  blk::theta_blocks<NT, GM, GN, GK, float>(c, op.k, ss, theta, smem, tm);
   int sw32 = 0, sw64 = 0;
   int64_t cost = -1;
   constexpr int64_t cap = (int64_t)(kBlockSmem / sizeof(float));
-  for (int b0 = 0; b0 < ss.nblk;) {
+  if (tid == 0) blk::own_blocks(ss, tm, wv, [&](int q, int p) { return block_floats(q, p) <= cap; });
+  __syncthreads();
+  const int nown = wv.nown;
+  bool failed = false;
+  for (int b0 = 0; b0 < nown && !failed;) {
     if (tid == 0) {
-      // as many consecutive blocks as fit in shared memory (at most 15 and
+      // as many of the CTA's blocks as fit in shared memory (at most 15 and
       // one warp each); a block that does not fit alone takes the global path
       int64_t used = 0;
-      int n = 0, koff = 0, p[15];
-      while (b0 + n < ss.nblk && n < 15 && n < NT / 32) {
-        const blk::BlockRec& r = ss.b[b0 + n];
-        const int64_t need = (int64_t)r.p * blk::ld4(r.q) + (int64_t)r.p * blk::ld4(r.p) +
-                             blk::ld4(refine::extra(r.p));
+      int n = 0, p[15];
+      while (b0 + n < nown && n < 15 && n < NT / 32) {
+        const blk::BlockRec& r = ss.b[blk::own_block(wv, b0 + n)];
+        const int64_t need = block_floats(r.q, r.p);
         if (used + need > cap) break;
         wv.off[n] = (int32_t)used;
-        wv.koff[n] = koff;
-        koff += r.p * refine::ldk_of(r.p);
         p[n] = r.p;
         used += need;
         ++n;
@@ -508,7 +516,7 @@ __device__ void two_site_op_mixed(ChainDev* c, const OpDev op, int t, int bcols,
     __syncthreads();
     const int n = wv.n;
     if (n == 0) {
-      const blk::BlockRec& r = ss.b[b0];
+      const blk::BlockRec& r = ss.b[blk::own_block(wv, b0)];
       float* W32 = c->X;
       float* V32 = c->X + (size_t)r.q * r.p;
       int c0 = 0;
@@ -517,7 +525,8 @@ __device__ void two_site_op_mixed(ChainDev* c, const OpDev op, int t, int bcols,
       const int sw = cta_jacobi_f32(W32, r.q, r.p, V32, bcols, smem, sc, nullptr);
       if (sw < 0) {
         set_error(c, HM_ERR_NUMERIC, t, ctx_err);
-        return;
+        failed = true;
+        break;
       }
       double* W64 = c->W + r.woff;
       double* V64 = c->V + r.voff;
@@ -530,7 +539,8 @@ __device__ void two_site_op_mixed(ChainDev* c, const OpDev op, int t, int bcols,
       promote_v(V32, r.p, r.q, r.p, W64, V64, c->sig, polish);
       if (s64 < 0) {
         set_error(c, HM_ERR_NUMERIC, t, ctx_err);
-        return;
+        failed = true;
+        break;
       }
       const int64_t cb = (int64_t)r.q * r.p * r.p;
       if (cb > cost) cost = cb, sw32 = sw, sw64 = s64;
@@ -539,7 +549,7 @@ __device__ void two_site_op_mixed(ChainDev* c, const OpDev op, int t, int bcols,
     }
     int c0 = 0;
     for (int i = 0; i < n; ++i) {
-      const blk::BlockRec& r = ss.b[b0 + i];
+      const blk::BlockRec& r = ss.b[blk::own_block(wv, b0 + i)];
       float* W32 = smem + wv.off[i];
       float* V32 = W32 + (size_t)r.p * blk::ld4(r.q);
       blk::gather_block<NT, float, float>(c, op.k, ss, r, theta, W32, blk::ld4(r.q), V32, blk::ld4(r.p), c0);
@@ -547,13 +557,14 @@ __device__ void two_site_op_mixed(ChainDev* c, const OpDev op, int t, int bcols,
     __syncthreads();
     const int g = blk::my_group(wv, warp);
     if (g >= 0) {
-      const blk::BlockRec& r = ss.b[b0 + g];
+      const int ib = blk::own_block(wv, b0 + g);
+      const blk::BlockRec& r = ss.b[ib];
       float* W32 = smem + wv.off[g];
       float* V32 = W32 + (size_t)r.p * blk::ld4(r.q);
       const int sw = blk::jacobi_group<float>(W32, r.q, blk::ld4(r.q), r.p, V32, blk::ld4(r.p), V32 + (size_t)r.p * blk::ld4(r.p),
                                               warp - wv.w0[g], wv.nw[g], g + 1, g, gs,
                                               polish ? kStop32Polished : kStop32, kMaxSweeps);
-      const int s64 = sw < 0 ? 0 : refine_block(c, r, W32, V32, c->X + wv.koff[g], polish, warp - wv.w0[g], wv.nw[g],
+      const int s64 = sw < 0 ? 0 : refine_block(c, r, W32, V32, c->X + refine::k_offset(ss, ib), polish, warp - wv.w0[g], wv.nw[g],
                                                 g + 1, g, gs);
       if (warp == wv.w0[g] && (tid & 31) == 0) wv.sw[g] = sw < 0 || s64 < 0 ? -1 : sw + 1000 * s64;
     }
@@ -562,40 +573,47 @@ __device__ void two_site_op_mixed(ChainDev* c, const OpDev op, int t, int bcols,
       const int code = wv.sw[i];
       if (code < 0) {
         set_error(c, HM_ERR_NUMERIC, t, ctx_err);
-        return;
+        failed = true;
+        break;
       }
-      const blk::BlockRec& r = ss.b[b0 + i];
+      const blk::BlockRec& r = ss.b[blk::own_block(wv, b0 + i)];
       const int64_t cb = (int64_t)r.q * r.p * r.p;
       if (cb > cost) cost = cb, sw32 = code % 1000, sw64 = code / 1000;
     }
     b0 += n;
     __syncthreads();
   }
+  // a failed decomposition ends in finish(), behind the team's barrier
+  __syncthreads();
   double* tiles = reinterpret_cast<double*>(smem);
   char* scratch = reinterpret_cast<char*>(tiles + kTileDoubles);
-  if (kTileDoubles * sizeof(double) + blk::finish_bytes(ss.P) > kBlockSmem) scratch = reinterpret_cast<char*>(c->theta);
-  blk::finish<NT>(c, op, t, ss, scratch, tiles, ctx_err, sw32, sw64);
-  __syncthreads();
+  const size_t need = blk::finish_bytes(ss.P);
+  if (kTileDoubles * sizeof(double) + need > kBlockSmem) scratch = reinterpret_cast<char*>(c->theta) + tm.rank * need;
+  blk::finish<NT>(c, op, t, ss, wv, tm, scratch, tiles, ctx_err, sw32, sw64);
 }
 
-__global__ void __launch_bounds__(NT, kCtasPerSm) evolve_mixed_kernel(BatchArg b, OutArg o, int bcols, int polish) {
+// team: CTAs of a cluster that share one chain (1: no cluster).
+__global__ void __launch_bounds__(NT, kCtasPerSm) evolve_mixed_kernel(BatchArg b, OutArg o, int bcols, int polish,
+                                                                      int team) {
   extern __shared__ float smem[];
   __shared__ Scal sc;
   __shared__ blk::SplitSh ss;
   __shared__ blk::WaveSh wv;
   __shared__ blk::GroupSh gs;
-  ChainDev* c = b.c[blockIdx.x];
+  const blk::Team tm = {(int)blockIdx.x % team, team};
+  ChainDev* c = b.c[blockIdx.x / team];
   const OpDev* ops = b.ops_override ? b.ops_override : c->ops;
   const int n_ops = b.ops_override ? b.n_override : c->n_ops;
   const int t0 = b.budget > 0 ? c->counters[4] : b.t0;
   const int t1 = b.budget > 0 ? min(t0 + b.budget, n_ops) : (b.t1 < n_ops ? b.t1 : n_ops);
-  __syncthreads();                                           // every thread has read the cursor
-  if (b.budget > 0 && threadIdx.x == 0) c->counters[4] = t1;
+  blk::team_sync(tm);                                        // every thread has read the cursor
+  if (b.budget > 0 && threadIdx.x == 0 && tm.rank == 0) c->counters[4] = t1;
   for (int t = t0; t < t1; ++t) {
+    // the team agrees: a CTA sets the status only behind a barrier of the op
     if (*(volatile int32_t*)c->status != 0) return;
     __syncthreads();
-    two_site_op_mixed(c, ops[t], t, bcols, polish, smem, sc, ss, wv, gs, o.ctx_err);
-    __syncthreads();
+    two_site_op_mixed(c, ops[t], t, bcols, polish, smem, sc, ss, wv, gs, tm, o.ctx_err);
+    blk::team_sync(tm);
   }
 }
 
@@ -618,7 +636,11 @@ int launch_kernel(const BatchArg& b, const OutArg& o, int chi_cap, int polish, v
       if (dev >= 0 && dev < 64) configured[dev] = smem;
     }
   }
-  evolve_mixed_kernel<<<b.n, NT, smem, (cudaStream_t)stream>>>(b, o, bcols, polish);
+#if HM_MIXED_CTAS_PER_SM == 1 && !defined(HM_HOST_EMULATION)
+  const int team = team_size((const void*)evolve_mixed_kernel, NT, smem, b.n);
+  if (team > 1) return launch_team(evolve_mixed_kernel, b, o, team, NT, smem, stream, bcols, polish, team);
+#endif
+  evolve_mixed_kernel<<<b.n, NT, smem, (cudaStream_t)stream>>>(b, o, bcols, polish, 1);
   return cudaGetLastError() == cudaSuccess ? HM_OK : HM_ERR_CUDA;
 }
 

@@ -93,6 +93,13 @@ __device__ __forceinline__ int extra(int p) { return 3 * p; }
 // Leading dimension of K's transpose (four entries are loaded at once).
 __device__ __forceinline__ int ldk_of(int p) { return (p + 3) & ~3; }
 
+// Offset (floats, a multiple of 4) of block b's K in the chain's scratch.
+__device__ __forceinline__ int k_offset(const blk::SplitSh& s, int b) {
+  int k = 0;
+  for (int i = 0; i < b; ++i) k += s.b[i].p * ldk_of(s.b[i].p);
+  return k;
+}
+
 __device__ __forceinline__ bool near_pair(float a, float b) { return fabsf(b - a) < kNear * fmaxf(a, b); }
 
 // Squared norm of one column by a warp.
@@ -324,7 +331,7 @@ __device__ inline void ortho_terms64(const double* V, int p, int ldv, float* KT,
 // out = A V: A q x p binary64 column-major (leading dimension q, global), V p x
 // p (shared, leading dimension ldv), out leading dimension ldo.  32 rows x 4
 // columns a warp.
-__device__ inline void product64(const double* __restrict__ A, int q, int p, const double* V, int ldv, double* out,
+__device__ inline void product64(const double* A, int q, int p, const double* V, int ldv, double* out,
                                  int ldo, int lw, int nw) {
   const int lane = threadIdx.x & 31;
   int x = 0;

@@ -1,0 +1,87 @@
+// Host side of a team: the thread-block cluster that works on one chain
+// when a batch has fewer chains than the GPU has SMs.
+//
+// A chain's ops are serial, but the charge blocks of one split are not: a team
+// shares out theta's tiles, the blocks (each decomposed by one CTA, the
+// costliest first), the zero fill and the absorb, and meets at four cluster
+// barriers an op.  Everything a CTA needs from another goes through the chain's
+// own buffers in global memory.  A Markov step, one CTA -> a team: 4 chains of Lx = 4, 2W =
+// 4, binary64, 206 -> 113 ms (8 CTAs); 8 mixed chains of Lx = 4, 30.4 -> 22.4
+// ms (8); one METTS chain of small blocks, 22.1 -> 20.4 ms (8).
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include <mutex>
+
+#include "hm_internal.h"
+
+namespace hm {
+
+#if !defined(HM_HOST_EMULATION)
+// Largest cluster size of 8, 4 or 2 for which n clusters of `kernel` are
+// resident at once, else 1.  The occupancy answers are kept per device and
+// kernel (at most four kernels).
+inline int team_size(const void* kernel, int threads, size_t smem, int n) {
+  struct Known {
+    const void* kernel;
+    int dev, most[4];                       // clusters of 2, 4 and 8 that fit
+  };
+  static std::mutex mu;
+  static Known known[16] = {};
+  static int n_known = 0;
+  if (2 * n > device_sm_count()) return 1;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+  std::lock_guard<std::mutex> lock(mu);
+  Known* k = nullptr;
+  for (int i = 0; i < n_known; ++i)
+    if (known[i].kernel == kernel && known[i].dev == dev) k = &known[i];
+  Known own = {kernel, dev, {0, 0, 0, 0}};
+  if (!k) {
+    for (int e = 1; e <= 3; ++e) {
+      cudaLaunchAttribute at = {};
+      at.id = cudaLaunchAttributeClusterDimension;
+      at.val.clusterDim.x = 1u << e;
+      at.val.clusterDim.y = at.val.clusterDim.z = 1;
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(1u << e);
+      cfg.blockDim = dim3(threads);
+      cfg.dynamicSmemBytes = smem;
+      cfg.attrs = &at;
+      cfg.numAttrs = 1;
+      if (cudaOccupancyMaxActiveClusters(&own.most[e], kernel, &cfg) != cudaSuccess) {
+        own.most[e] = 0;
+        cudaGetLastError();                 // an unsupported size is not an error of the launch
+      }
+    }
+    k = &own;
+    if (n_known < 16) {
+      known[n_known] = own;
+      k = &known[n_known++];
+    }
+  }
+  for (int e = 3; e >= 1; --e)
+    if (k->most[e] >= n) return 1 << e;
+  return 1;
+}
+
+template <typename... P, typename... A>
+int launch_team(void (*kernel)(BatchArg, OutArg, P...), const BatchArg& b, const OutArg& o, int team, int threads,
+                size_t smem, void* stream, A... more) {
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = team;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)b.n * team);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = (cudaStream_t)stream;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, b, o, P(more)...) == cudaSuccess ? HM_OK : HM_ERR_CUDA;
+}
+#endif
+
+}  // namespace hm
