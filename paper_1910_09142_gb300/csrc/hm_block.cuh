@@ -1272,42 +1272,72 @@ __device__ int jacobi_group(T* __restrict__ W, int q, int ldw, int p, TV* __rest
   return jacobi_lanes<T, TV, 8, B>(W, q, ldw, p, V, ldv, nrm, lw, nw, bar, g, gs, stop, max_sweeps);
 }
 
-// Warp groups for one wave of charge blocks: every block gets at least one
-// warp, then warps go one at a time to the block whose sweep takes longest
-// ((p - 1) rounds of ceil(p / (2 w)) pairs per warp), never beyond p / 2.
-// nblk <= 15 and nblk <= nwarps.  Writes the first warp and the warp count
-// of every block.  One thread.
-__device__ inline void assign_warps(const int* p, int nblk, int nwarps, int* w0, int* nw) {
-  int used = 0;
-  for (int b = 0; b < nblk; ++b) nw[b] = 1, ++used;
-  while (used < nwarps) {
-    int best = -1;
-    long long bt = -1;
-    for (int b = 0; b < nblk; ++b) {
-      const int cap = (p[b] + 1) / 2;
-      if (nw[b] >= cap) continue;
-      const long long t = (long long)(p[b] - 1) * ((p[b] + 2 * nw[b] - 1) / (2 * nw[b]));
-      if (t > bt) bt = t, best = b;
+// Work of one block's sweeps, in units that only matter relative to each
+// other: p^2 / 2 pairs, each a fixed part (reduction, angle) and its rows.
+__device__ __forceinline__ int block_cost(int q, int p) { return p * p * (q + 48) / 8 + 256 * p; }
+
+// Warp groups for one wave of nblk <= 15 blocks (costs `cost`, columns p).
+// With warps for all super-pairs of all blocks (a sub-round handles eight
+// columns), every block has a group of its own.  Otherwise a block that is
+// worth a warp or more does, and smaller ones are put together, one after
+// another, until they are worth one: with one warp at least for every block,
+// a split of eight blocks on eight warps took 2.6 times as long as its work
+// (Lx = 16, chi = 256, 256 chains: 808 -> 750 ms a step; but 16 chains of Lx = 5,
+// where the warps are plenty, 77 -> 84 ms, hence the first case).  Then the
+// warps go one at a time to the group that takes longest, at most p / 2 to
+// one.  Writes every block's group and every group's first warp and warp
+// count; returns the groups.  One thread.
+__device__ inline int assign_warps(const int* p, const int* cost, int nblk, int nwarps, int32_t* grp, int32_t* w0,
+                                   int32_t* nw) {
+  int total = 0, pairs = 0;
+  for (int b = 0; b < nblk; ++b) total += cost[b] >> 4, pairs += (p[b] + 7) / 8;
+  const bool plenty = pairs <= nwarps;
+  const int share = total / nwarps + 1;
+  int load[15], cap[15], ng = 0, open = -1;
+  for (int b = 0; b < nblk; ++b) {
+    const bool own = plenty || ((cost[b] >> 4) >= share && ng < nwarps);
+    int g = own ? -1 : open;
+    if (g < 0) {
+      // at most nwarps groups: past that, blocks join the lightest one
+      if (ng < nwarps) {
+        g = ng++;
+        load[g] = 0;
+        cap[g] = 1;
+        nw[g] = 1;
+      } else {
+        g = 0;
+        for (int i = 1; i < ng; ++i)
+          if (load[i] < load[g]) g = i;
+      }
     }
+    grp[b] = g;
+    load[g] += cost[b] >> 4;
+    cap[g] = max(cap[g], (p[b] + 1) / 2);
+    if (!own) open = load[g] >= share ? -1 : g;
+  }
+  for (int used = ng; used < nwarps; ++used) {
+    int best = -1, bt = -1;
+    for (int g = 0; g < ng; ++g)
+      if (nw[g] < cap[g] && load[g] / nw[g] > bt) bt = load[g] / nw[g], best = g;
     if (best < 0) break;
     ++nw[best];
-    ++used;
   }
-  int w = 0;
-  for (int b = 0; b < nblk; ++b) w0[b] = w, w += nw[b];
+  for (int g = 0, w = 0; g < ng; ++g) w0[g] = w, w += nw[g];
+  return ng;
 }
 
 // Blocks a team shares out one by one; a split with more stays with rank 0.
 constexpr int kTeamBlk = 64;
 
 // One wave of the blocks a CTA owns: its blocks [b0, b0 + n) decomposed at
-// once, block i by warps [w0[i], w0[i] + nw[i]) (barrier id i + 1).
+// once, group g (barrier id g + 1) taking those with grp[i] = g in turn on its
+// warps [w0[g], w0[g] + nw[g]).
 struct WaveSh {
   int32_t nown;                           // blocks of this CTA
   int32_t all;                            // it has them all (own unused)
   int16_t own[kTeamBlk];
-  int32_t b0, n;
-  int32_t w0[15], nw[15], sw[15];
+  int32_t b0, n, ng;
+  int32_t grp[15], w0[15], nw[15], sw[15];
   int32_t off[15];                        // shared-memory offset (elements) of block i
 };
 
@@ -1331,7 +1361,7 @@ __device__ inline void own_blocks(const SplitSh& s, const Team& tm, WaveSh& wv, 
   for (int t = 0; t < s.nblk; ++t) {
     int best = -1, bc = -1;
     for (int b = 0; b < s.nblk; ++b) {
-      const int cost = (int)s.b[b].p * s.b[b].p + 64;     // a sweep is p rounds of p / 2 pairs
+      const int cost = block_cost(s.b[b].q, s.b[b].p);
       if (!((done >> b) & 1ull) && cost > bc) bc = cost, best = b;
     }
     done |= 1ull << best;
@@ -1345,7 +1375,7 @@ __device__ inline void own_blocks(const SplitSh& s, const Team& tm, WaveSh& wv, 
 
 // Index of this warp's group in the wave, or -1 (an idle warp).
 __device__ __forceinline__ int my_group(const WaveSh& wv, int warp) {
-  for (int i = 0; i < wv.n; ++i)
+  for (int i = 0; i < wv.ng; ++i)
     if (warp >= wv.w0[i] && warp < wv.w0[i] + wv.nw[i]) return i;
   return -1;
 }

@@ -510,19 +510,20 @@ __device__ void two_site_op_blocked(ChainDev* c, const OpDev op, int t, double* 
   for (int b0 = 0; b0 < nown && !failed;) {
     if (tid == 0) {
       int64_t used = 0;
-      int n = 0, p[15];
+      int n = 0, p[15], cost[15];
       while (b0 + n < nown && n < 15 && n < NTE / 32) {
         const blk::BlockRec& r = ss.b[blk::own_block(wv, b0 + n)];
         const int64_t need = block_doubles(r.q, r.p);
         if (used + need > cap) break;
         wv.off[n] = (int32_t)used;
         p[n] = r.p;
+        cost[n] = blk::block_cost(r.q, r.p);
         used += need;
         ++n;
       }
       wv.b0 = b0;
       wv.n = n;
-      if (n > 0) blk::assign_warps(p, n, NTE / 32, wv.w0, wv.nw);
+      wv.ng = n > 0 ? blk::assign_warps(p, cost, n, NTE / 32, wv.grp, wv.w0, wv.nw) : 0;
     }
     __syncthreads();
     const int n = wv.n;
@@ -542,20 +543,22 @@ __device__ void two_site_op_blocked(ChainDev* c, const OpDev op, int t, double* 
       continue;
     }
     const int g = blk::my_group(wv, warp);
-    if (g >= 0) {
-      const int ib = blk::own_block(wv, b0 + g);
+    for (int i = 0; g >= 0 && i < n; ++i) {
+      if (wv.grp[i] != g) continue;
+      const int ib = blk::own_block(wv, b0 + i);
       const blk::BlockRec& r = ss.b[ib];
       const int lw = warp - wv.w0[g], nw = wv.nw[g], q = r.q, p = r.p;
-      double* W = buf + wv.off[g];
+      double* W = buf + wv.off[i];
       // the transfer workspace is free during an evolution: it holds the K's
       const int sw = decompose_block(c->W + r.woff, q, p, W,
                                      reinterpret_cast<float*>(c->env_ws) + refine::k_offset(ss, ib), lw, nw, g + 1, g,
                                      sh.gs);
-      if (lw == 0 && lane == 0) wv.sw[g] = sw;
+      if (lw == 0 && lane == 0) wv.sw[i] = sw;
+      blk::group_sync(g + 1, 32 * nw);          // every warp's last rotations; the flags are free again
       const double* V = W + w_doubles(q, p);
       for (int j = lw; j < p; j += nw) {
-        for (int i = lane; i < q; i += 32) c->W[r.woff + (size_t)j * q + i] = W[(size_t)j * (q | 1) + i];
-        for (int i = lane; i < p; i += 32) c->V[r.voff + (size_t)j * p + i] = V[(size_t)j * (p | 1) + i];
+        for (int e = lane; e < q; e += 32) c->W[r.woff + (size_t)j * q + e] = W[(size_t)j * (q | 1) + e];
+        for (int e = lane; e < p; e += 32) c->V[r.voff + (size_t)j * p + e] = V[(size_t)j * (p | 1) + e];
       }
     }
     __syncthreads();

@@ -499,19 +499,20 @@ __device__ void two_site_op_mixed(ChainDev* c, const OpDev op, int t, int bcols,
       // as many of the CTA's blocks as fit in shared memory (at most 15 and
       // one warp each); a block that does not fit alone takes the global path
       int64_t used = 0;
-      int n = 0, p[15];
+      int n = 0, p[15], cost[15];
       while (b0 + n < nown && n < 15 && n < NT / 32) {
         const blk::BlockRec& r = ss.b[blk::own_block(wv, b0 + n)];
         const int64_t need = block_floats(r.q, r.p);
         if (used + need > cap) break;
         wv.off[n] = (int32_t)used;
         p[n] = r.p;
+        cost[n] = blk::block_cost(r.q, r.p);
         used += need;
         ++n;
       }
       wv.b0 = b0;
       wv.n = n;
-      if (n > 0) blk::assign_warps(p, n, NT / 32, wv.w0, wv.nw);
+      wv.ng = n > 0 ? blk::assign_warps(p, cost, n, NT / 32, wv.grp, wv.w0, wv.nw) : 0;
     }
     __syncthreads();
     const int n = wv.n;
@@ -556,17 +557,20 @@ __device__ void two_site_op_mixed(ChainDev* c, const OpDev op, int t, int bcols,
     }
     __syncthreads();
     const int g = blk::my_group(wv, warp);
-    if (g >= 0) {
-      const int ib = blk::own_block(wv, b0 + g);
+    for (int i = 0; g >= 0 && i < n; ++i) {
+      if (wv.grp[i] != g) continue;
+      const int ib = blk::own_block(wv, b0 + i);
       const blk::BlockRec& r = ss.b[ib];
-      float* W32 = smem + wv.off[g];
+      float* W32 = smem + wv.off[i];
       float* V32 = W32 + (size_t)r.p * blk::ld4(r.q);
-      const int sw = blk::jacobi_group<float>(W32, r.q, blk::ld4(r.q), r.p, V32, blk::ld4(r.p), V32 + (size_t)r.p * blk::ld4(r.p),
-                                              warp - wv.w0[g], wv.nw[g], g + 1, g, gs,
+      const int lw = warp - wv.w0[g], nw = wv.nw[g];
+      const int sw = blk::jacobi_group<float>(W32, r.q, blk::ld4(r.q), r.p, V32, blk::ld4(r.p),
+                                              V32 + (size_t)r.p * blk::ld4(r.p), lw, nw, g + 1, g, gs,
                                               polish ? kStop32Polished : kStop32, kMaxSweeps);
-      const int s64 = sw < 0 ? 0 : refine_block(c, r, W32, V32, c->X + refine::k_offset(ss, ib), polish, warp - wv.w0[g], wv.nw[g],
-                                                g + 1, g, gs);
-      if (warp == wv.w0[g] && (tid & 31) == 0) wv.sw[g] = sw < 0 || s64 < 0 ? -1 : sw + 1000 * s64;
+      const int s64 =
+          sw < 0 ? 0 : refine_block(c, r, W32, V32, c->X + refine::k_offset(ss, ib), polish, lw, nw, g + 1, g, gs);
+      if (lw == 0 && (tid & 31) == 0) wv.sw[i] = sw < 0 || s64 < 0 ? -1 : sw + 1000 * s64;
+      blk::group_sync(g + 1, 32 * nw);          // the group's flags are free for its next block
     }
     __syncthreads();
     for (int i = 0; i < n; ++i) {
