@@ -1089,6 +1089,42 @@ __device__ __forceinline__ void move_rows(float2 (&x)[2 * U], int n, int src) {
   }
 }
 
+template <int U>
+__device__ __forceinline__ float dot_rows(const float2 (&x)[2 * U], const float2 (&y)[2 * U]) {
+  float2 a = {0.0f, 0.0f}, b = {0.0f, 0.0f};
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    a = fma2(x[2 * u], y[2 * u], a);
+    b = fma2(x[2 * u + 1], y[2 * u + 1], b);
+  }
+  return (a.x + b.x) + (a.y + b.y);
+}
+
+// Rotation (c, s) and tangent t of a pair with squared norms na, nb and dot
+// product ga, by half-angle forms: with d = nb - na and h = sqrt(d^2 + 4 ga^2), c^2
+// = (1 + |d| / h) / 2 and s = sign(d) ga / (h c).  Two dependent reciprocal
+// square roots instead of two divides and two reciprocal square roots: the
+// angle is the longest link of a sub-round's chain.  d and ga are scaled by 1 /
+// sqrt(na nb), known before the dot product is.  (c, s) is conformal whatever
+// its rounding.  Returns the ratio |ga| / sqrt(na nb), or 0 (and c = 1, s = t =
+// 0) when the pair is not rotated: below tol, or a column below kTiny32 (noise
+// at binary32 resolution; the fast reciprocal square root flushes subnormal
+// inputs to 0).
+__device__ __forceinline__ float jacobi_angle32(float na, float nb, float ga, float tol, float& c, float& s, float& t) {
+  const float inv = rsqrtf(fmaxf(na, kTiny32)) * rsqrtf(fmaxf(nb, kTiny32));
+  const float d = (nb - na) * inv, g = ga * inv;
+  const float ratio = fabsf(g);
+  const bool go = ratio > tol && na > kTiny32 && nb > kTiny32;
+  const float ih = rsqrtf(fmaf(d, d, 4.0f * (g * g)));
+  const float c2 = fmaf(0.5f, fabsf(d) * ih, 0.5f);
+  const float rc = rsqrtf(c2);
+  const float sg = d < 0.0f ? -g : g;
+  c = go ? c2 * rc : 1.0f;
+  s = go ? sg * ih * rc : 0.0f;
+  t = go ? s * rc : 0.0f;
+  return go ? ratio : 0.0f;
+}
+
 // Block-ordered one-sided Jacobi as in jacobi_blocks, with super-columns of C
 // and a super-pair's 2 C columns of W and V in registers for its C sub-rounds
 // of cross pairs (L = 32 / C lanes a pair, q <= 4 L U; W and V 16-byte aligned,
@@ -1173,41 +1209,34 @@ __device__ int jacobi_regs(float* __restrict__ W, int q, int ldw, int p, float* 
           load_rows<U, L>(V + (size_t)b * ldv, p, sl, b < p, vb);
           float na = a < p ? nrm[a] : 0.0f, nb = b < p ? nrm[b] : 0.0f;   // 0: no pair
           int dirty = 0;
+          float ga = dot_rows<U>(xa, xb);
+#pragma unroll
+          for (int o = L / 2; o > 0; o >>= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
 #pragma unroll 1
           for (int k = 0; k < C; ++k) {
-            float2 acc = {0.0f, 0.0f}, acc2 = {0.0f, 0.0f};
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-              acc = fma2(xa[2 * u], xb[2 * u], acc);
-              acc2 = fma2(xa[2 * u + 1], xb[2 * u + 1], acc2);
-            }
-            float ga = (acc.x + acc2.x) + (acc.y + acc2.y);
-#pragma unroll
-            for (int o = L / 2; o > 0; o >>= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
-            // columns below kTiny32 are noise at binary32 resolution, and the
-            // fast reciprocal square root flushes subnormal inputs to 0
-            const float ratio = fabsf(ga) * (rsqrtf(fmaxf(na, kTiny32)) * rsqrtf(fmaxf(nb, kTiny32)));
-            const bool go = ga != 0.0f && na > kTiny32 && nb > kTiny32 && ratio > tol;
-            if (__any_sync(0xffffffffu, go)) {
-              float cs = 1.0f, sn = 0.0f;
-              if (go) {
-                rmax = fmaxf(rmax, ratio);
-                const float t = jacobi_tangent32(nb - na, ga);
-                cs = rsqrtf(1.0f + t * t);
-                sn = cs * t;
-                na -= t * ga;
-                nb += t * ga;
-              }
-              rotate_rows<U, L>(xa, xb, cs, sn, q);
-              rotate_rows<U, L>(va, vb, cs, sn, p);
-              dirty = 1;
-            }
+            float cs, sn, t;
+            const float ratio = jacobi_angle32(na, nb, ga, tol, cs, sn, t);
+            rmax = fmaxf(rmax, ratio);
+            dirty |= ratio > 0.0f;
+            na -= t * ga;
+            nb += t * ga;
+            rotate_rows<U, L>(xa, xb, cs, sn, q);
             if (k < C - 1) {
+              // the next pair's dot product first: V's rotation and move fill the
+              // latency of its reduction
               move_rows<U, L>(xb, q, next);
-              move_rows<U, L>(vb, p, next);
               nb = lane_value(nb, next);
+              ga = dot_rows<U>(xa, xb);
+              ga += __shfl_xor_sync(0xffffffffu, ga, 4);
+              rotate_rows<U, L>(va, vb, cs, sn, p);
+              ga += __shfl_xor_sync(0xffffffffu, ga, 2);
+              move_rows<U, L>(vb, p, next);
+              ga += __shfl_xor_sync(0xffffffffu, ga, 1);
+            } else {
+              rotate_rows<U, L>(va, vb, cs, sn, p);
             }
           }
+          dirty = __any_sync(0xffffffffu, dirty);
           if (dirty) {
             rot = 1;
             b = Bc * C + ((sub + C - 1) & (C - 1));    // the column it holds after C - 1 moves
