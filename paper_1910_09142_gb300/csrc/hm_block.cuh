@@ -464,7 +464,7 @@ __device__ void theta_direct(const ChainDev* c, int k, const SplitSh& s, T* __re
         acc[x] = T(0);
       }
       const int nr = min(R, Mv - g * R);
-#pragma unroll 4
+#pragma unroll 2
       for (int kk = 0; kk < K; ++kk) {
         const T bv = from64<T>(b[(size_t)kk * n]);
 #pragma unroll
@@ -1034,12 +1034,14 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) {
 // hit different banks).
 __host__ __device__ __forceinline__ int ld4(int n) { return (((n + 3) >> 2) | 1) * 4; }
 
-// Rows 4 (sl + L u) .. + 3 of a column (n rows, padded with zeros to a multiple of 4).
-template <int U, int L>
+// Register rows of jacobi_regs: lane sl of a column's eight holds rows 4 (sl + 8
+// u) .. + 3, u < U, as two pairs; n rows (zeros beyond, and up to a multiple of 4
+// in memory).
+template <int U>
 __device__ __forceinline__ void load_rows(const float* col, int n, int sl, bool ok, float2 (&x)[2 * U]) {
 #pragma unroll
   for (int u = 0; u < U; ++u) {
-    const int r = 4 * (sl + L * u);
+    const int r = 4 * (sl + 8 * u);
     float4 v = {0.0f, 0.0f, 0.0f, 0.0f};
     if (ok && r < n) v = *reinterpret_cast<const float4*>(col + r);
     x[2 * u] = {v.x, v.y};
@@ -1047,11 +1049,11 @@ __device__ __forceinline__ void load_rows(const float* col, int n, int sl, bool 
   }
 }
 
-template <int U, int L>
+template <int U>
 __device__ __forceinline__ void store_rows(float* col, int n, int sl, bool ok, const float2 (&x)[2 * U]) {
 #pragma unroll
   for (int u = 0; u < U; ++u) {
-    const int r = 4 * (sl + L * u);
+    const int r = 4 * (sl + 8 * u);
     if (ok && r < n)
       *reinterpret_cast<float4*>(col + r) = {x[2 * u].x, x[2 * u].y, x[2 * u + 1].x, x[2 * u + 1].y};
   }
@@ -1061,31 +1063,23 @@ __device__ __forceinline__ void store_rows(float* col, int n, int sl, bool ok, c
 // three shears by tan(angle / 2) and sin(angle) would take three operations
 // instead of four, but those two are rounded apart, and V's overlaps then
 // grew to 2e-6 (measured).
-template <int U, int L>
-__device__ __forceinline__ void rotate_rows(float2 (&x)[2 * U], float2 (&y)[2 * U], float c, float s, int n) {
+template <int U>
+__device__ __forceinline__ void rotate_rows(float2 (&x)[2 * U], float2 (&y)[2 * U], float c, float s) {
   const float2 cc = {c, c}, ss = {s, s}, ms = {-s, -s};
 #pragma unroll
-  for (int u = 0; u < U; ++u) {
-    if (4 * L * u >= n) break;                  // warp-uniform
-#pragma unroll
-    for (int v = 2 * u; v < 2 * u + 2; ++v) {
-      const float2 a = x[v], b = y[v];
-      x[v] = fma2(cc, a, mul2(ms, b));
-      y[v] = fma2(cc, b, mul2(ss, a));
-    }
+  for (int v = 0; v < 2 * U; ++v) {
+    const float2 a = x[v], b = y[v];
+    x[v] = fma2(cc, a, mul2(ms, b));
+    y[v] = fma2(cc, b, mul2(ss, a));
   }
 }
 
-template <int U, int L>
-__device__ __forceinline__ void move_rows(float2 (&x)[2 * U], int n, int src) {
+template <int U>
+__device__ __forceinline__ void move_rows(float2 (&x)[2 * U], int src) {
 #pragma unroll
-  for (int u = 0; u < U; ++u) {
-    if (4 * L * u >= n) break;                  // warp-uniform
-#pragma unroll
-    for (int v = 2 * u; v < 2 * u + 2; ++v) {
-      x[v].x = lane_value(x[v].x, src);
-      x[v].y = lane_value(x[v].y, src);
-    }
+  for (int v = 0; v < 2 * U; ++v) {
+    x[v].x = lane_value(x[v].x, src);
+    x[v].y = lane_value(x[v].y, src);
   }
 }
 
@@ -1125,10 +1119,42 @@ __device__ __forceinline__ float jacobi_angle32(float na, float nb, float ga, fl
   return go ? ratio : 0.0f;
 }
 
-// Block-ordered one-sided Jacobi as in jacobi_blocks, with super-columns of C
-// and a super-pair's 2 C columns of W and V in registers for its C sub-rounds
-// of cross pairs (L = 32 / C lanes a pair, q <= 4 L U; W and V 16-byte aligned,
-// leading dimensions multiples of 4).
+// The three rounds of pairs inside a super-column of four, its column a lane
+// group's x (W) and v (V) with squared norm nx (0: no column): groups exchange
+// copies with the group m away, m = 1, 2, 3, and each rotates its own column.
+template <int U>
+__device__ __forceinline__ void intra_rows(float2 (&x)[2 * U], float2 (&v)[2 * U], float& nx, float tol, float& rmax) {
+  const int lane = threadIdx.x & 31, sub = lane >> 3;
+#pragma unroll 1
+  for (int m = 1; m < 4; ++m) {
+    const int src = lane ^ (8 * m);
+    const bool first = sub < (sub ^ m);
+    float2 y[2 * U];
+#pragma unroll
+    for (int u = 0; u < 2 * U; ++u) y[u] = x[u];
+    move_rows<U>(y, src);
+    const float ny = lane_value(nx, src);
+    float ga = dot_rows<U>(x, y);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
+    float c, s, t;
+    const float ratio = jacobi_angle32(first ? nx : ny, first ? ny : nx, ga, tol, c, s, t);
+    rmax = fmaxf(rmax, ratio);
+    nx += first ? -t * ga : t * ga;
+    const float ps = first ? -s : s;
+    const float2 cc = {c, c}, ss = {ps, ps};
+#pragma unroll
+    for (int u = 0; u < 2 * U; ++u) {
+      x[u] = fma2(cc, x[u], mul2(ss, y[u]));
+      const float2 o = {lane_value(v[u].x, src), lane_value(v[u].y, src)};
+      v[u] = fma2(cc, v[u], mul2(ss, o));
+    }
+  }
+}
+
+// Block-ordered one-sided Jacobi as in jacobi_blocks, with a super-pair's eight
+// columns of W and V in registers for all of its sub-rounds (q <= 32 U; W
+// and V 16-byte aligned, leading dimensions multiples of 4).
 //
 // jacobi_blocks loads and stores every column of W and V once per rotation: 8 n
 // shared-memory words a pair against 9 n multiply-adds, and shared memory moves
@@ -1138,15 +1164,23 @@ __device__ __forceinline__ float jacobi_angle32(float na, float nb, float ga, fl
 // super-pair (128-bit accesses); lane group `sub` keeps column A + sub, and the
 // columns of the other super-column move on to the next group by shuffles.
 // What is left is the chain of a sub-round (dot product, reduction, angle,
-// rotation: ~300 clocks).  C = 4: eight pairs a sub-round (C = 8, 4 lanes a
-// pair) measured 3 % faster on blocks of up to 32 rows and 10 % slower above.
+// rotation: ~300 clocks).  Super-columns of eight (4 lanes a pair) measured 3 %
+// faster on blocks of up to 32 rows and 10 % slower above.
 // Lx = 9, 2W = 8, chi = 256, binary32, 152 chains: 269 ms a Markov step with
 // jacobi_blocks, 208 ms with this.
-template <int U, int C>
+//
+// Two copies, U = 2 and 4, for every size.  The groups of a CTA work on blocks of
+// different sizes at once, and four copies (and the shared-memory pass for the pairs
+// inside a super-column) overflowed the instruction cache: 8.6 of 21.9
+// clocks an instruction went to waiting for instructions (Lx = 6, chi = 96, two
+// chains per SM).  One copy that skips unused rows by branches was faster
+// there (ladder of Lx = 16, 256 chains: 761 -> 651 ms a step) but its branches sit
+// on the chain of every sub-round (Lx = 9, one chain per SM: 196 -> 256 ms).
+template <int U>
 __device__ int jacobi_regs(float* __restrict__ W, int q, int ldw, int p, float* __restrict__ V, int ldv,
-                           float* __restrict__ nrm, int lw, int nw, int bar, int g, GroupSh& gs, float stop,
-                           int max_sweeps) {
-  constexpr int L = 32 / C;
+                                  float* __restrict__ nrm, int lw, int nw, int bar, int g, GroupSh& gs, float stop,
+                                  int max_sweeps) {
+  constexpr int L = 8, C = 4;
   const int lane = threadIdx.x & 31;
   const int sub = lane / L, sl = lane % L;
   const int nthr = 32 * nw;
@@ -1165,13 +1199,9 @@ __device__ int jacobi_regs(float* __restrict__ W, int q, int ldw, int p, float* 
       s2 = warp_sum_t(s2);
       if (lane == 0) nrm[j] = s2;
     }
-    if (lw == 0 && lane == 0) {
-      gs.flag[g] = 0;
-      gs.rbits[g] = 0u;
-    }
+    if (lw == 0 && lane == 0) gs.rbits[g] = 0u;
     group_sync(bar, nthr);
-    float rmax = 0.0f;
-    int rot = 0;
+    float rmax = 0.0f;                     // > 0: some pair was rotated
     for (int sr = 0; sr < ns2 - 1; ++sr) {
       for (int sp = lw; sp < nsp; sp += nw) {                       // warp-uniform
         const int m = ns2 - 1;             // (sr +- sp) mod m, as for the columns
@@ -1185,98 +1215,74 @@ __device__ int jacobi_regs(float* __restrict__ W, int q, int ldw, int p, float* 
           Bc = sr - sp;
           if (Bc < 0) Bc += m;
         }
-        const bool okA = A < ns, okB = Bc < ns;
+        const bool both = A < ns && Bc < ns;         // ns2 > ns: one padding super-column
+        if (!both && sr > 0) continue;
+        const int a = A * C + sub;
+        int b = Bc * C + sub;
+        float2 xa[2 * U], xb[2 * U], va[2 * U], vb[2 * U];
+        load_rows<U>(W + (size_t)a * ldw, q, sl, a < p, xa);
+        load_rows<U>(W + (size_t)b * ldw, q, sl, b < p, xb);
+        load_rows<U>(V + (size_t)a * ldv, p, sl, a < p, va);
+        load_rows<U>(V + (size_t)b * ldv, p, sl, b < p, vb);
+        float na = a < p ? nrm[a] : 0.0f, nb = b < p ? nrm[b] : 0.0f;   // 0: no pair
+        float rs = 0.0f;                             // largest ratio rotated here
         if (sr == 0) {
-          // pairs inside A (the lower half of the groups) and inside B (the upper):
-          // the round robin of C columns
-          const int base = (sub < C / 2 ? A : Bc) * C, x = sub & (C / 2 - 1);
-          const bool ok = sub < C / 2 ? okA : okB;
-          for (int k = 0; k < C - 1; ++k) {
-            int a = base + (x == 0 ? k : (k + x) % (C - 1));
-            int b = base + (x == 0 ? C - 1 : (k + C - 1 - x) % (C - 1));
-            if (!ok || a >= p || b >= p) a = b = -1;
-            jacobi_pass<float, float, L, 4>(W, q, ldw, p, V, ldv, nrm, a, b, sl, tol, stop, rmax, rot);
-            __syncwarp();
-          }
+          intra_rows<U>(xa, va, na, tol, rs);
+          intra_rows<U>(xb, vb, nb, tol, rs);
         }
-        if (okA && okB) {
-          const int a = A * C + sub;
-          int b = Bc * C + sub;
-          float2 xa[2 * U], xb[2 * U], va[2 * U], vb[2 * U];
-          load_rows<U, L>(W + (size_t)a * ldw, q, sl, a < p, xa);
-          load_rows<U, L>(W + (size_t)b * ldw, q, sl, b < p, xb);
-          load_rows<U, L>(V + (size_t)a * ldv, p, sl, a < p, va);
-          load_rows<U, L>(V + (size_t)b * ldv, p, sl, b < p, vb);
-          float na = a < p ? nrm[a] : 0.0f, nb = b < p ? nrm[b] : 0.0f;   // 0: no pair
-          int dirty = 0;
+        if (both) {
           float ga = dot_rows<U>(xa, xb);
 #pragma unroll
           for (int o = L / 2; o > 0; o >>= 1) ga += __shfl_xor_sync(0xffffffffu, ga, o);
 #pragma unroll 1
           for (int k = 0; k < C; ++k) {
             float cs, sn, t;
-            const float ratio = jacobi_angle32(na, nb, ga, tol, cs, sn, t);
-            rmax = fmaxf(rmax, ratio);
-            dirty |= ratio > 0.0f;
+            rs = fmaxf(rs, jacobi_angle32(na, nb, ga, tol, cs, sn, t));
             na -= t * ga;
             nb += t * ga;
-            rotate_rows<U, L>(xa, xb, cs, sn, q);
-            if (k < C - 1) {
-              // the next pair's dot product first: V's rotation and move fill the
-              // latency of its reduction
-              move_rows<U, L>(xb, q, next);
-              nb = lane_value(nb, next);
-              ga = dot_rows<U>(xa, xb);
-              ga += __shfl_xor_sync(0xffffffffu, ga, 4);
-              rotate_rows<U, L>(va, vb, cs, sn, p);
-              ga += __shfl_xor_sync(0xffffffffu, ga, 2);
-              move_rows<U, L>(vb, p, next);
-              ga += __shfl_xor_sync(0xffffffffu, ga, 1);
-            } else {
-              rotate_rows<U, L>(va, vb, cs, sn, p);
-            }
+            rotate_rows<U>(xa, xb, cs, sn);
+            // the next pair's dot product first: V's rotation and move fill the
+            // latency of its reduction (the last move brings the columns home)
+            move_rows<U>(xb, next);
+            nb = lane_value(nb, next);
+            ga = dot_rows<U>(xa, xb);
+            ga += __shfl_xor_sync(0xffffffffu, ga, 4);
+            rotate_rows<U>(va, vb, cs, sn);
+            ga += __shfl_xor_sync(0xffffffffu, ga, 2);
+            move_rows<U>(vb, next);
+            ga += __shfl_xor_sync(0xffffffffu, ga, 1);
           }
-          dirty = __any_sync(0xffffffffu, dirty);
-          if (dirty) {
-            rot = 1;
-            b = Bc * C + ((sub + C - 1) & (C - 1));    // the column it holds after C - 1 moves
-            store_rows<U, L>(W + (size_t)a * ldw, q, sl, a < p, xa);
-            store_rows<U, L>(W + (size_t)b * ldw, q, sl, b < p, xb);
-            store_rows<U, L>(V + (size_t)a * ldv, p, sl, a < p, va);
-            store_rows<U, L>(V + (size_t)b * ldv, p, sl, b < p, vb);
-            if (sl == 0) {
-              if (a < p) nrm[a] = na;
-              if (b < p) nrm[b] = nb;
-            }
-          }
-          __syncwarp();
         }
+        if (__any_sync(0xffffffffu, rs > 0.0f)) {
+          rmax = fmaxf(rmax, rs);
+          store_rows<U>(W + (size_t)a * ldw, q, sl, a < p, xa);
+          store_rows<U>(W + (size_t)b * ldw, q, sl, b < p, xb);
+          store_rows<U>(V + (size_t)a * ldv, p, sl, a < p, va);
+          store_rows<U>(V + (size_t)b * ldv, p, sl, b < p, vb);
+          if (sl == 0) {
+            if (a < p) nrm[a] = na;
+            if (b < p) nrm[b] = nb;
+          }
+        }
+        __syncwarp();
       }
       group_sync(bar, nthr);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
-    const int anyrot = __any_sync(0xffffffffu, rot);
-    if (lane == 0) {
-      if (anyrot) atomicMax(&gs.flag[g], 1);
-      atomicMax(&gs.rbits[g], __float_as_uint(rmax));
-    }
+    if (lane == 0) atomicMax(&gs.rbits[g], __float_as_uint(rmax));
     group_sync(bar, nthr);
-    const int any = gs.flag[g];
     const float rm = __uint_as_float(gs.rbits[g]);
     group_sync(bar, nthr);
-    if (!any || rm < stop) return sweep;
+    if (rm < stop) return sweep;             // 0: no rotation
   }
   return -1;
 }
 
-constexpr int kRegsMin = 16;
-
-// One-sided Jacobi of one block by a warp group: the block ordering for
-// binary32 blocks of 16 columns or more (jacobi_regs up to 128 rows, where the
-// columns fit in registers, jacobi_blocks above), otherwise the
-// round-robin ordering with 8 lanes a pair.  Neither depends on the number of
-// warps, nor does anything else a block goes through, so a chain's results are
+// One-sided Jacobi of one block by a warp group: jacobi_regs for binary32
+// blocks of up to 128 rows; above, the block ordering in shared memory for 16
+// columns or more; otherwise (binary64) the round-robin ordering with 8 lanes a
+// pair.  None of them depends on the number of warps, nor does anything else a block goes through, so a chain's results are
 // the same bits whatever batch or team it runs in.
 // TV: element type of V.  A binary64 polish of a binary32 result may keep V
 // in binary32: V carries binary32 accuracy from the preconditioning sweeps
@@ -1290,12 +1296,8 @@ __device__ int jacobi_group(T* __restrict__ W, int q, int ldw, int p, TV* __rest
                             T* __restrict__ nrm, int lw, int nw, int bar, int g, GroupSh& gs, T stop, int max_sweeps) {
   if constexpr (sizeof(T) == sizeof(float)) {
     const bool vec = ((ldw | ldv) & 3) == 0 && ((reinterpret_cast<uintptr_t>(W) | reinterpret_cast<uintptr_t>(V)) & 15) == 0;
-    if (p >= kRegsMin && vec) {
-      if (q <= 32) return jacobi_regs<1, 4>(W, q, ldw, p, V, ldv, nrm, lw, nw, bar, g, gs, stop, max_sweeps);
-      if (q <= 64) return jacobi_regs<2, 4>(W, q, ldw, p, V, ldv, nrm, lw, nw, bar, g, gs, stop, max_sweeps);
-      if (q <= 96) return jacobi_regs<3, 4>(W, q, ldw, p, V, ldv, nrm, lw, nw, bar, g, gs, stop, max_sweeps);
-      if (q <= 128) return jacobi_regs<4, 4>(W, q, ldw, p, V, ldv, nrm, lw, nw, bar, g, gs, stop, max_sweeps);
-    }
+    if (vec && q <= 64) return jacobi_regs<2>(W, q, ldw, p, V, ldv, nrm, lw, nw, bar, g, gs, stop, max_sweeps);
+    if (vec && q <= 128) return jacobi_regs<4>(W, q, ldw, p, V, ldv, nrm, lw, nw, bar, g, gs, stop, max_sweeps);
     if (p >= 16) return jacobi_blocks<T, TV, B>(W, q, ldw, p, V, ldv, nrm, lw, nw, bar, g, gs, stop, max_sweeps);
   }
   return jacobi_lanes<T, TV, 8, B>(W, q, ldw, p, V, ldv, nrm, lw, nw, bar, g, gs, stop, max_sweeps);

@@ -476,6 +476,13 @@ __device__ int decompose_block(const double* A, int q, int p, double* base, floa
   return blk::jacobi_group<double, double, 2>(W, q, ldw, p, V, ldv, nrm, lw, nw, bar, g, gs, kStop64, kMaxSweeps);
 }
 
+// The sweeps of a block too large for shared memory, in global memory by the
+// whole CTA.  Rare: kept out of line, away from the hot code.
+__device__ HM_COLD int sweep_global(double* W, int q, int p, double* V, double* nrm, int warp, int nw,
+                                         blk::GroupSh& gs) {
+  return blk::jacobi_group<double, double, 2>(W, q, q, p, V, p, nrm, warp, nw, 1, 0, gs, kStop64, kMaxSweeps);
+}
+
 // One two-site op of a chain, block by block in the S^z charge of the new
 // middle bond (Sec. II.C): theta by block GEMMs, the gate within its
 // conserved sectors, the blocks' decompositions, then one truncation over the
@@ -529,8 +536,7 @@ __device__ void two_site_op_blocked(ChainDev* c, const OpDev op, int t, double* 
     const int n = wv.n;
     if (n == 0) {
       const blk::BlockRec& r = ss.b[blk::own_block(wv, b0)];
-      const int sw = blk::jacobi_group<double, double, 2>(c->W + r.woff, r.q, r.q, r.p, c->V + r.voff, r.p, c->sig, warp,
-                                                          NTE / 32, 1, 0, sh.gs, kStop64, kMaxSweeps);
+      const int sw = sweep_global(c->W + r.woff, r.q, r.p, c->V + r.voff, c->sig, warp, NTE / 32, sh.gs);
       if (sw < 0) {
         set_error(c, HM_ERR_NUMERIC, t, ctx_err);
         failed = true;

@@ -7,6 +7,14 @@
 
 #include "../../include/hmetts.h"
 
+// A rarely taken device function: out of line, so that its code does not crowd
+// the hot path's out of the instruction cache.
+#if defined(__CUDACC__)
+#define HM_COLD __noinline__
+#else
+#define HM_COLD
+#endif
+
 namespace hm {
 
 // Site kinds of the hybrid state (Sec. I.C, Fig. 4).

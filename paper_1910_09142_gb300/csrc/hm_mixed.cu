@@ -408,6 +408,13 @@ constexpr double kPolishStop = 1e-5;
 // kPolishStop, so one binary64 sweep still ends the polish.
 constexpr float kStop32 = 2e-4f, kStop32Polished = 1e-3f;
 
+// The binary64 sweeps of a block the first-order step does not settle.  Rare:
+// kept out of line, away from the hot code.
+__device__ HM_COLD int sweep64(double* W, int q, int p, double* V, double* nrm, int lw, int nw, int bar, int g,
+                                    blk::GroupSh& gs) {
+  return blk::jacobi_group<double, double, 2>(W, q, q, p, V, p, nrm, lw, nw, bar, g, gs, kPolishStop, kMaxSweeps);
+}
+
 // From a block's binary32 result (W32, V32 in shared memory, followed by
 // refine::extra floats) to its binary64 W and V (global memory), by the nw
 // warps of its group.  polish: the binary64-accurate finish of hm_refine.cuh;
@@ -431,8 +438,9 @@ __device__ int refine_block(ChainDev* c, const blk::BlockRec& r, float* W32, flo
   }
   blk::group_sync(bar, nthr);
   if (!polish) {
-    refine::scale_columns(W32, q, ldw, p, dl, W64, lw, nw);
-    refine::scale_columns(V32, p, ldv, p, dl, V64, lw, nw);
+#pragma unroll 1
+    for (int side = 0; side < 2; ++side)
+      refine::scale_columns(side ? V32 : W32, side ? p : q, side ? ldv : ldw, p, dl, side ? V64 : W64, lw, nw);
     return 0;
   }
   float e = refine::pair_terms<false>(W32, q, ldw, p, ah, al, K, lw, nw);
@@ -441,8 +449,11 @@ __device__ int refine_block(ChainDev* c, const blk::BlockRec& r, float* W32, flo
   if ((threadIdx.x & 31) == 0) atomicMax(&gs.rbits[g], __float_as_uint(e));
   blk::group_sync(bar, nthr);                 // K and its largest entry are complete
   int x = 0;
-  refine::add_product<false>(W32, q, ldw, p, K, W64, q, lw, nw, x);
-  refine::add_product<false>(V32, p, ldv, p, K, V64, p, lw, nw, x);
+#pragma unroll 1
+  for (int side = 0; side < 2; ++side) {
+    const int n = side ? p : q;
+    refine::add_product<false>(side ? V32 : W32, n, side ? ldv : ldw, p, K, side ? V64 : W64, n, lw, nw, x);
+  }
   blk::group_sync(bar, nthr);
   if (lw == 0) {
     const int found = refine::rotate_near(W64, q, V64, p, ah, 2 * p);
@@ -455,12 +466,38 @@ __device__ int refine_block(ChainDev* c, const blk::BlockRec& r, float* W32, flo
   blk::group_sync(bar, nthr);                 // every warp has read the flag
   int s64 = 1;
   if (more == 2) {
-    s64 = blk::jacobi_group<double, double, 2>(W64, q, q, p, V64, p, c->sig + r.svoff, lw, nw, bar, g, gs, kPolishStop,
-                                               kMaxSweeps);
+    s64 = sweep64(W64, q, p, V64, c->sig + r.svoff, lw, nw, bar, g, gs);
     blk::group_sync(bar, nthr);
   }
   refine::unit_columns(W64, q, V64, p, lw, nw);
   return s64;
+}
+
+// One block too large for shared memory, by the whole CTA: binary32 sweeps on
+// column blocks staged from global memory, then the binary64 sweep.  Returns
+// the binary32 sweeps + 1000 x the binary64 ones, or -1.  Out of line: it is
+// rare, and its code would crowd the usual path's.
+__device__ HM_COLD int decompose_staged(ChainDev* c, int k, const blk::SplitSh& ss, const blk::BlockRec& r,
+                                             const float* theta, int bcols, int polish, float* smem, Scal& sc,
+                                             blk::GroupSh& gs) {
+  const int warp = threadIdx.x >> 5;
+  float* W32 = c->X;
+  float* V32 = c->X + (size_t)r.q * r.p;
+  int c0 = 0;
+  blk::gather_block<NT, float, float>(c, k, ss, r, theta, W32, r.q, V32, r.p, c0);
+  __syncthreads();
+  const int sw = cta_jacobi_f32(W32, r.q, r.p, V32, bcols, smem, sc, nullptr);
+  if (sw < 0) return -1;
+  double* W64 = c->W + r.woff;
+  double* V64 = c->V + r.voff;
+  promote_w(W32, r.q, V32, r.p, r.q, r.p, W64, c->sig);
+  __syncthreads();
+  const int s64 = polish ? blk::jacobi_group<double, float, 2>(W64, r.q, r.q, r.p, V32, r.p, c->sig, warp, NT / 32, 1,
+                                                               0, gs, kPolishStop, kMaxSweeps)
+                         : 0;
+  __syncthreads();
+  promote_v(V32, r.p, r.q, r.p, W64, V64, c->sig, polish);
+  return s64 < 0 ? -1 : sw + 1000 * s64;
 }
 
 // Shared-memory floats of one block: W, V and the finish's terms.
@@ -518,33 +555,14 @@ __device__ void two_site_op_mixed(ChainDev* c, const OpDev op, int t, int bcols,
     const int n = wv.n;
     if (n == 0) {
       const blk::BlockRec& r = ss.b[blk::own_block(wv, b0)];
-      float* W32 = c->X;
-      float* V32 = c->X + (size_t)r.q * r.p;
-      int c0 = 0;
-      blk::gather_block<NT, float, float>(c, op.k, ss, r, theta, W32, r.q, V32, r.p, c0);
-      __syncthreads();
-      const int sw = cta_jacobi_f32(W32, r.q, r.p, V32, bcols, smem, sc, nullptr);
-      if (sw < 0) {
-        set_error(c, HM_ERR_NUMERIC, t, ctx_err);
-        failed = true;
-        break;
-      }
-      double* W64 = c->W + r.woff;
-      double* V64 = c->V + r.voff;
-      promote_w(W32, r.q, V32, r.p, r.q, r.p, W64, c->sig);
-      __syncthreads();
-      const int s64 = polish ? blk::jacobi_group<double, float, 2>(W64, r.q, r.q, r.p, V32, r.p, c->sig, warp, NT / 32,
-                                                                1, 0, gs, kPolishStop, kMaxSweeps)
-                             : 0;
-      __syncthreads();
-      promote_v(V32, r.p, r.q, r.p, W64, V64, c->sig, polish);
-      if (s64 < 0) {
+      const int code = decompose_staged(c, op.k, ss, r, theta, bcols, polish, smem, sc, gs);
+      if (code < 0) {
         set_error(c, HM_ERR_NUMERIC, t, ctx_err);
         failed = true;
         break;
       }
       const int64_t cb = (int64_t)r.q * r.p * r.p;
-      if (cb > cost) cost = cb, sw32 = sw, sw64 = s64;
+      if (cb > cost) cost = cb, sw32 = code % 1000, sw64 = code / 1000;
       b0 += 1;
       continue;
     }
