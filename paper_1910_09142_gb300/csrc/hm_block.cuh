@@ -999,7 +999,7 @@ __device__ int jacobi_blocks(T* __restrict__ W, int q, int ldw, int p, TV* __res
   return -1;
 }
 
-// Two binary32 multiply-adds (products) in one instruction (sm_100 and later).
+// Two binary32 operations in one instruction (sm_100 and later).
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
 #if defined(__CUDA_ARCH__)
   unsigned long long x, y, z, r;
@@ -1028,6 +1028,23 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) {
   return {a.x * b.x, a.y * b.y};
 #endif
 }
+
+__device__ __forceinline__ float2 add2p(float2 a, float2 b) {
+#if defined(__CUDA_ARCH__)
+  unsigned long long x, y, r;
+  memcpy(&x, &a, 8);
+  memcpy(&y, &b, 8);
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+  float2 d;
+  memcpy(&d, &r, 8);
+  return d;
+#else
+  return {a.x + b.x, a.y + b.y};
+#endif
+}
+
+// a - b as one multiply-add (exact product with -1).
+__device__ __forceinline__ float2 sub2p(float2 a, float2 b) { return fma2(b, {-1.0f, -1.0f}, a); }
 
 // Leading dimension of a binary32 column for jacobi_regs: a multiple of four
 // (128-bit loads), an odd one (lanes that read the same rows of eight columns

@@ -430,6 +430,10 @@ __device__ int refine_block(ChainDev* c, const blk::BlockRec& r, float* W32, flo
   double* W64 = c->W + r.woff;
   double* V64 = c->V + r.voff;
   const int nthr = 32 * nw;
+  if (q > 128) {                              // the sweeps went through jacobi_blocks: pad the columns
+    refine::pad_rows(W32, q, ldw, p, lw, nw);
+    refine::pad_rows(V32, p, ldv, p, lw, nw);
+  }
   blk::group_sync(bar, nthr);                 // the sweeps' last reads of the norms
   refine::column_terms(W32, q, ldw, V32, p, ldv, ah, al, dl, polish ? K : nullptr, lw, nw);
   if (lw == 0 && (threadIdx.x & 31) == 0) {

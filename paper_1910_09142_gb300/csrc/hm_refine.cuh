@@ -61,24 +61,26 @@ __device__ __forceinline__ F2 normal2(F2 a) {
   return {s, a.l - (s - a.h)};
 }
 
-// Running dot product: t = big + the products rounded to big's last bit, l =
-// everything below.  big > 2 |every partial sum|, so t + p, (t + p) - t and
-// p - ((t + p) - t) are exact splits (Dekker's fast two-sum).
+// Two running dot products (of the even and the odd rows): t = big + the
+// products rounded to big's last bit, l = everything below.  big > 2 |every
+// partial sum|, so t + p, (t + p) - t and p - ((t + p) - t) are exact splits
+// (Dekker's fast two-sum).  Seven packed instructions for two terms.
 struct Dot2 {
-  float t, l;
+  float2 t, l;
   __device__ __forceinline__ void start(float big) {
-    t = big;
-    l = 0.0f;
+    t = {big, big};
+    l = {0.0f, 0.0f};
   }
-  __device__ __forceinline__ void add(float x, float y) {
-    const float p = x * y;
-    const float e = fmaf(x, y, -p);
-    const float s = t + p;
-    l += p - (s - t);
-    l += e;
+  // ny = -y
+  __device__ __forceinline__ void add(float2 x, float2 y, float2 ny) {
+    const float2 p = blk::mul2(x, y);
+    const float2 e = blk::fma2(x, ny, p);                  // -(the product's low part)
+    const float2 s = blk::add2p(t, p);
+    l = blk::add2p(l, blk::sub2p(p, blk::sub2p(s, t)));
+    l = blk::sub2p(l, e);
     t = s;
   }
-  __device__ __forceinline__ F2 get(float big) const { return {t - big, l}; }
+  __device__ __forceinline__ F2 get(float big) const { return add2({t.x - big, l.x}, {t.y - big, l.y}); }
 };
 
 // Power of two above 4 x (x > 0, normal).
@@ -102,20 +104,21 @@ __device__ __forceinline__ int k_offset(const blk::SplitSh& s, int b) {
 
 __device__ __forceinline__ bool near_pair(float a, float b) { return fabsf(b - a) < kNear * fmaxf(a, b); }
 
-// Squared norm of one column by a warp.
-__device__ __forceinline__ F2 warp_norm2(const float* x, int n) {
-  const int lane = threadIdx.x & 31;
-  float m = 0.0f;
-  for (int i = lane; i < n; i += 32) m = fmaf(x[i], x[i], m);
-  m = blk::warp_sum_t(m);
-  if (!(m > 0.0f)) return {0.0f, 0.0f};
-  const float big = above(m);
+// Squared norm of a column (zero rows up to a multiple of four) by its eight
+// lanes; top: about its size, not below half of it.
+__device__ __forceinline__ F2 norm2(const float* x, int n, float top) {
+  const int sl = threadIdx.x & 7;
+  const float big = above(fmaxf(top, 1e-36f));
   Dot2 d;
   d.start(big);
-  for (int i = lane; i < n; i += 32) d.add(x[i], x[i]);
+  for (int r = 4 * sl; r < n; r += 32) {
+    const float4 v = *reinterpret_cast<const float4*>(x + r);
+    d.add({v.x, v.y}, {v.x, v.y}, {-v.x, -v.y});
+    d.add({v.z, v.w}, {v.z, v.w}, {-v.z, -v.w});
+  }
   F2 s = d.get(big);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
+  for (int o = 4; o > 0; o >>= 1)
     s = add2(s, {__shfl_xor_sync(0xffffffffu, s.h, o), __shfl_xor_sync(0xffffffffu, s.l, o)});
   return normal2(s);
 }
@@ -123,15 +126,21 @@ __device__ __forceinline__ F2 warp_norm2(const float* x, int n) {
 // x' = x + (x delta + products with K): one column entry, binary64.
 __device__ __forceinline__ double corrected(float x, float corr) { return blk::widen(x) + blk::widen(corr); }
 
-// delta_j and the squared norms of the columns; KT: zeroed padding and the
-// diagonal; W: zeroed rows up to a multiple of four.
-__device__ inline void column_terms(float* W, int q, int ldw, const float* V, int p, int ldv, float* ah, float* al,
-                             float* dl, float* KT, int lw, int nw) {
-  const int lane = threadIdx.x & 31;
+// delta_j and the squared norms of the columns (ah holds the sweeps' running
+// ones); KT: zeroed padding and the diagonal.  W and V: zero rows up to a
+// multiple of four (jacobi_regs leaves them so; padded here for the other
+// orderings by pad_rows).  Eight lanes a column.
+__device__ inline void column_terms(const float* W, int q, int ldw, const float* V, int p, int ldv, float* ah, float* al,
+                                    float* dl, float* KT, int lw, int nw) {
+  const int sub = (threadIdx.x & 31) >> 3, sl = threadIdx.x & 7;
   const int ldk = ldk_of(p);
-  for (int j = lw; j < p; j += nw) {
-    const F2 a = warp_norm2(W + (size_t)j * ldw, q), v = warp_norm2(V + (size_t)j * ldv, p);
-    if (lane == 0) {
+  for (int j0 = 4 * lw; j0 < p; j0 += 4 * nw) {
+    const int j = j0 + sub, jj = j < p ? j : p - 1;
+    const F2 a = norm2(W + (size_t)jj * ldw, q, 1.5f * ah[jj]);
+    const F2 v = norm2(V + (size_t)jj * ldv, p, 1.5f);
+    __syncwarp();                             // every lane has read its column's running norm
+    if (j >= p) continue;
+    if (sl == 0) {
       ah[j] = a.h;
       al[j] = a.l;
       // 1 / sqrt(1 + u) - 1 (u ~ 1e-5; a null column keeps its scale)
@@ -140,23 +149,31 @@ __device__ inline void column_terms(float* W, int q, int ldw, const float* V, in
       dl[j] = d;
       if (KT) KT[(size_t)j * ldk + j] = d;
     }
-    if (KT && lane >= 1 && p + lane - 1 < ldk) KT[(size_t)j * ldk + p + lane - 1] = 0.0f;
-    if (q + lane < ((q + 3) & ~3)) W[(size_t)j * ldw + q + lane] = 0.0f;   // pair_terms reads rows in fours
+    if (KT && p + sl < ldk) KT[(size_t)j * ldk + p + sl] = 0.0f;
   }
 }
 
-// The diagonal of the orthonormalisation step, -1/2 of |v_j|^2 - 1, and the
-// squared norms (ah); KT: zeroed padding.
-__device__ inline void unit_terms(const float* V, int p, int ldv, float* ah, float* KT, int lw, int nw) {
+// Zero rows n .. up to a multiple of four of p columns.
+__device__ inline void pad_rows(float* X, int n, int ldx, int p, int lw, int nw) {
   const int lane = threadIdx.x & 31;
+  for (int j = lw; j < p; j += nw)
+    if (n + lane < ((n + 3) & ~3)) X[(size_t)j * ldx + n + lane] = 0.0f;
+}
+
+// The diagonal of the orthonormalisation step, -1/2 of |v_j|^2 - 1, and the
+// squared norms (ah); KT: zeroed padding.  V: zero rows up to a multiple of four.
+__device__ inline void unit_terms(const float* V, int p, int ldv, float* ah, float* KT, int lw, int nw) {
+  const int sub = (threadIdx.x & 31) >> 3, sl = threadIdx.x & 7;
   const int ldk = ldk_of(p);
-  for (int j = lw; j < p; j += nw) {
-    const F2 v = warp_norm2(V + (size_t)j * ldv, p);
-    if (lane == 0) {
+  for (int j0 = 4 * lw; j0 < p; j0 += 4 * nw) {
+    const int j = j0 + sub, jj = j < p ? j : p - 1;
+    const F2 v = norm2(V + (size_t)jj * ldv, p, 1.5f);
+    if (j >= p) continue;
+    if (sl == 0) {
       ah[j] = v.h;
       KT[(size_t)j * ldk + j] = -0.5f * ((v.h - 1.0f) + v.l);
     }
-    if (lane >= 1 && p + lane - 1 < ldk) KT[(size_t)j * ldk + p + lane - 1] = 0.0f;
+    if (p + sl < ldk) KT[(size_t)j * ldk + p + sl] = 0.0f;
   }
 }
 
@@ -194,13 +211,12 @@ __device__ inline float pair_terms(const float* W, int q, int ldw, int p, const 
       // rows in fours (128-bit loads; the rows from q on are zeros)
       for (int k = 0; k < q; k += 4) {
         const float4 yv = *reinterpret_cast<const float4*>(y + k);
+        const float2 y0 = {yv.x, yv.y}, y1 = {yv.z, yv.w}, n0 = {-yv.x, -yv.y}, n1 = {-yv.z, -yv.w};
 #pragma unroll
         for (int r = 0; r < R; ++r) {
           const float4 xv = *reinterpret_cast<const float4*>(xi[r] + k);
-          d[r].add(xv.x, yv.x);
-          d[r].add(xv.y, yv.y);
-          d[r].add(xv.z, yv.z);
-          d[r].add(xv.w, yv.w);
+          d[r].add({xv.x, xv.y}, y0, n0);
+          d[r].add({xv.z, xv.w}, y1, n1);
         }
       }
 #pragma unroll
@@ -229,50 +245,53 @@ __device__ inline float pair_terms(const float* W, int q, int ldw, int p, const 
 
 // out[:, j] = base[:, j] + X K[:, j], X n x p (shared, leading dimension ldx); base
 // = X, or out itself (ADD).  out: binary64 column-major, leading dimension
-// ldo.  A warp takes 128 rows x 4 columns; K comes four entries at a time, the
-// same for all lanes.  x: running task count (the tasks go round the warps).
+// ldo.  A warp takes 64 rows x 4 columns.  Its four columns of K are loaded
+// 32 entries at a time, an entry a lane, and handed round by shuffles: K lies in
+// global memory, and a load per step of the product would wait for each.
+// x: running task count (the tasks go round the warps).
 template <bool ADD>
 __device__ inline void add_product(const float* X, int n, int ldx, int p, const float* KT, double* out, int ldo,
                                    int lw, int nw, int& x) {
   const int lane = threadIdx.x & 31;
   const int ldk = ldk_of(p);
-  for (int r0 = 0; r0 < n; r0 += 128) {
-    const int nu = min(4, (n - r0 + 31) >> 5);
+  for (int r0 = 0; r0 < n; r0 += 64) {
+    const bool in0 = r0 + lane < n, in1 = r0 + 32 + lane < n;
     for (int j0 = 0; j0 < p; j0 += 4, ++x) {
       if (x % nw != lw) continue;
-      float acc[4][4];
+      float acc[2][4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+      for (int y = 0; y < 4; ++y) acc[0][y] = acc[1][y] = 0.0f;
+      for (int i0 = 0; i0 < p; i0 += 32) {
+        float k[4];
 #pragma unroll
-        for (int y = 0; y < 4; ++y) acc[u][y] = 0.0f;
-      for (int i = 0; i < p; i += 4) {
-        float4 kv[4];
+        for (int y = 0; y < 4; ++y) {
+          const float* col = KT + (size_t)min(j0 + y, p - 1) * ldk;
+          k[y] = i0 + lane < p ? col[i0 + lane] : 0.0f;
+        }
+        const int ni = min(32, p - i0);
+        const float* row = X + (size_t)i0 * ldx + r0 + lane;
+#pragma unroll 4
+        for (int i = 0; i < ni; ++i) {
+          const float w0 = in0 ? row[0] : 0.0f, w1 = in1 ? row[32] : 0.0f;
+          row += ldx;
 #pragma unroll
-        for (int y = 0; y < 4; ++y) kv[y] = *reinterpret_cast<const float4*>(KT + (size_t)min(j0 + y, p - 1) * ldk + i);
-#pragma unroll
-        for (int z = 0; z < 4; ++z) {
-          const float* col = X + (size_t)min(i + z, p - 1) * ldx + r0 + lane;   // K's padding is 0
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-            if (u < nu) {
-              const float w = r0 + lane + 32 * u < n ? col[32 * u] : 0.0f;
-#pragma unroll
-              for (int y = 0; y < 4; ++y) {
-                const float kz = z == 0 ? kv[y].x : (z == 1 ? kv[y].y : (z == 2 ? kv[y].z : kv[y].w));
-                acc[u][y] = fmaf(w, kz, acc[u][y]);
-              }
-            }
+          for (int y = 0; y < 4; ++y) {
+            const float kz = blk::lane_value(k[y], i);
+            acc[0][y] = fmaf(w0, kz, acc[0][y]);
+            acc[1][y] = fmaf(w1, kz, acc[1][y]);
+          }
         }
       }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int r = r0 + lane + 32 * u;
-        if (u >= nu || r >= n) continue;
+#pragma unroll 1
+      for (int u = 0; u < 2; ++u) {
+        const int r = r0 + 32 * u + lane;
+        if (r >= n) break;
 #pragma unroll
         for (int y = 0; y < 4; ++y)
           if (j0 + y < p) {
             double* o = out + (size_t)(j0 + y) * ldo + r;
-            *o = ADD ? *o + blk::widen(acc[u][y]) : corrected(X[(size_t)(j0 + y) * ldx + r], acc[u][y]);
+            const float c = u ? acc[1][y] : acc[0][y];
+            *o = ADD ? *o + blk::widen(c) : corrected(X[(size_t)(j0 + y) * ldx + r], c);
           }
       }
     }
