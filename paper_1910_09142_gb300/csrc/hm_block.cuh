@@ -421,21 +421,26 @@ __device__ __forceinline__ void share(const Team& tm, int n, int& c0, F&& f) {
 // charge absent from the middle bond are written as 0.  A, B are binary64
 // site tensors; T is the accumulation and storage type of theta.
 //
-// Two forms.  Direct: a warp takes 4 rows x 32 columns of a block and reads
-// both operands through L1, all blocks at once, no barrier.  Binary64 always
-// takes it: its pipe (16 clocks a warp instruction) hides the two loads a
-// product costs, and a padded tile would be charged in full.  Binary32 takes it
-// while the split has at most kThetaDirect products; above, the CTA goes
-// through the blocks in TM x TN x TK tiles in shared memory, which convert and
-// load each operand once per tile instead of once per product.
+// Two forms.  Direct: a warp takes R rows x 32 columns of a block and reads both
+// operands through L1, all blocks at once, no barrier.  Binary64 always takes
+// it: its pipe (16 clocks a warp instruction) hides the loads, and a padded
+// tile would be charged in full.  Binary32 takes it while the split has at most
+// kThetaDirect products; there a conversion costs as much as several products,
+// so A's entries are loaded and converted 32 at a time, one a lane, and handed
+// round by shuffles.  Above, the CTA goes through the blocks in TM x TN x TK
+// tiles in shared memory, which load and convert each operand once per tile.
 #ifndef HM_THETA_DIRECT
-#define HM_THETA_DIRECT 131072.0
+#define HM_THETA_DIRECT 262144.0
 #endif
 constexpr double kThetaDirect = HM_THETA_DIRECT;
 
 template <int NT, typename T>
 __device__ void theta_direct(const ChainDev* c, int k, const SplitSh& s, T* __restrict__ theta, const Team& tm) {
-  constexpr int R = 4;
+  constexpr bool F32 = sizeof(T) < sizeof(double);
+  constexpr int R = F32 ? 8 : 4;
+  const int lane = threadIdx.x & 31;
+  const unsigned nw = NT / 32 * tm.size;           // a power of two
+  const int warp = (threadIdx.x >> 5) + NT / 32 * tm.rank;
   const int chim = c->chi[k + 1], chir = c->chi[k + 2];
   const int n = 3 * chir;
   const double* A = c->site[k];
@@ -444,38 +449,52 @@ __device__ void theta_direct(const ChainDev* c, int k, const SplitSh& s, T* __re
   for (int bi = 0; bi < s.nin; ++bi) {
     const InRec& r = s.in[bi];
     const int Mv = r.roff[3], Nv = r.coff[3], K = r.mlen, mst = r.mst;
-    const int nu = (Nv + 31) >> 5;
-    // one element a lane: (row group, column), columns padded to whole warps
-    share<NT>(tm, ((Mv + R - 1) / R) * nu * 32, c0, [&](int e) {
-      const int g = e / (nu * 32), u = e - g * nu * 32;
-      const int uu = u < Nv ? u : Nv - 1;
+    const int nu = (Nv + 31) >> 5, tasks = ((Mv + R - 1) / R) * nu;
+    for (int x = (unsigned)(warp - c0) & (nw - 1); x < tasks; x += nw) {
+      const int g = x / nu, u = (x - g * nu) * 32 + lane;
+      const int uu = min(u, Nv - 1);
       const int t2 = uu >= r.coff[2] ? 2 : (uu >= r.coff[1] ? 1 : 0);
       const int col = t2 * chir + r.cst[t2] + uu - r.coff[t2];
       const double* b = B + (size_t)mst * n + col;
-      const double* a[R];
+      const int nr = min(R, Mv - g * R);
       int row[R];
       T acc[R];
 #pragma unroll
-      for (int x = 0; x < R; ++x) {
-        const int v = min(g * R + x, Mv - 1);
+      for (int y = 0; y < R; ++y) {
+        const int v = min(g * R + y, Mv - 1);
         const int t = v >= r.roff[2] ? 2 : (v >= r.roff[1] ? 1 : 0);
-        row[x] = 3 * (r.rst[t] + v - r.roff[t]) + t;
-        a[x] = A + (size_t)row[x] * chim + mst;
-        acc[x] = T(0);
+        row[y] = 3 * (r.rst[t] + v - r.roff[t]) + t;
+        acc[y] = T(0);
       }
-      const int nr = min(R, Mv - g * R);
-#pragma unroll 2
-      for (int kk = 0; kk < K; ++kk) {
-        const T bv = from64<T>(b[(size_t)kk * n]);
+      if constexpr (F32) {
+        for (int k0 = 0; k0 < K; k0 += 32) {
+          const int kn = min(32, K - k0);
+          T av[R];
 #pragma unroll
-        for (int x = 0; x < R; ++x)
-          if (x < nr) acc[x] = fma(from64<T>(a[x][kk]), bv, acc[x]);
+          for (int y = 0; y < R; ++y)
+            av[y] = lane < kn ? from64<T>(A[(size_t)row[y] * chim + mst + k0 + lane]) : T(0);
+#pragma unroll 2
+          for (int kk = 0; kk < kn; ++kk) {
+            const T bv = from64<T>(b[(size_t)(k0 + kk) * n]);
+#pragma unroll
+            for (int y = 0; y < R; ++y) acc[y] = fma(lane_value(av[y], kk), bv, acc[y]);
+          }
+        }
+      } else {
+#pragma unroll 4
+        for (int kk = 0; kk < K; ++kk) {
+          const double bv = b[(size_t)kk * n];
+#pragma unroll
+          for (int y = 0; y < R; ++y)
+            if (y < nr) acc[y] = fma(A[(size_t)row[y] * chim + mst + kk], bv, acc[y]);
+        }
       }
       if (u < Nv)
 #pragma unroll
-        for (int x = 0; x < R; ++x)
-          if (x < nr) theta[(size_t)row[x] * n + col] = acc[x];
-    });
+        for (int y = 0; y < R; ++y)
+          if (y < nr) theta[(size_t)row[y] * n + col] = acc[y];
+    }
+    c0 += tasks;
   }
   team_sync(tm);
 }
