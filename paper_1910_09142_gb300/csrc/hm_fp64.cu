@@ -667,11 +667,11 @@ __global__ void __launch_bounds__(NT) measure_fp64_kernel(BatchArg b, OutArg o) 
   // A chain in frame 1 stores R^N |psi> (R exchanges S^x and S^z, R S^z R =
   // S^x): there <Sz_i Sz_j> of |psi> is <Sx_i Sx_j> of the stored state,
   // which for a state of definite total S^z is (<S+_i S-_j> + <S-_i S+_j>)/4;
-  // S_i.S_j is invariant.  Passes: (Sz Sz), (S+ S-), (S- S+); operator
-  // charge shifts dO = 0, +1, -1 and -dO.
+  // S_i.S_j is invariant.  Passes: (Sz Sz) and (S+ S-); the tensors are real,
+  // so <S-_i S+_j>, the adjoint of <S+_i S-_j>, is the same number.
   const int frame = c->counters[2];
-  const tr::Op1 ops1[3] = {tr::op_sz(), tr::op_sp(), tr::op_sm()};
-  const tr::Op1 ops2[3] = {tr::op_sz(), tr::op_sm(), tr::op_sp()};
+  const tr::Op1 ops1[2] = {tr::op_sz(), tr::op_sp()};
+  const tr::Op1 ops2[2] = {tr::op_sz(), tr::op_sm()};
   int bi = 0;
   while (bi < c->n_meas) {
     const int a = c->meas_i[bi];
@@ -683,8 +683,8 @@ __global__ void __launch_bounds__(NT) measure_fp64_kernel(BatchArg b, OutArg o) 
       cur ^= 1;
       ++pos;
     }
-    double vals[3][8];   // up to 8 bonds per start site
-    for (int o1 = 0; o1 < 3; ++o1) {
+    double vals[2][8];   // up to 8 bonds per start site
+    for (int o1 = 0; o1 < 2; ++o1) {
       int ec = 0;
       int D = tr::left_transfer<NT>(c, a, Lp[cur], 0, ops1[o1], Ep[ec], Z, false, false, sh.tab, fma_n);
       for (int kk = a + 1; kk <= blast; ++kk) {
@@ -705,7 +705,7 @@ __global__ void __launch_bounds__(NT) measure_fp64_kernel(BatchArg b, OutArg o) 
     }
     if (tid == 0) {
       for (int q = bi; q < bend; ++q) {
-        const double pm = (vals[1][q - bi] + vals[2][q - bi]) / nrm;
+        const double pm = 2.0 * vals[1][q - bi] / nrm;
         const double ss = vals[0][q - bi] / nrm + 0.5 * pm;
         const double zz = frame ? 0.25 * pm : vals[0][q - bi] / nrm;
         out[1 + 2 * q] = ss;
@@ -724,11 +724,12 @@ __global__ void __launch_bounds__(NT) measure_fp64_kernel(BatchArg b, OutArg o) 
 // Uniform susceptibility (Eq. sus, Sec. II.A): the double sum
 // sum_{a in M} sum_{b physical} <S_a . S_b> / <psi|psi>, written to o.obs[chain].
 // A right sweep carries the plain right environment R and the running sums
-// R_z, R_-, R_+ of right environments with S^z, S^-, S^+ inserted on every
-// physical site to the right, and keeps all four at each region site a
-// (R(a+1)); a left sweep carries the mirrored sums L, L_z, L_+, L_- and
-// closes, at each region site a, O_a on L against the right sums (b > a)
-// and the left sums with O_a against R (b < a).  Linear in the chain length.
+// R_z, R_- of right environments with S^z, S^- inserted on every physical site
+// to the right, and keeps all three at each region site a (R(a+1)); a left
+// sweep carries the mirrored sums L, L_z, L_+ and closes, at each region site
+// a, O_a on L against the right sums (b > a) and the left sums with O_a against R
+// (b < a).  The tensors are real, so <S-_a S+_b>, the adjoint of <S+_a S-_b>, is
+// the same number and takes no sums of its own.  Linear in the chain length.
 // Charge blocks throughout: S^z leaves an environment's shift at 0, S^+ and
 // S^- move it by the sign of the physical legs.  A chain whose physical
 // positions hold legs of different signs (explicit op lists can leave it so)
@@ -743,11 +744,12 @@ __global__ void __launch_bounds__(NT) susceptibility_fp64_kernel(BatchArg b, Out
     return;
   }
   const int64_t cc = (int64_t)c->chi_cap * c->chi_cap;
-  double* Rc[4];
-  double* Rn[4];
-  double* Lc[4];
-  double* Ln[4];
-  for (int qq = 0; qq < 4; ++qq) {
+  constexpr int NE = 3;                    // plain, S^z, S^- (right) or S^+ (left)
+  double* Rc[NE];
+  double* Rn[NE];
+  double* Lc[NE];
+  double* Ln[NE];
+  for (int qq = 0; qq < NE; ++qq) {
     Rc[qq] = c->env_ws + qq * cc;
     Rn[qq] = c->env_ws + (4 + qq) * cc;
     Lc[qq] = c->env_ws + (8 + qq) * cc;
@@ -756,9 +758,8 @@ __global__ void __launch_bounds__(NT) susceptibility_fp64_kernel(BatchArg b, Out
   double* Z = c->env_ws + 16 * cc;         // 3 cc
   double* Et = c->env_ws + 19 * cc;
   double* store = c->env_ws + 20 * cc;     // 4 cc per region site
-  // right sums carry S^z, S^-, S^+ ; left sums carry S^z, S^+, S^-
-  const tr::Op1 ropk[4] = {tr::op_id(), tr::op_sz(), tr::op_sm(), tr::op_sp()};
-  const tr::Op1 lopk[4] = {tr::op_id(), tr::op_sz(), tr::op_sp(), tr::op_sm()};
+  const tr::Op1 ropk[NE] = {tr::op_id(), tr::op_sz(), tr::op_sm()};
+  const tr::Op1 lopk[NE] = {tr::op_id(), tr::op_sz(), tr::op_sp()};
   // the one sign of the physical legs; dense when there is none
   int leg = 0;
   bool dense = false;
@@ -769,14 +770,14 @@ __global__ void __launch_bounds__(NT) susceptibility_fp64_kernel(BatchArg b, Out
   }
   if (dense) leg = 0;
   // shifts of the right sums (bra minus ket charge) and of the left ones
-  const int rD[4] = {0, 0, leg, -leg};
-  const int lD[4] = {0, 0, leg, -leg};
+  const int rD[NE] = {0, 0, leg};
+  const int lD[NE] = {0, 0, leg};
   long long fma_n = 0;
   if (tid == 0) {
     Rc[0][0] = 1.0;
-    Rc[1][0] = Rc[2][0] = Rc[3][0] = 0.0;
+    Rc[1][0] = Rc[2][0] = 0.0;
     Lc[0][0] = 1.0;
-    Lc[1][0] = Lc[2][0] = Lc[3][0] = 0.0;
+    Lc[1][0] = Lc[2][0] = 0.0;
   }
   __syncthreads();
   const int n = c->n_sites;
@@ -788,16 +789,16 @@ __global__ void __launch_bounds__(NT) susceptibility_fp64_kernel(BatchArg b, Out
     for (int s2 = 0; s2 < c->n_region; ++s2)
       if (c->region[s2] == pos) slot = s2;
     if (slot >= 0) {
-      for (int qq = 0; qq < 4; ++qq)
+      for (int qq = 0; qq < NE; ++qq)
         for (int e = tid; e < cr * cr; e += NT) store[(size_t)(4 * slot + qq) * cc + e] = Rc[qq][e];
       __syncthreads();
     }
     const bool phys = c->site_kind[pos] != SITE_ANC;
-    for (int qq = 0; qq < 4; ++qq) {
+    for (int qq = 0; qq < NE; ++qq) {
       tr::right_transfer<NT>(c, pos, Rc[qq], rD[qq], tr::op_id(), Rn[qq], Z, false, dense, sh.tab, fma_n);
       if (qq > 0 && phys) tr::right_transfer<NT>(c, pos, Rc[0], 0, ropk[qq], Rn[qq], Z, true, dense, sh.tab, fma_n);
     }
-    for (int qq = 0; qq < 4; ++qq) {
+    for (int qq = 0; qq < NE; ++qq) {
       double* t = Rc[qq];
       Rc[qq] = Rn[qq];
       Rn[qq] = t;
@@ -814,25 +815,24 @@ __global__ void __launch_bounds__(NT) susceptibility_fp64_kernel(BatchArg b, Out
       const double* R0 = store + (size_t)(4 * slot) * cc;
       const double* Rz = R0 + cc;
       const double* Rm = R0 + 2 * cc;
-      const double* Rp = R0 + 3 * cc;
       // b > a: O_a on L, closed against the right sums; b < a: the left sums
       // with O_a, closed against R
-      const tr::Op1 oa[6] = {tr::op_sz(), tr::op_sp(), tr::op_sm(), tr::op_sz(), tr::op_sm(), tr::op_sp()};
-      const double* right[6] = {Rz, Rm, Rp, R0, R0, R0};
-      for (int u = 0; u < 6; ++u) {
-        const int from = u < 3 ? 0 : u - 2;
+      const tr::Op1 oa[4] = {tr::op_sz(), tr::op_sp(), tr::op_sz(), tr::op_sm()};
+      const double* right[4] = {Rz, Rm, R0, R0};
+      for (int u = 0; u < 4; ++u) {
+        const int from = u < 2 ? 0 : u - 1;
         const int D = tr::left_transfer<NT>(c, pos, Lc[from], lD[from], oa[u], Et, Z, false, dense, sh.tab, fma_n);
-        total += (u % 3 == 0 ? 1.0 : 0.5) * tr::block_dot<NT>(sh.tab, D, Et, right[u], cr, sh.red);
+        total += tr::block_dot<NT>(sh.tab, D, Et, right[u], cr, sh.red);
       }
       total += 2.0 * nrm;                  // b = a: S.S = s(s+1) = 2
     }
     if (pos == amax) break;
     const bool phys = c->site_kind[pos] != SITE_ANC;
-    for (int qq = 0; qq < 4; ++qq) {
+    for (int qq = 0; qq < NE; ++qq) {
       tr::left_transfer<NT>(c, pos, Lc[qq], lD[qq], tr::op_id(), Ln[qq], Z, false, dense, sh.tab, fma_n);
       if (qq > 0 && phys) tr::left_transfer<NT>(c, pos, Lc[0], 0, lopk[qq], Ln[qq], Z, true, dense, sh.tab, fma_n);
     }
-    for (int qq = 0; qq < 4; ++qq) {
+    for (int qq = 0; qq < NE; ++qq) {
       double* t = Lc[qq];
       Lc[qq] = Ln[qq];
       Ln[qq] = t;
