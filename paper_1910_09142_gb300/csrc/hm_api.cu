@@ -1144,6 +1144,24 @@ int hm_get_mps(hm_ctx* ctx, hm_chain chain, int32_t* dims_out, int32_t dims_cap,
     HM_CUDA(ctx, cudaMemcpy(buf + o, base + c->mp.slot_off[s], sz * sizeof(double), cudaMemcpyDeviceToHost));
     o += sz;
   }
+  {
+    // a split writes only the entries its charges allow; the others are zero
+    const int cap = (int)c->mp.chi_cap;
+    std::vector<int16_t> qn((size_t)(n + 1) * cap);
+    std::vector<int32_t> sgn(n);
+    HM_CUDA(ctx, cudaMemcpy(qn.data(), base + c->mp.off_qn, qn.size() * sizeof(int16_t), cudaMemcpyDeviceToHost));
+    HM_CUDA(ctx, cudaMemcpy(sgn.data(), base + c->mp.off_sgn, n * sizeof(int32_t), cudaMemcpyDeviceToHost));
+    o = 0;
+    for (int s = 0; s < n; ++s) {
+      const int cl = dims_out[s], cr = dims_out[s + 1];
+      const int16_t* qL = &qn[(size_t)s * cap];
+      const int16_t* qR = qL + cap;
+      for (int l = 0; l < cl; ++l)
+        for (int m = 0; m < 3; ++m, o += cr)
+          for (int x = 0; x < cr; ++x)
+            if (qL[l] + sgn[s] * (1 - m) != qR[x]) buf[o + x] = 0.0;
+    }
+  }
   int32_t cnt[4];
   HM_CUDA(ctx, cudaMemcpy(cnt, base + c->mp.off_cnt, sizeof cnt, cudaMemcpyDeviceToHost));
   if (cnt[2] == 1) {

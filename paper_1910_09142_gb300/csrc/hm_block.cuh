@@ -22,10 +22,10 @@
 // runs, one per local state.  A chain in dense mode (every charge and sign 0)
 // has a single block: the unblocked split.
 //
-// Entries outside the blocks are never computed: the block GEMMs write only
-// entries whose row and column charges agree, the gate is applied only
-// within its conserved sectors, and the absorb writes explicit zeros.  So the
-// structure holds exactly, in any precision.
+// Entries outside the blocks are never computed, written or read: the block
+// GEMMs write only entries whose row and column charges agree, the gate is
+// applied only within its conserved sectors, and the absorb writes the blocks
+// alone (clear_forbidden).  So the structure holds exactly, in any precision.
 #pragma once
 
 #include <cstdint>
@@ -186,11 +186,31 @@ __device__ __forceinline__ float from64<float>(double d) {
   return narrow(d);
 }
 
+// Zeros in the entries of every site tensor that its charges forbid.  A split
+// writes only the allowed entries (finish) and every kernel reads only those,
+// so the others hold whatever an earlier, differently shaped tensor left in the
+// slot; whoever wants the full tensors clears them first.
+template <int NT>
+__device__ void clear_forbidden(ChainDev* c) {
+  for (int k = 0; k < c->n_sites; ++k) {
+    const int cl = c->chi[k], cr = c->chi[k + 1], sg = c->sgn[k];
+    const int16_t* qL = c->qn + (size_t)k * c->chi_cap;
+    const int16_t* qR = qL + c->chi_cap;
+    double* A = c->site[k];
+    for (int e = threadIdx.x; e < cl * 3 * cr; e += NT) {
+      const int row = e / cr, r = e - row * cr, l = row / 3;
+      if (qL[l] + sg * mval(row - 3 * l) != qR[r]) A[e] = 0.0;
+    }
+  }
+  __syncthreads();
+}
+
 // Marks a chain as having no usable charge structure from here on: every
 // charge and sign 0 (one block per split).  Sec. II.C's blocking is an
 // optimisation; the dense split computes the same decomposition.
 template <int NT>
 __device__ void go_dense(ChainDev* c) {
+  clear_forbidden<NT>(c);
   const int nb = (c->n_sites + 1) * c->chi_cap;
   for (int e = threadIdx.x; e < nb; e += NT) c->qn[e] = 0;
   for (int e = threadIdx.x; e < c->n_sites; e += NT) c->sgn[e] = 0;
@@ -1534,16 +1554,17 @@ __device__ inline int warp_trunc_rank(const double* s, int n, int chi_max, doubl
 // Phase D: singular values of every block (column norms of its converged W,
 // binary64), one descending order over all blocks, the truncation rule,
 // renormalisation, then the new bond grouped by charge (ascending; by value
-// within a charge), the absorb into A_k and A_{k+1} (zeros outside the
-// blocks) and the new middle charges.  W and V hold every block's binary64
+// within a charge), the absorb into A_k and A_{k+1} (the blocks only) and the
+// new middle charges.  W and V hold every block's binary64
 // result.  scratch: finish_bytes(P) bytes; tiles: per warp 8 x 33 doubles of
 // shared memory (the transposition of the left factor).
 //
 // The binary64 pipe and dependent loads bound this phase, not its traffic: the
 // order compares integer keys, the truncation sums run over a warp, a kept
-// value's scales cost one divide each (not one per element), and the absorb
-// goes block by block, after a plain zero fill, instead of looking up each
-// element's block.
+// value's scales cost one divide each (not one per element), the absorb goes
+// block by block instead of looking up each element's block, and it writes the
+// blocks only: zeros around them were four fifths of its writes (two tensors
+// of 3 chi^2 doubles a split).
 template <int NT>
 __device__ void finish(ChainDev* c, const OpDev& op, int t, SplitSh& s, const WaveSh& wv, const Team& tm,
                        char* __restrict__ scratch, double* tiles, int32_t* ctx_err, int sweeps32, int sweeps64) {
@@ -1567,15 +1588,19 @@ __device__ void finish(ChainDev* c, const OpDev& op, int t, SplitSh& s, const Wa
     for (int i = 0; i < wv.nown; ++i) {
       const BlockRec& r = s.b[own_block(wv, i)];
       const double* Wb = c->W + r.woff;
-      for (int j = (unsigned)(warp - c0) % NW; j < r.p; j += NW) {
-        const double* cj = Wb + (size_t)j * r.q;
+      // four columns a warp, eight lanes each
+      const int nj = (r.p + 3) >> 2;
+      for (int x = (unsigned)(warp - c0) % NW; x < nj; x += NW) {
+        const int j = 4 * x + (lane >> 3);
+        const double* cj = Wb + (size_t)min(j, r.p - 1) * r.q;
         double s2 = 0.0;
 #pragma unroll 4
-        for (int e = lane; e < r.q; e += 32) s2 = fma(cj[e], cj[e], s2);
-        s2 = warp_sum64(s2);
-        if (lane == 0) c->sig[r.svoff + j] = sqrt(s2);
+        for (int e = lane & 7; e < r.q; e += 8) s2 = fma(cj[e], cj[e], s2);
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+        if ((lane & 7) == 0 && j < r.p) c->sig[r.svoff + j] = sqrt(s2);
       }
-      c0 += r.p;
+      c0 += nj;
     }
   }
   team_sync(tm);                          // every block's W, V and values are there
@@ -1650,16 +1675,7 @@ __device__ void finish(ChainDev* c, const OpDev& op, int t, SplitSh& s, const Wa
   // new position of kept rank i: kept values of lower-charge blocks first,
   // then by rank within the block
   for (int i = tid; i < kk; i += NT) key[i] = sblk[perm[i]] * 16384 + i;
-  // zeros everywhere (site slots are 256-byte aligned)
-  for (int h = 0; h < 2; ++h) {
-    double* A = h ? Ak1 : Ak;
-    const int tot = h ? kk * n : m * kk;
-    double2* A2 = reinterpret_cast<double2*>(A);
-    const double2 z = {0.0, 0.0};
-    for (int e = tid + NT * tm.rank; e < tot / 2; e += NT * tm.size) A2[e] = z;
-    if ((tot & 1) && tid == 0 && tm.rank == 0) A[tot - 1] = 0.0;
-  }
-  team_sync(tm);
+  __syncthreads();
   const bool absorb_left = op.absorb == 0;
   int16_t* qM = c->qn + (size_t)(k + 1) * c->chi_cap;
   for (int i = tid; i < kk; i += NT) {

@@ -768,7 +768,10 @@ __global__ void __launch_bounds__(NT) susceptibility_fp64_kernel(BatchArg b, Out
     if (leg == 0) leg = c->sgn[pos];
     if (c->sgn[pos] != leg || leg == 0) dense = true;
   }
-  if (dense) leg = 0;
+  if (dense) {
+    leg = 0;
+    blk::clear_forbidden<NT>(c);
+  }
   // shifts of the right sums (bra minus ket charge) and of the left ones
   const int rD[NE] = {0, 0, leg};
   const int lD[NE] = {0, 0, leg};

@@ -3,8 +3,7 @@
 //
 // A chain's ops are serial, but the charge blocks of one split are not: a team
 // shares out theta's tiles, the blocks (each decomposed by one CTA, the
-// costliest first), the zero fill and the absorb, and meets at four cluster
-// barriers an op.  Everything a CTA needs from another goes through the chain's
+// costliest first) and the absorb, and meets at three cluster barriers an op.  Everything a CTA needs from another goes through the chain's
 // own buffers in global memory.  A Markov step, one CTA -> a team: 4 chains of Lx = 4, 2W =
 // 4, binary64, 206 -> 113 ms (8 CTAs); 8 mixed chains of Lx = 4, 30.4 -> 22.4
 // ms (8); one METTS chain of small blocks, 22.1 -> 20.4 ms (8).

@@ -162,3 +162,40 @@ def test_records_in_the_workspace_and_tiled_theta(tmp_path, prec):
     assert np.abs(obs - r["obs"]).max() <= tol * max(1.0, np.abs(r["obs"]).max())
     assert env == r["env_out"] and abs(lp - r["logp"]) < 10 * tol
     e.close()
+
+
+@pytest.mark.parametrize("prec", ["HM_FP64", "HM_MIXED"])
+def test_nothing_is_read_that_was_not_written(emu, prec):
+    """A split writes only the entries its charges allow.  With an arena full
+    of NaN the state, susceptibility, observables, outcomes and log p of two
+    samples are the bits they are with an arena of zeros."""
+    P, vp, i32, i64 = ctypes.POINTER, ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64
+    for name, args in {"hm_create": [P(vp), ctypes.c_int, vp, ctypes.c_size_t, vp], "hm_destroy": [vp],
+                       "hm_init_chain": [vp, P(binding.Params), vp, P(i64)], "hm_evolve": [vp, P(i64), i32],
+                       "hm_measure_cluster": [vp, P(i64), i32, vp, i32], "hm_collapse": [vp, P(i64), i32, vp, vp],
+                       "hm_measure_susceptibility": [vp, P(i64), i32, vp],
+                       "hm_get_mps": [vp, i64, P(i32), i32, vp, ctypes.c_size_t, P(i32), P(ctypes.c_size_t)],
+                       "hm_last_error": [vp]}.items():
+        getattr(emu, name).argtypes = args
+    emu.hm_last_error.restype = ctypes.c_char_p
+    cfg = dict(Lx=3, two_W=2, J_leg=1.0, J_rung=0.7, beta=0.2, tau=0.1, chi_max=20, cutoff=1e-10)
+    p = binding.params(**cfg, seed=4, chain_id=2, precision=getattr(binding, prec))
+    runs = []
+    for byte in (0, 255):
+        e = Emu(emu)
+        base = -e.mem.ctypes.data % 256
+        e.mem[base + 256:] = byte                 # the context's error word lies in front
+        cid = e.init(p)
+        got = []
+        for _ in range(2):
+            e.evolve(cid)
+            got += [t.copy() for t in e.mps(cid)]
+            chi = np.zeros(2)
+            e._ok(emu.hm_measure_susceptibility(e.h, e._ids(cid), 1, _ptr(chi)))
+            env, lp = None, None
+            got += [chi, e.measure(cid, p)]
+            env, lp = e.collapse(cid, p)
+            got += [np.array(env), np.array(lp)]
+        runs.append(got)
+        e.close()
+    assert all(np.isfinite(x).all() and np.array_equal(x, y) for x, y in zip(*runs))

@@ -117,3 +117,33 @@ def test_legs_out_of_place(emu):  # noqa: F811
     chi, raw = omeasure.susceptibility(st, ref.ladder, _region(ref), cfg["beta"])
     assert _close(_chi(e, emu, cid), [chi, raw])
     e.close()
+
+
+@pytest.mark.parametrize("prec", ["HM_FP64", "HM_MIXED"])
+def test_a_gate_that_breaks_the_labels(emu, prec):  # noqa: F811
+    """A bond gate on a cluster site and its ancilla breaks the charge rule: the
+    chain drops its labels first, and its tensors' forbidden entries, which
+    no split wrote, have to be zeros by then.  The arena starts full of NaN."""
+    from oracle import model
+    cfg = dict(BASE, Lx=3, two_W=2, beta=0.2, chi_max=24)
+    e = Emu(emu)
+    e.mem[-e.mem.ctypes.data % 256 + 256:] = 255        # behind the context's error word
+    p = binding.params(**cfg, seed=2, chain_id=3, precision=getattr(binding, prec))
+    cid = e.init(p)
+    ref = ochain.HybridChain(seed=2, chain_id=3, **cfg)
+    e.evolve(cid)
+    before = [t.copy() for t in e.mps(cid)]
+    site = ref.ladder.cluster_sites[0]
+    ops = np.array([[k, 0, 1, 1] for k in range(site)] + [[site, 2, 0, 0]] +
+                   [[k, 0, 0, 1] for k in range(site - 1, -1, -1)], dtype=np.int32)
+    emu.hm_apply_ops.argtypes = [ctypes.c_void_p, ctypes.c_int64, ctypes.c_void_p, ctypes.c_int32]
+    e._ok(emu.hm_apply_ops(e.h, cid, ops.ctypes.data_as(ctypes.c_void_p), len(ops)))
+    st = omps.MPS(before, 0)
+    for k in range(site):
+        omps.move_right(st, k)
+    omps.split(st, site, model.bond_gate(0.5 * 0.1 * 0.7), model.ABSORB_L, 24, 1e-12)   # tau / 2 on a rung
+    for k in range(site, 0, -1):
+        omps.move_left(st, k)
+    a, b = omps.MPS(e.mps(cid)).to_dense(), st.to_dense()
+    assert np.abs(a - np.sign(a @ b) * b).max() < (1e-10 if prec == "HM_FP64" else 1e-5)
+    e.close()
