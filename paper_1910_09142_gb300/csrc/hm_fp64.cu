@@ -1,15 +1,14 @@
 // FP64 path of the hybrid purification-METTS sampler (arXiv:1910.09142).
 //
-// One CTA owns one Markov chain for the whole call: every two-site op of the
-// Trotter schedule, the cluster measurement and the environment collapse run
-// as a device-side loop over that chain's data.  On GB300 the binary64 pipe
-// (about 2 DFMA per clock per SM) is the bound of every step here, so the
-// design keeps all SMs busy with independent chains rather than tiling for
-// bandwidth: a batch of >= 152 chains fills the chip.
+// One CTA (in small batches of an evolution a cluster, hm_team.h) owns one
+// Markov chain for the whole call: every two-site op of the Trotter schedule,
+// the cluster measurement and the environment collapse run as a device-side
+// loop over that chain's data.  On GB300 the binary64 pipe (about 2 DFMA per
+// clock per SM) is the scarce unit of every step here.
 //
 // Steps (Sec. I.C.1): evolve (step 2) = theta GEMM + 9x9 gate + one-sided
-// Jacobi SVD + truncation (Sec. II) + absorb, all in S^z charge blocks
-// (Sec. II.C, hm_block.cuh); measure (step 3) = transfer matrices with S^z /
+// Jacobi SVD (found in binary32, finished in binary64) + truncation (Sec. II) +
+// absorb, all in S^z charge blocks (Sec. II.C, hm_block.cuh); measure (step 3) = transfer matrices with S^z /
 // S^+ / S^- insertions (Eq. H), contracted by charge block; collapse + reset
 // (step 4, Eq. detailbalance1, Bell pairs of Sec. I.C), the reset writing the
 // next initial state with its charges.  An S^x-basis sample is stored with

@@ -7,17 +7,17 @@
 // each block so that the singular values and left vectors become
 // binary64-accurate for that tensor (hm_refine.cuh: one first-order sweep as a
 // product, binary64 rotations where that does not hold); HM_MIXED32 stops at
-// the binary32 sweeps.  The truncation weights (Sec. II), the renormalisation of the kept
-// singular values and the stored site tensors stay binary64.  Measurement
-// and collapse (steps 3-4) are the binary64 kernels of hm_fp64.cu.
+// the binary32 sweeps.  The truncation weights (Sec. II), the renormalisation
+// of the kept singular values and the stored site tensors stay binary64.
+// Measurement and collapse (steps 3-4) are the binary64 kernels of hm_fp64.cu.
 //
-// One CTA owns one chain: 512 threads, one CTA per SM, or (hm_mixed_pair.cu)
-// 256 threads, two CTAs per SM, for batches wider than the GPU.  The blocks
-// of a split that fit in shared memory together form a wave and are
-// decomposed at once, each by its own warp group; a block too large for
-// shared memory keeps W and V in global memory and works on pairs of column
-// blocks staged in shared memory (intra-block pairs once per sweep, then
-// every cross pair of two staged blocks).
+// A chain has one CTA of 512 threads on an SM of its own, a cluster of such CTAs
+// in small batches (hm_team.h), or (hm_mixed_pair.cu) half an SM, 256
+// threads, in batches wider than the GPU.  The blocks of a split that fit in
+// shared memory together form a wave and are decomposed at once by warp
+// groups; a block too large for shared memory keeps W and V in global memory
+// and works on pairs of column blocks staged in shared memory (intra-block
+// pairs once per sweep, then every cross pair of two staged blocks).
 #include <cuda_runtime.h>
 
 #include <cfloat>
@@ -392,6 +392,11 @@ __device__ void promote_v(const float* V32, int ldv, int q, int p, double* W64, 
 // memory is at least this (and at least the staged fallback's plan).  Two
 // CTAs per SM share the SM's 228 KB.
 constexpr size_t kBlockSmem = kCtasPerSm == 1 ? 210 * 1024 : kPairBlockSmem;
+// Of it, what the blocks of a wave may take.
+#ifndef HM_WAVE_SMEM
+#define HM_WAVE_SMEM kBlockSmem
+#endif
+constexpr size_t kWaveSmem = HM_WAVE_SMEM;
 constexpr int kTileDoubles = NT / 32 * 8 * 33;   // finish()'s transposition tiles
 static_assert(sizeof(blk::PrepTab) <= kBlockSmem, "prepare's tables");
 
@@ -530,7 +535,7 @@ __device__ void two_site_op_mixed(ChainDev* c, const OpDev op, int t, int bcols,
   blk::theta_blocks<NT, GM, GN, GK, float>(c, op.k, ss, theta, smem, tm);
   int sw32 = 0, sw64 = 0;
   int64_t cost = -1;
-  constexpr int64_t cap = (int64_t)(kBlockSmem / sizeof(float));
+  constexpr int64_t cap = (int64_t)(kWaveSmem / sizeof(float));
   if (tid == 0) blk::own_blocks(ss, tm, wv, [&](int q, int p) { return block_floats(q, p) <= cap; });
   __syncthreads();
   const int nown = wv.nown;
@@ -643,11 +648,24 @@ __global__ void __launch_bounds__(NT, kCtasPerSm) evolve_mixed_kernel(BatchArg b
   }
 }
 
+// Dynamic shared memory the staged path may plan for: what one CTA may opt into
+// less the kernel's static shared memory.
+#ifndef HM_STAGED_SMEM
+#define HM_STAGED_SMEM (kMaxSharedOptIn - 8 * 1024)
+#endif
+constexpr size_t kStagedSmem = HM_STAGED_SMEM;
+
 // Opt-in to the kernel's dynamic shared memory (per device, cached, under a
 // lock: serving workers may launch from several host threads), then launch.
 int launch_kernel(const BatchArg& b, const OutArg& o, int chi_cap, int polish, void* stream) {
   int bcols = 16;
-  const size_t plan = mixed_smem_bytes(chi_cap, &bcols, kBlockSmem);
+  size_t plan = mixed_smem_bytes(chi_cap, &bcols, kBlockSmem);
+  if (plan > kStagedSmem) {
+    // caps near the admission limit: one column a staged block, so that the
+    // plan fits beside the kernel's static shared memory
+    bcols = 1;
+    plan = (2 * 6 + 3) * (size_t)chi_cap * sizeof(float);
+  }
   const size_t smem = plan > kBlockSmem ? plan : kBlockSmem;
   static std::mutex mu;
   static size_t configured[64] = {};

@@ -138,11 +138,7 @@ def test_orthonormalisation_reaches_binary64(emu, p):
     assert np.abs(V64 - start).max() <= 2e-5
 
 
-@pytest.mark.parametrize("prec", ["HM_FP64", "HM_MIXED", "HM_MIXED32"])
-def test_records_in_the_workspace_and_tiled_theta(tmp_path, prec):
-    """Every split with more records than shared memory holds (limit 2
-    instead of 14), and theta always in tiles: one sample against the oracle."""
-    lib = _build(tmp_path, "#define HM_SH_BLK 2\n#define HM_THETA_DIRECT 0.0\n", ())
+def _check_one_sample(lib, prec):
     P, vp, i32, i64 = ctypes.POINTER, ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64
     lib.hm_create.argtypes = [P(vp), ctypes.c_int, vp, ctypes.c_size_t, vp]
     lib.hm_destroy.argtypes = [vp]
@@ -162,6 +158,23 @@ def test_records_in_the_workspace_and_tiled_theta(tmp_path, prec):
     assert np.abs(obs - r["obs"]).max() <= tol * max(1.0, np.abs(r["obs"]).max())
     assert env == r["env_out"] and abs(lp - r["logp"]) < 10 * tol
     e.close()
+
+
+@pytest.mark.parametrize("prec", ["HM_FP64", "HM_MIXED", "HM_MIXED32"])
+def test_records_in_the_workspace_and_tiled_theta(tmp_path, prec):
+    """Every split with more records than shared memory holds (limit 2
+    instead of 14), and theta always in tiles: one sample against the oracle."""
+    lib = _build(tmp_path, "#define HM_SH_BLK 2\n#define HM_THETA_DIRECT 0.0\n", ())
+    _check_one_sample(lib, prec)
+
+
+@pytest.mark.parametrize("prec,smem", [("HM_MIXED", "kMaxSharedOptIn"), ("HM_MIXED", "0"), ("HM_MIXED32", "0")])
+def test_blocks_beyond_shared_memory(tmp_path, prec, smem):
+    """Every block of two columns or more takes the staged path, with two columns
+    or more a staged block (as for bond caps up to about 2000) or one
+    (above): one sample against the oracle."""
+    lib = _build(tmp_path, "#define HM_WAVE_SMEM 48\n#define HM_STAGED_SMEM %s\n" % smem, ())
+    _check_one_sample(lib, prec)
 
 
 @pytest.mark.parametrize("prec", ["HM_FP64", "HM_MIXED"])
