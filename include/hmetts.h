@@ -38,10 +38,11 @@
  *   the two-site tensor and applies the gate in binary32 (binary64 site
  *   tensors rounded on load, gate coefficients as binary32 hi + lo pairs),
  *   decomposes each charge block with binary32 one-sided Jacobi sweeps, then
- *   finishes with binary64 sweeps so the singular values and vectors are
+ *   finishes it (a first-order sweep from exactly split sums, binary64
+ *   rotations where that does not hold) so the singular values and vectors are
  *   binary64-accurate for that tensor; truncation, renormalisation, stored
  *   tensors, measurement and collapse are binary64.  HM_MIXED32 is HM_MIXED
- *   without the binary64 sweeps.  Measured on GB300 against HM_FP64 (same
+ *   without that finish.  Measured on GB300 against HM_FP64 (same
  *   chains, same draws): per-sample energies within ~1e-6 relative for both
  *   mixed forms (the tests state 1e-5).
  */
@@ -65,7 +66,7 @@ extern "C" {
 
 #define HM_FP64 0            /* every step in binary64                              */
 #define HM_MIXED 1           /* evolve: contraction and gate in binary32, Jacobi SVD */
-                             /* in binary32 then binary64 sweeps; truncation,        */
+                             /* in binary32, then to binary64 accuracy; truncation,  */
                              /* renormalisation, stored tensors, measurement and     */
                              /* collapse in binary64                                 */
 #define HM_MIXED32 2         /* HM_MIXED with the SVD left at its binary32 sweeps    */
@@ -243,11 +244,12 @@ int hm_collapse_conditionals(hm_ctx* ctx, const hm_chain* ids, int32_t n, int8_t
  *     4 M^2 N + 8 M N^2 + 9 N^3 (M >= N) of every charge block,
  * [3] measurement + collapse transfer-matrix flops,
  * [4] sum of discarded weights, [5] largest bond dimension seen,
- * [6] Jacobi sweeps (largest block of each split; binary32 sweeps under
- *     HM_MIXED), [7] two-site splits,
+ * [6] Jacobi sweeps (costliest block of each split; binary32 sweeps under
+ *     HM_MIXED, the binary64 sweeps after the binary32 start under HM_FP64),
+ *     [7] two-site splits,
  * [8] the dense-SVD count of the same splits without blocking (what one
- *     unblocked SVD per split would be charged), [9] binary64 polish sweeps
- *     (HM_MIXED), [10] charge blocks decomposed, [11] reserved.
+ *     unblocked SVD per split would be charged), [9] binary64-accurate
+ *     finishing passes (HM_MIXED), [10] charge blocks decomposed, [11] reserved.
  * Synchronises. */
 int hm_chain_stats(hm_ctx* ctx, hm_chain chain, double* out);
 
