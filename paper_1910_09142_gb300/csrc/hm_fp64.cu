@@ -397,8 +397,11 @@ __device__ void two_site_op(ChainDev* c, const OpDev op, int t, Shared& sh, int3
   __syncthreads();
 }
 
-// Blocks of fewer columns go straight to the binary64 sweeps.
-constexpr int kPrecond = 12;
+// Blocks of fewer columns go straight to the binary64 sweeps.  GB300, ms a
+// Markov step with the line at 6, 12, 20 and 32 columns: one METTS chain of Lx = 4
+// 17.6, 19.6, 22.3, 22.4; 4 chains of Lx = 4, 2W = 4 (chi = 64) 99, 98, 120, 132;
+// 152 chains of Lx = 6, 2W = 4 (chi = 96) 254, 264, 312, 415.
+constexpr int kPrecond = 6;
 // Stopping ratios: of the binary64 sweeps (the next sweep's off-diagonals
 // would be of order its square), and of the binary32 sweeps before them (what
 // they leave, ~1e-6, is binary32 resolution).

@@ -125,7 +125,7 @@ def test_binary32_block_to_binary64_accuracy(emu, case):
         assert G.max() <= (1e-9 if out[1] == 0 else 2e-6)
 
 
-@pytest.mark.parametrize("p", [12, 15, 16, 31, 32, 33, 60, 65, 130])
+@pytest.mark.parametrize("p", [6, 7, 8, 9, 11, 12, 15, 16, 31, 32, 33, 60, 65, 130])
 def test_orthonormalisation_reaches_binary64(emu, p):
     rng = np.random.default_rng(p)
     Q = np.linalg.qr(rng.standard_normal((p, p)))[0]
