@@ -115,6 +115,11 @@ __device__ __forceinline__ void team_sync(const Team& tm) {
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
     return;
   }
+#elif defined(HM_TEAM_EMULATION)
+  if (tm.size > 1) {
+    simt::team_sync();
+    return;
+  }
 #endif
   __syncthreads();
 }
@@ -1608,11 +1613,16 @@ __device__ void finish(ChainDev* c, const OpDev& op, int t, SplitSh& s, const Wa
     }
   }
   team_sync(tm);                          // every block's W, V and values are there
-  if (*(volatile int32_t*)c->status != 0) return;   // a decomposition failed (the same answer in every CTA)
+  // A decomposition failed: nothing to absorb.  One thread reads the status for
+  // its CTA: rank 0 may set it below while another CTA of the team is still
+  // here, and threads of one CTA that saw different values would part at the next
+  // barrier.  (A CTA that sees that later value returns, as it would below.)
+  if (tid == 0) s.ok = *(volatile int32_t*)c->status == 0;
   for (int j = tid; j < P; j += NT) sraw[j] = c->sig[j];
   for (int b = warp; b < nb; b += NW)
     for (int j = lane; j < s.b[b].p; j += 32) sblk[s.b[b].svoff + j] = b;
   __syncthreads();
+  if (!s.ok) return;
   // descending rank (ties by slot): sig[rank] = value, perm[rank] = slot
   for (int j = tid; j < P; j += NT) {
     const double sj = sraw[j];
