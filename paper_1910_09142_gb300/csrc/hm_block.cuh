@@ -1648,12 +1648,16 @@ __device__ void finish(ChainDev* c, const OpDev& op, int t, SplitSh& s, const Wa
         tail /= total;
       }
     } else {
-      int pos = 0;                           // nonzero values
-      for (int i = lane; i < P; i += 32) pos += sort_key(sig[i]) != 0ull;
+      int pos = 0, nan = 0;                  // nonzero values; any that is no number
+      for (int i = lane; i < P; i += 32) {
+        const unsigned long long v = sort_key(sig[i]);
+        pos += v != 0ull;
+        nan |= v > 0x7ff0000000000000ull;
+      }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) pos += __shfl_xor_sync(0xffffffffu, pos, o);
       kk = min(pos, chim);
-      if (kk == 0) kk = -1;
+      if (kk == 0 || __any_sync(0xffffffffu, nan)) kk = -1;
     }
     if (lane == 0) {
       s.kk = kk;

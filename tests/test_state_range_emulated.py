@@ -1,0 +1,60 @@
+"""States handed in by hm_set_mps that are not normalised or not finite, on the
+CPU emulation of the kernels."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import test_kernels_emulated  # noqa: F401  (puts tests/simt on the path)
+import build_emulated
+from paper_1910_09142_gb300 import binding
+from test_kernels_emulated import Emu
+
+pytestmark = pytest.mark.slow
+
+
+@pytest.fixture(scope="module")
+def emu(tmp_path_factory):
+    try:
+        lib = ctypes.CDLL(build_emulated.build(str(tmp_path_factory.mktemp("range"))))
+    except FileNotFoundError as e:
+        pytest.skip(str(e))
+    P, vp, i32, i64 = ctypes.POINTER, ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64
+    for name, args in {"hm_create": [P(vp), ctypes.c_int, vp, ctypes.c_size_t, vp], "hm_destroy": [vp],
+                       "hm_init_chain": [vp, P(binding.Params), vp, P(i64)],
+                       "hm_set_mps": [vp, i64, P(i32), i32, vp, ctypes.c_size_t, i32, i32],
+                       "hm_apply_ops": [vp, i64, P(i32), i32], "hm_last_error": [vp],
+                       "hm_get_mps": [vp, i64, P(i32), i32, vp, ctypes.c_size_t, P(i32), P(ctypes.c_size_t)]}.items():
+        getattr(lib, name).argtypes = args
+    lib.hm_last_error.restype = ctypes.c_char_p
+    return lib
+
+
+def _apply(emu, prec, tensors, ops):
+    """Return code of hm_apply_ops on a chain that holds `tensors`, and the state after it."""
+    P32 = ctypes.POINTER(ctypes.c_int32)
+    e = Emu(emu)
+    cid = e.init(binding.params(Lx=len(tensors) // 2, two_W=0, beta=0.2, tau=0.1, chi_max=9, cutoff=0.0, seed=1,
+                                precision=getattr(binding, prec)))
+    dims = np.array([t.shape[0] for t in tensors] + [1], dtype=np.int32)
+    buf = np.concatenate([t.reshape(-1) for t in tensors])
+    e._ok(emu.hm_set_mps(e.h, cid, dims.ctypes.data_as(P32), len(tensors), buf.ctypes.data_as(ctypes.c_void_p),
+                         len(buf), 0, 0))
+    ops = np.array(ops, dtype=np.int32)
+    rc = emu.hm_apply_ops(e.h, cid, ops.ctypes.data_as(P32), len(ops))
+    state = e.mps(cid) if rc == 0 else None
+    e.close()
+    return rc, state
+
+
+@pytest.mark.parametrize("prec", ["HM_FP64", "HM_MIXED", "HM_MIXED32"])
+@pytest.mark.parametrize("exact", [1, 0])
+@pytest.mark.parametrize("where", ["all", "one"])
+def test_a_nan_is_an_error_of_any_split(emu, prec, exact, where):
+    rng = np.random.default_rng(2)
+    ten = [rng.standard_normal(s) for s in ((1, 3, 3), (3, 3, 9), (9, 3, 3), (3, 3, 1))]
+    if where == "all":
+        ten[1][:] = np.nan
+    else:
+        ten[1][0, 1, 2] = np.nan
+    assert _apply(emu, prec, ten, [[1, 0, 1, exact]])[0] == binding.HM_ERR_NUMERIC
