@@ -1174,8 +1174,10 @@ __device__ __forceinline__ float jacobi_angle32(float na, float nb, float ga, fl
   const float d = (nb - na) * inv, g = ga * inv;
   const float ratio = fabsf(g);
   const bool go = ratio > tol && na > kTiny32 && nb > kTiny32;
-  const float ih = rsqrtf(fmaf(d, d, 4.0f * (g * g)));
-  const float c2 = fmaf(0.5f, fabsf(d) * ih, 0.5f);
+  // d = sqrt(longer / shorter) has no square in binary32 from 1e19 on: there h = |d|
+  const float ad = fabsf(d);
+  const float ih = ad < 1e18f ? rsqrtf(fmaf(d, d, 4.0f * (g * g))) : __fdividef(1.0f, ad);
+  const float c2 = fmaf(0.5f, ad * ih, 0.5f);
   const float rc = rsqrtf(c2);
   const float sg = d < 0.0f ? -g : g;
   c = go ? c2 * rc : 1.0f;

@@ -58,3 +58,27 @@ def test_a_nan_is_an_error_of_any_split(emu, prec, exact, where):
     else:
         ten[1][0, 1, 2] = np.nan
     assert _apply(emu, prec, ten, [[1, 0, 1, exact]])[0] == binding.HM_ERR_NUMERIC
+
+
+def _centre_pair(M):
+    """A four-site state whose middle pair has theta = M (9 x 9)."""
+    return [np.eye(3).reshape(1, 3, 3), np.ascontiguousarray(M).reshape(3, 3, 9), np.eye(9).reshape(9, 3, 3),
+            np.eye(3).reshape(3, 3, 1)]
+
+
+@pytest.mark.parametrize("prec", ["HM_FP64", "HM_MIXED", "HM_MIXED32"])
+@pytest.mark.parametrize("top", [1e-6, 1.0, 1e5, 1e7, 1e12])
+def test_a_graded_state_of_any_norm_splits(emu, prec, top):
+    """Columns 1e-14 long that overlap with one of length `top`: squared norms up
+    to 1e52 apart.  An exact move gives theta back, in orthonormal left vectors.
+    Bar: 2e-6 of the largest entry, the mixed forms' binary32 theta (FP64: 1e-13)."""
+    M = np.diag(np.full(9, 1e-14)) * (1 + np.arange(9.0)[:, None])
+    M[0] = 1e-14
+    M[0, 0] = top
+    rc, state = _apply(emu, prec, _centre_pair(M), [[1, 0, 1, 1]])
+    assert rc == 0
+    U, R = state[1].reshape(9, -1), state[2].reshape(-1, 9)
+    tol = 1e-13 if prec == "HM_FP64" else 2e-6
+    assert np.abs(U @ R - M).max() <= tol * np.abs(M).max()
+    big = np.linalg.norm(R, axis=1) > 1e-6 * top
+    assert np.abs(np.linalg.norm(U[:, big], axis=0) - 1).max() <= tol
