@@ -1166,18 +1166,19 @@ __device__ __forceinline__ float dot_rows(const float2 (&x)[2 * U], const float2
 // angle is the longest link of a sub-round's chain.  d and ga are scaled by 1 /
 // sqrt(na nb), known before the dot product is.  (c, s) is conformal whatever
 // its rounding.  Returns the ratio |ga| / sqrt(na nb), or 0 (and c = 1, s = t =
-// 0) when the pair is not rotated: below tol, or a column below kTiny32 (noise
+// 0) when the pair is not rotated: below tol, a column below kTiny32 (noise
 // at binary32 resolution; the fast reciprocal square root flushes subnormal
-// inputs to 0).
+// inputs to 0), or |d|, the ratio of the two lengths, above 1e18: its square
+// would overflow from 1.8e19 on, and the angle is far below binary32 resolution.  (An
+// exact form for those, one more reciprocal and a select on the chain, took
+// 2 to 3 % of a step; the binary64 finish rotates such a pair.)
 __device__ __forceinline__ float jacobi_angle32(float na, float nb, float ga, float tol, float& c, float& s, float& t) {
   const float inv = rsqrtf(fmaxf(na, kTiny32)) * rsqrtf(fmaxf(nb, kTiny32));
   const float d = (nb - na) * inv, g = ga * inv;
   const float ratio = fabsf(g);
-  const bool go = ratio > tol && na > kTiny32 && nb > kTiny32;
-  // d = sqrt(longer / shorter) has no square in binary32 from 1e19 on: there h = |d|
-  const float ad = fabsf(d);
-  const float ih = ad < 1e18f ? rsqrtf(fmaf(d, d, 4.0f * (g * g))) : __fdividef(1.0f, ad);
-  const float c2 = fmaf(0.5f, ad * ih, 0.5f);
+  const bool go = ratio > tol && na > kTiny32 && nb > kTiny32 && fabsf(d) < 1e18f;
+  const float ih = rsqrtf(fmaf(d, d, 4.0f * (g * g)));
+  const float c2 = fmaf(0.5f, fabsf(d) * ih, 0.5f);
   const float rc = rsqrtf(c2);
   const float sg = d < 0.0f ? -g : g;
   c = go ? c2 * rc : 1.0f;
