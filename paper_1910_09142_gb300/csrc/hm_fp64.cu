@@ -1113,6 +1113,7 @@ __global__ void __launch_bounds__(NT) reset_kernel(BatchArg b, OutArg o, int dra
     c->counters[2] = c->counters[1];
     c->counters[3] = 0;
     c->counters[4] = 0;
+    c->counters[5] = 0;
   }
 }
 

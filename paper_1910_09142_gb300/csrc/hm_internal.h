@@ -70,7 +70,8 @@ struct ChainDev {
   int32_t* counters;         // [0] sample index n, [1] basis of the current initial state,
                              // [2] frame of the stored state (0: as is, 1: every leg rotated by R,
                              //     which exchanges S^x and S^z), [3] dense mode (no charge labels),
-                             // [4] op cursor of a partial evolution (hm_evolve_partial)
+                             // [4] op cursor of a partial evolution (hm_evolve_partial),
+                             // [5] explicit ops since the last reset (norm not known to be 1)
   double* stats;             // ST_N
   int32_t* status;           // 0 = ok, else a negative HM_ERR_* code
   int32_t* err_where;        // op index / site where the error happened

@@ -422,8 +422,9 @@ __device__ HM_COLD int sweep64(double* W, int q, int p, double* V, double* nrm, 
 
 // From a block's binary32 result (W32, V32 in shared memory, followed by
 // refine::extra floats) to its binary64 W and V (global memory), by the nw
-// warps of its group.  polish: the binary64-accurate finish of hm_refine.cuh;
-// otherwise only the unit-column scales.  K: scratch for the block's K.  Returns
+// warps of its group.  polish: the binary64-accurate finish of hm_refine.cuh
+// (2: on a state whose norm is not known to be 1, see check_range); otherwise only
+// the unit-column scales.  K: scratch for the block's K.  Returns
 // the polish passes (1, or the binary64 sweeps it fell back on), -1 when
 // those did not converge.
 __device__ int refine_block(ChainDev* c, const blk::BlockRec& r, float* W32, float* V32, float* K,
@@ -440,32 +441,34 @@ __device__ int refine_block(ChainDev* c, const blk::BlockRec& r, float* W32, flo
     refine::pad_rows(V32, p, ldv, p, lw, nw);
   }
   blk::group_sync(bar, nthr);                 // the sweeps' last reads of the norms
-  refine::column_terms(W32, q, ldw, V32, p, ldv, ah, al, dl, polish ? K : nullptr, lw, nw);
+  const bool out =
+      refine::column_terms(W32, q, ldw, V32, p, ldv, ah, al, dl, polish ? K : nullptr, lw, nw, polish == 2);
   if (lw == 0 && (threadIdx.x & 31) == 0) {
     gs.flag[g] = 0;
     gs.rbits[g] = 0u;
   }
   blk::group_sync(bar, nthr);
-  if (!polish) {
-#pragma unroll 1
-    for (int side = 0; side < 2; ++side)
-      refine::scale_columns(side ? V32 : W32, side ? p : q, side ? ldv : ldw, p, dl, side ? V64 : W64, lw, nw);
-    return 0;
-  }
-  float e = refine::pair_terms<false>(W32, q, ldw, p, ah, al, K, lw, nw);
+  bool plain = polish == 0;                   // only the unit-column scales
+  if (polish) {
+    float e = refine::pair_terms<false>(W32, q, ldw, p, ah, al, K, lw, nw);
+    if (out) e = refine::kOutOfRange;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) e = fmaxf(e, __shfl_xor_sync(0xffffffffu, e, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(&gs.rbits[g], __float_as_uint(e));
-  blk::group_sync(bar, nthr);                 // K and its largest entry are complete
+    for (int o = 16; o > 0; o >>= 1) e = fmaxf(e, __shfl_xor_sync(0xffffffffu, e, o));
+    if ((threadIdx.x & 31) == 0) atomicMax(&gs.rbits[g], __float_as_uint(e));
+    blk::group_sync(bar, nthr);               // K and its largest entry are complete
+    plain = __uint_as_float(gs.rbits[g]) >= refine::kOutOfRange;
+  }
   int x = 0;
 #pragma unroll 1
   for (int side = 0; side < 2; ++side) {
     const int n = side ? p : q;
-    refine::add_product<false>(side ? V32 : W32, n, side ? ldv : ldw, p, K, side ? V64 : W64, n, lw, nw, x);
+    if (plain) refine::scale_columns(side ? V32 : W32, n, side ? ldv : ldw, p, dl, side ? V64 : W64, lw, nw);
+    else refine::add_product<false>(side ? V32 : W32, n, side ? ldv : ldw, p, K, side ? V64 : W64, n, lw, nw, x);
   }
+  if (!polish) return 0;
   blk::group_sync(bar, nthr);
   if (lw == 0) {
-    const int found = refine::rotate_near(W64, q, V64, p, ah, 2 * p);
+    const int found = plain ? 0 : refine::rotate_near(W64, q, V64, p, ah, 2 * p);
     if ((threadIdx.x & 31) == 0)
       gs.flag[g] = found > 2 * p || __uint_as_float(gs.rbits[g]) >= (float)kPolishStop ? 2 : (found > 0 ? 1 : 0);
   }
@@ -623,6 +626,13 @@ __device__ void two_site_op_mixed(ChainDev* c, const OpDev op, int t, int bcols,
   blk::finish<NT>(c, op, t, ss, wv, tm, scratch, tiles, ctx_err, sw32, sw64);
 }
 
+// Whether the state's norm may be far from 1, so that a column's length does not
+// say what it weighs: a state from outside (dense until its next collapse), or explicit ops now or since
+// the last reset.  The planned schedules start at norm 1 and keep it.
+__device__ __forceinline__ bool check_range(const BatchArg& b, const ChainDev* c) {
+  return b.ops_override || c->counters[3] || c->counters[5];
+}
+
 // team: CTAs of a cluster that share one chain (1: no cluster).
 __global__ void __launch_bounds__(NT, kCtasPerSm) evolve_mixed_kernel(BatchArg b, OutArg o, int bcols, int polish,
                                                                       int team) {
@@ -637,8 +647,10 @@ __global__ void __launch_bounds__(NT, kCtasPerSm) evolve_mixed_kernel(BatchArg b
   const int n_ops = b.ops_override ? b.n_override : c->n_ops;
   const int t0 = b.budget > 0 ? c->counters[4] : b.t0;
   const int t1 = b.budget > 0 ? min(t0 + b.budget, n_ops) : (b.t1 < n_ops ? b.t1 : n_ops);
-  blk::team_sync(tm);                                        // every thread has read the cursor
+  if (polish && check_range(b, c)) polish = 2;
+  blk::team_sync(tm);                                        // every thread has read the cursor and the marks
   if (b.budget > 0 && threadIdx.x == 0 && tm.rank == 0) c->counters[4] = t1;
+  if (b.ops_override && threadIdx.x == 0 && tm.rank == 0) c->counters[5] = 1;
   for (int t = t0; t < t1; ++t) {
     // the team agrees: a CTA sets the status only behind a barrier of the op
     if (*(volatile int32_t*)c->status != 0) return;

@@ -21,7 +21,8 @@
 // overlap; their pairs (|b - a| < kNear max(a, b)) are left out of K and
 // rotated one after another in binary64 afterwards.  When too many pairs are near (an
 // exactly degenerate spectrum), or E is not small, the binary64 sweeps of
-// jacobi_group run on W' and V' as well.
+// jacobi_group run on W' and V' as well; they run on W and V themselves when a
+// state of unknown norm has columns outside binary32's range (column_terms).
 //
 // The columns of V come out of the sweeps up to ~1e-5 longer than 1 (a
 // binary32 rotation with a small angle has cosine exactly 1, so it stretches
@@ -43,6 +44,13 @@ namespace refine {
 // explicitly.  Outside it |t| < E / 0.02 ~ 1e-4, and the terms the first
 // order leaves out are below 1e-4 E.
 constexpr float kNear = 0.02f;
+
+// Squared norm above which a sum of binary32 products may overflow (Dot2's
+// constant is up to 24 times the norm).
+constexpr float kHuge32 = 1e36f;
+
+// What a block's largest |E| becomes when a column lies outside [kTiny32, kHuge32].
+constexpr float kOutOfRange = 4.0f;
 
 // A value as an unevaluated binary32 sum.
 struct F2 {
@@ -129,17 +137,24 @@ __device__ __forceinline__ double corrected(float x, float corr) { return blk::w
 // delta_j and the squared norms of the columns (ah holds the sweeps' running
 // ones); KT: zeroed padding and the diagonal.  W and V: zero rows up to a
 // multiple of four (jacobi_regs leaves them so; padded here for the other
-// orderings by pad_rows).  Eight lanes a column.
-__device__ inline void column_terms(const float* W, int q, int ldw, const float* V, int p, int ldv, float* ah, float* al,
-                                    float* dl, float* KT, int lw, int nw) {
+// orderings by pad_rows).  Eight lanes a column.  check: returns whether this lane saw
+// a nonzero column that the binary32 sweeps have left alone (blk::kTiny32) or
+// cannot sum (kHuge32).  In a state of norm 1 a column shorter than 1e-15 lies
+// below the resolution of theta itself, and swept in binary64 it only shrinks
+// on (a null column loses 16 digits a sweep: 3 % of a step at Lx = 6, chi = 96, 304 chains).
+__device__ inline bool column_terms(const float* W, int q, int ldw, const float* V, int p, int ldv, float* ah, float* al,
+                                    float* dl, float* KT, int lw, int nw, bool check = false) {
   const int sub = (threadIdx.x & 31) >> 3, sl = threadIdx.x & 7;
   const int ldk = ldk_of(p);
+  bool out = false;
   for (int j0 = 4 * lw; j0 < p; j0 += 4 * nw) {
     const int j = j0 + sub, jj = j < p ? j : p - 1;
     const F2 a = norm2(W + (size_t)jj * ldw, q, 1.5f * ah[jj]);
     const F2 v = norm2(V + (size_t)jj * ldv, p, 1.5f);
     __syncwarp();                             // every lane has read its column's running norm
     if (j >= p) continue;
+    if (check && !(a.h > blk::kTiny32 && a.h < kHuge32))
+      for (int r = sl; r < q; r += 8) out |= W[(size_t)j * ldw + r] != 0.0f;
     if (sl == 0) {
       ah[j] = a.h;
       al[j] = a.l;
@@ -151,6 +166,7 @@ __device__ inline void column_terms(const float* W, int q, int ldw, const float*
     }
     if (KT && p + sl < ldk) KT[(size_t)j * ldk + p + sl] = 0.0f;
   }
+  return out;
 }
 
 // Zero rows n .. up to a multiple of four of p columns.

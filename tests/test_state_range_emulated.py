@@ -82,3 +82,41 @@ def test_a_graded_state_of_any_norm_splits(emu, prec, top):
     assert np.abs(U @ R - M).max() <= tol * np.abs(M).max()
     big = np.linalg.norm(R, axis=1) > 1e-6 * top
     assert np.abs(np.linalg.norm(U[:, big], axis=0) - 1).max() <= tol
+
+
+@pytest.mark.parametrize("prec", ["HM_FP64", "HM_MIXED"])
+@pytest.mark.parametrize("scale", [1e-30, 1e-20, 1e-12, 1.0, 1e12, 3e18, 1e20, 1e37])
+@pytest.mark.parametrize("kind", ["random", "graded"])
+def test_left_vectors_are_orthonormal_at_any_scale(emu, prec, scale, kind):
+    """The sweeps in binary32 leave columns shorter than 1e-15 alone and cannot sum
+    squares above 1e38: binary64 sweeps take such blocks.  Bars: U R = theta to
+    2e-6 of its largest entry (the mixed form's binary32 theta; FP64 1e-13), the
+    vectors kept by an exact move orthonormal to 1e-9 (no two values are near)."""
+    rng = np.random.default_rng(5)
+    M = rng.standard_normal((9, 9))
+    if kind == "graded":
+        q = np.linalg.qr(rng.standard_normal((2, 9, 9)))[0]
+        M = q[0] @ np.diag(np.logspace(0, -12, 9)) @ q[1].T
+    M = M * scale
+    rc, state = _apply(emu, prec, _centre_pair(M), [[1, 0, 1, 1]])
+    assert rc == 0
+    U, R = state[1].reshape(9, -1), state[2].reshape(-1, 9)
+    assert np.abs(U @ R - M).max() <= (1e-13 if prec == "HM_FP64" else 2e-6) * np.abs(M).max()
+    assert np.abs(U.T @ U - np.eye(U.shape[1])).max() <= 1e-9
+
+
+def test_explicit_ops_on_a_labelled_chain_are_checked_too(emu):
+    """Exact ops with bond gates do not keep the norm: weak gates entangle the
+    pairs, then a rung's exp(10 S.S) takes up to e^10 an op, four times."""
+    e = Emu(emu)
+    p = binding.params(Lx=2, two_W=0, J_leg=0.5, J_rung=-40.0, beta=1.0, tau=0.5, chi_max=9, cutoff=0.0, seed=2,
+                       precision=binding.HM_MIXED)
+    cid = e.init(p, env=[0, 1, 1, 2])
+    ops = np.array([[1, 3, 1, 0], [2, 3, 0, 0], [1, 3, 0, 0], [0, 3, 1, 0], [1, 3, 1, 0], [2, 3, 0, 0], [1, 3, 0, 0]] +
+                   [[0, 2, 1, 1]] * 5 + [[1, 0, 1, 1]], dtype=np.int32)
+    e._ok(emu.hm_apply_ops(e.h, cid, ops.ctypes.data_as(ctypes.POINTER(ctypes.c_int32)), len(ops)))
+    A = e.mps(cid)
+    assert np.linalg.norm(A[2]) > 1e19
+    U = A[1].reshape(-1, A[1].shape[2])
+    assert U.shape[1] >= 5 and np.abs(U.T @ U - np.eye(U.shape[1])).max() <= 1e-9
+    e.close()
