@@ -34,13 +34,18 @@
  *   asynchronous.  One context must not be used from two host threads at once.
  * - Data layout: an MPS site tensor A[k] has shape (chi_{k-1}, 3, chi_k),
  *   row-major FP64, local basis m = +1, 0, -1.  Bond dims live on the device.
- * - Precision: HM_FP64 runs every step in IEEE binary64.  HM_MIXED forms
+ * - Precision: HM_FP64 computes every result in IEEE binary64; its Jacobi
+ *   sweeps start from vectors that binary32 sweeps have found and end under a
+ *   binary64 stopping rule (blocks of fewer than 6 columns, or too large for
+ *   shared memory: binary64 sweeps only).  HM_MIXED forms
  *   the two-site tensor and applies the gate in binary32 (binary64 site
  *   tensors rounded on load, gate coefficients as binary32 hi + lo pairs),
  *   decomposes each charge block with binary32 one-sided Jacobi sweeps, then
  *   finishes it (a first-order sweep from exactly split sums, binary64
- *   rotations where that does not hold) so the singular values and vectors are
- *   binary64-accurate for that tensor; truncation, renormalisation, stored
+ *   rotations where that does not hold): the left factor's columns end
+ *   orthogonal to ~1e-10 (up to ~1e-6 among three or more values within 1 % of
+ *   each other), the right one's have length 1 to ~1e-12 and overlap by the binary32
+ *   sweeps' ~1e-6; truncation, renormalisation, stored
  *   tensors, measurement and collapse are binary64.  HM_MIXED32 is HM_MIXED
  *   without that finish.  Measured on GB300 against HM_FP64 (same
  *   chains, same draws): per-sample energies within ~1e-6 relative for both
@@ -64,9 +69,9 @@ extern "C" {
 #define HM_ERR_TIMEOUT (-5)  /* a device-side iteration budget ran out             */
 #define HM_ERR_STATE (-6)    /* call out of order (e.g. evolve twice, no collapse) */
 
-#define HM_FP64 0            /* every step in binary64                              */
+#define HM_FP64 0            /* binary64 results; the SVDs start from binary32 sweeps */
 #define HM_MIXED 1           /* evolve: contraction and gate in binary32, Jacobi SVD */
-                             /* in binary32, then to binary64 accuracy; truncation,  */
+                             /* in binary32, finished in binary64; truncation,       */
                              /* renormalisation, stored tensors, measurement and     */
                              /* collapse in binary64                                 */
 #define HM_MIXED32 2         /* HM_MIXED with the SVD left at its binary32 sweeps    */
@@ -248,7 +253,7 @@ int hm_collapse_conditionals(hm_ctx* ctx, const hm_chain* ids, int32_t n, int8_t
  *     HM_MIXED, the binary64 sweeps after the binary32 start under HM_FP64),
  *     [7] two-site splits,
  * [8] the dense-SVD count of the same splits without blocking (what one
- *     unblocked SVD per split would be charged), [9] binary64-accurate
+ *     unblocked SVD per split would be charged), [9] binary64
  *     finishing passes (HM_MIXED), [10] charge blocks decomposed, [11] reserved.
  * Synchronises. */
 int hm_chain_stats(hm_ctx* ctx, hm_chain chain, double* out);

@@ -4,10 +4,9 @@
 // 1.2 TFLOP/s on 152 SMs), so this path forms the two-site tensor and applies
 // the 9x9 gate in binary32 and runs the one-sided Jacobi sweeps of every
 // charge block (Sec. II.C, hm_block.cuh) in binary32.  HM_MIXED then finishes
-// each block so that the singular values and left vectors become
-// binary64-accurate for that tensor (hm_refine.cuh: one first-order sweep as a
-// product, binary64 rotations where that does not hold); HM_MIXED32 stops at
-// the binary32 sweeps.  The truncation weights (Sec. II), the renormalisation
+// each block as a binary64 sweep would (hm_refine.cuh: one first-order sweep as a
+// product, binary64 rotations where that does not hold; what it leaves is stated
+// there); HM_MIXED32 stops at the binary32 sweeps.  The truncation weights (Sec. II), the renormalisation
 // of the kept singular values and the stored site tensors stay binary64.
 // Measurement and collapse (steps 3-4) are the binary64 kernels of hm_fp64.cu.
 //
@@ -422,7 +421,7 @@ __device__ HM_COLD int sweep64(double* W, int q, int p, double* V, double* nrm, 
 
 // From a block's binary32 result (W32, V32 in shared memory, followed by
 // refine::extra floats) to its binary64 W and V (global memory), by the nw
-// warps of its group.  polish: the binary64-accurate finish of hm_refine.cuh
+// warps of its group.  polish: the binary64 finish of hm_refine.cuh
 // (2: on a state whose norm is not known to be 1, see check_range); otherwise only
 // the unit-column scales.  K: scratch for the block's K.  Returns
 // the polish passes (1, or the binary64 sweeps it fell back on), -1 when
@@ -522,11 +521,9 @@ __device__ __forceinline__ int64_t block_floats(int q, int p) {
 // tensors, binary32 accumulation, gate coefficients as binary32 pairs); the
 // blocks of a split in waves that fit in shared memory, each block of a wave
 // decomposed by its own warp group at the same time: a binary32 one-sided
-// Jacobi as a preconditioner, then binary64 sweeps on the promoted W and V
-// until the binary64 stopping rule holds, so the singular values and the kept
-// vectors are binary64-accurate for that theta.  A block too large for
+// Jacobi, then (HM_MIXED) refine_block.  A block too large for
 // shared memory runs alone, its binary32 sweeps on column blocks staged from
-// global memory.  Then the truncation rule (Sec. II), renormalisation and
+// global memory, then a binary64 sweep.  Then the truncation rule (Sec. II), renormalisation and
 // absorb in binary64.
 __device__ void two_site_op_mixed(ChainDev* c, const OpDev op, int t, int bcols, int polish, float* smem, Scal& sc,
                                   blk::SplitSh& ss, blk::WaveSh& wv, blk::GroupSh& gs, const blk::Team& tm,

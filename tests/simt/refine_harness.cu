@@ -1,0 +1,47 @@
+// TEST INFRASTRUCTURE: the mixed kernel's own path of one block in the CPU
+// emulation: binary32 sweeps, then refine_block (hm_mixed.cu) with its flags and
+// fallbacks.  The kernel source is built once more under another namespace.  Built
+// only by test_refine_emulated.py.
+#define hm hm_probe_ns
+#define HM_MIXED_NT 256
+#define HM_MIXED_CTAS_PER_SM 2
+#include "hm_mixed.cu"
+#undef hm
+
+namespace {
+
+namespace p_ = hm_probe_ns;
+
+// buf: W (p x ld4(q)), V (p x ld4(p)), the finish's terms.
+__global__ void refine_probe(float* buf, int q, int p, float* K, p_::ChainDev* c, int polish, int* out) {
+  __shared__ p_::blk::GroupSh gs;
+  const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  float* V = buf + (size_t)p * p_::blk::ld4(q);
+  p_::blk::BlockRec r = {};
+  r.q = (int16_t)q;
+  r.p = (int16_t)p;
+  const int sw = p_::blk::jacobi_group<float>(buf, q, p_::blk::ld4(q), p, V, p_::blk::ld4(p),
+                                              V + (size_t)p * p_::blk::ld4(p), warp, nw, 1, 0, gs,
+                                              p_::kStop32Polished, p_::kMaxSweeps);
+  const int s64 = p_::refine_block(c, r, buf, V, K, polish, warp, nw, 1, 0, gs);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    out[0] = sw;
+    out[1] = s64;
+    out[2] = gs.flag[0];
+    out[3] = (int)gs.rbits[0];
+  }
+}
+
+}  // namespace
+
+// out: binary32 sweeps, refine_block's return value, its last flag, the bits of the
+// largest overlap (a binary64 sweep to its stop leaves 0 there).
+extern "C" void hm_probe_refine(float* buf, int q, int p, int polish, double* W64, double* V64, double* sig, int* out) {
+  alignas(16) static float K[260 * 260];
+  p_::ChainDev c = {};
+  c.W = W64;
+  c.V = V64;
+  c.sig = sig;
+  refine_probe<<<1, 128, 0, nullptr>>>(buf, q, p, K, &c, polish, out);
+}
