@@ -43,7 +43,7 @@
  *   decomposes each charge block with binary32 one-sided Jacobi sweeps, then
  *   finishes it (a first-order sweep from exactly split sums, binary64
  *   rotations where that does not hold): the left factor's columns end
- *   orthogonal to ~1e-10 (up to ~1e-6 among three or more values within 1 % of
+ *   orthogonal to ~1e-9 (up to ~1e-6 among three or more values within 1 % of
  *   each other), the right one's have length 1 to ~1e-12 and overlap by the binary32
  *   sweeps' ~1e-6; truncation, renormalisation, stored
  *   tensors, measurement and collapse are binary64.  HM_MIXED32 is HM_MIXED

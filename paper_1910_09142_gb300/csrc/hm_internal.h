@@ -138,7 +138,7 @@ void set_global_error(const char* msg);
 int launch_evolve_mixed(const BatchArg& b, const OutArg& o, int chi_cap, int polish, void* stream);
 int launch_evolve_mixed_pair(const BatchArg& b, const OutArg& o, int chi_cap, int polish, void* stream);
 constexpr int kPairChiCap = 256;
-constexpr size_t kPairBlockSmem = 108 * 1024;
+constexpr size_t kPairBlockSmem = 109 * 1024;
 
 // Binary32 GEMM tile of the mixed evolve kernel, and the dynamic shared
 // memory one CTA may opt into on sm_100-class parts (227 KB).
@@ -148,7 +148,7 @@ constexpr size_t kMaxSharedOptIn = 227 * 1024;
 // Dynamic shared memory of the mixed evolve kernel at bond cap chi_cap: two
 // column blocks of b columns of the q + p <= 6 chi_cap row panel, plus the
 // cached column norms; b = 16, halved (down to 2) while that exceeds the
-// budget (210 KB, or kPairBlockSmem with two CTAs per SM).
+// budget (210 KB, or 108 KB with two CTAs per SM).
 // The GEMM tile is the floor.  Writes b to *bcols.
 inline size_t mixed_smem_bytes(int chi_cap, int* bcols, size_t budget = 210 * 1024) {
   const size_t qp = 6 * (size_t)chi_cap;

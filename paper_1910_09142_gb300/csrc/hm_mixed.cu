@@ -33,9 +33,9 @@ namespace hm {
 
 namespace {
 
-// This file builds the kernel twice: one CTA of 512 threads per SM (210 KB
+// This file builds the kernel twice: one CTA of 512 threads per SM (218 KB
 // of shared memory), and, from hm_mixed_pair.cu, two CTAs of 256 threads per
-// SM (108 KB each) for batches with more chains than SMs.
+// SM (109 KB each) for batches with more chains than SMs.
 #ifndef HM_MIXED_NT
 #define HM_MIXED_NT 512
 #define HM_MIXED_CTAS_PER_SM 1
@@ -388,14 +388,17 @@ __device__ void promote_v(const float* V32, int ldv, int q, int p, double* W64, 
 }
 
 // Shared memory of the binary32 block Jacobi; the kernel's dynamic shared
-// memory is at least this (and at least the staged fallback's plan).  Two
-// CTAs per SM share the SM's 228 KB.
-constexpr size_t kBlockSmem = kCtasPerSm == 1 ? 210 * 1024 : kPairBlockSmem;
+// memory is at least this (and at least the staged fallback's plan, made for
+// kStagedBudget).  One CTA may opt into 227 KB with its 4 KB of static shared
+// memory; two CTAs share the SM's 228 KB, 1 KB of it reserved for each.
+constexpr size_t kBlockSmem = kCtasPerSm == 1 ? 218 * 1024 : kPairBlockSmem;
+constexpr size_t kStagedBudget = kCtasPerSm == 1 ? 210 * 1024 : 108 * 1024;
 // Of it, what the blocks of a wave may take.
 #ifndef HM_WAVE_SMEM
 #define HM_WAVE_SMEM kBlockSmem
 #endif
 constexpr size_t kWaveSmem = HM_WAVE_SMEM;
+constexpr int64_t kWaveFloats = (int64_t)(kWaveSmem / sizeof(float));
 constexpr int kTileDoubles = NT / 32 * 8 * 33;   // finish()'s transposition tiles
 static_assert(sizeof(blk::PrepTab) <= kBlockSmem, "prepare's tables");
 
@@ -484,36 +487,49 @@ __device__ int refine_block(ChainDev* c, const blk::BlockRec& r, float* W32, flo
   return s64;
 }
 
-// One block too large for shared memory, by the whole CTA: binary32 sweeps on
-// column blocks staged from global memory, then the binary64 sweep.  Returns
-// the binary32 sweeps + 1000 x the binary64 ones, or -1.  Out of line: it is
+// Shared-memory floats of one block: W, V and the finish's terms.
+__device__ __forceinline__ int64_t block_floats(int q, int p) {
+  return (int64_t)p * blk::ld4(q) + (int64_t)p * blk::ld4(p) + blk::ld4(refine::extra(p));
+}
+
+// The same with no padding but odd leading dimensions: W, V and the norms.
+__device__ __forceinline__ int64_t tight_floats(int q, int p) {
+  return (int64_t)p * (q | 1) + (int64_t)p * (p | 1) + p;
+}
+
+// One block by the whole CTA whose wave layout (block_floats) does not fit in
+// shared memory: binary32 sweeps, then a binary64 sweep.  Columns without padding
+// (tight_floats) take a few per cent less, and where they fit the sweeps run on
+// them in shared memory; otherwise on column blocks staged from global memory.
+// GB300, one split in a buffer of 210 KB: 168 x 159 13.6 ms against 17.0 ms staged,
+// 165 x 162 15.1 against 20.3 (both fit the wave layout in 218 KB).
+// Returns the binary32 sweeps + 1000 x the binary64 ones, or -1.  Out of line: it is
 // rare, and its code would crowd the usual path's.
 __device__ HM_COLD int decompose_staged(ChainDev* c, int k, const blk::SplitSh& ss, const blk::BlockRec& r,
                                              const float* theta, int bcols, int polish, float* smem, Scal& sc,
                                              blk::GroupSh& gs) {
-  const int warp = threadIdx.x >> 5;
-  float* W32 = c->X;
-  float* V32 = c->X + (size_t)r.q * r.p;
+  const int warp = threadIdx.x >> 5, q = r.q, p = r.p;
+  const bool fits = tight_floats(q, p) <= kWaveFloats;
+  const int ldw = fits ? q | 1 : q, ldv = fits ? p | 1 : p;
+  float* W32 = fits ? smem : c->X;
+  float* V32 = W32 + (size_t)p * ldw;
   int c0 = 0;
-  blk::gather_block<NT, float, float>(c, k, ss, r, theta, W32, r.q, V32, r.p, c0);
+  blk::gather_block<NT, float, float>(c, k, ss, r, theta, W32, ldw, V32, ldv, c0);
   __syncthreads();
-  const int sw = cta_jacobi_f32(W32, r.q, r.p, V32, bcols, smem, sc, nullptr);
+  const int sw = fits ? blk::jacobi_group<float>(W32, q, ldw, p, V32, ldv, V32 + (size_t)p * ldv, warp, NT / 32, 1, 0,
+                                                 gs, polish ? kStop32Polished : kStop32, kMaxSweeps)
+                      : cta_jacobi_f32(W32, q, p, V32, bcols, smem, sc, nullptr);
   if (sw < 0) return -1;
   double* W64 = c->W + r.woff;
   double* V64 = c->V + r.voff;
-  promote_w(W32, r.q, V32, r.p, r.q, r.p, W64, c->sig);
+  promote_w(W32, ldw, V32, ldv, q, p, W64, c->sig);
   __syncthreads();
-  const int s64 = polish ? blk::jacobi_group<double, float, 2>(W64, r.q, r.q, r.p, V32, r.p, c->sig, warp, NT / 32, 1,
-                                                               0, gs, kPolishStop, kMaxSweeps)
+  const int s64 = polish ? blk::jacobi_group<double, float, 2>(W64, q, q, p, V32, ldv, c->sig, warp, NT / 32, 1, 0, gs,
+                                                               kPolishStop, kMaxSweeps)
                          : 0;
   __syncthreads();
-  promote_v(V32, r.p, r.q, r.p, W64, V64, c->sig, polish);
+  promote_v(V32, ldv, q, p, W64, V64, c->sig, polish);
   return s64 < 0 ? -1 : sw + 1000 * s64;
-}
-
-// Shared-memory floats of one block: W, V and the finish's terms.
-__device__ __forceinline__ int64_t block_floats(int q, int p) {
-  return (int64_t)p * blk::ld4(q) + (int64_t)p * blk::ld4(p) + blk::ld4(refine::extra(p));
 }
 
 // One two-site op (step 2 of Sec. I.C.1) in charge blocks (Sec. II.C):
@@ -535,7 +551,7 @@ __device__ void two_site_op_mixed(ChainDev* c, const OpDev op, int t, int bcols,
   blk::theta_blocks<NT, GM, GN, GK, float>(c, op.k, ss, theta, smem, tm);
   int sw32 = 0, sw64 = 0;
   int64_t cost = -1;
-  constexpr int64_t cap = (int64_t)(kWaveSmem / sizeof(float));
+  constexpr int64_t cap = kWaveFloats;
   if (tid == 0) blk::own_blocks(ss, tm, wv, [&](int q, int p) { return block_floats(q, p) <= cap; });
   __syncthreads();
   const int nown = wv.nown;
@@ -668,7 +684,7 @@ constexpr size_t kStagedSmem = HM_STAGED_SMEM;
 // lock: serving workers may launch from several host threads), then launch.
 int launch_kernel(const BatchArg& b, const OutArg& o, int chi_cap, int polish, void* stream) {
   int bcols = 16;
-  size_t plan = mixed_smem_bytes(chi_cap, &bcols, kBlockSmem);
+  size_t plan = mixed_smem_bytes(chi_cap, &bcols, kStagedBudget);
   if (plan > kStagedSmem) {
     // caps near the admission limit: one column a staged block, so that the
     // plan fits beside the kernel's static shared memory

@@ -26,7 +26,8 @@
 //
 // What is left, on the CPU emulation of this code (blocks of 11 to 73 columns):
 // relative overlaps of W's columns of 1e-13 to 1e-10, as after a binary64 sweep on
-// the same blocks, but up to E where three or more values lie close together
+// the same blocks (at 147 to 162 columns, measured, 6e-10 to 2e-9 against the
+// sweep's 1e-10 to 5e-10), but up to E where three or more values lie close together
 // (2e-7 to 3e-7 on triple and six-fold values; 2e-7 to 4e-7 after the sweep).
 // Rotating such clusters down to 1e-9 took 1 to 4 % of a step.  V's columns have
 // length 1 to 1e-12 and overlap by the binary32 sweeps' ~1e-6, and W - theta V is

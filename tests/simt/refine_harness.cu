@@ -45,3 +45,56 @@ extern "C" void hm_probe_refine(float* buf, int q, int p, int polish, double* W6
   c.sig = sig;
   refine_probe<<<1, 128, 0, nullptr>>>(buf, q, p, K, &c, polish, out);
 }
+
+namespace {
+
+// A dense block (every charge 0) of a pair with bonds chil and chir.
+__global__ void staged_probe(const float* theta, int chil, int chir, p_::ChainDev* c, int polish, int* out) {
+  float* smem = (float*)simt::dynamic_smem();
+  __shared__ p_::Scal sc;
+  __shared__ p_::blk::SplitSh ss;
+  __shared__ p_::blk::GroupSh gs;
+  p_::blk::BlockRec r = {};
+  r.mq = (int16_t)(3 * chil);
+  r.nq = (int16_t)(3 * chir);
+  r.trans = chir > chil;
+  r.q = (int16_t)(3 * max(chil, chir));
+  r.p = (int16_t)(3 * min(chil, chir));
+  for (int t = 0; t < 3; ++t) {
+    r.roff[t] = (int16_t)(t * chil);
+    r.coff[t] = (int16_t)(t * chir);
+  }
+  if (threadIdx.x == 0)
+    for (int o = 0; o < 9; ++o) {
+      ss.nt[o] = 1;
+      ss.tt[o][0] = (int16_t)o;
+      ss.gh[o][0] = 1.0f;
+      ss.gl[o][0] = 0.0f;
+    }
+  __syncthreads();
+  const int code = p_::decompose_staged(c, 0, ss, r, theta, 4, polish, smem, sc, gs);
+  if (threadIdx.x == 0) *out = code;
+}
+
+}  // namespace
+
+// theta: 3 chil x 3 chir.  X: binary32 scratch, or null.  Returns binary32 sweeps + 1000 x binary64 ones.
+extern "C" int hm_probe_staged(const float* theta, int chil, int chir, float* X, int polish, double* W64, double* V64,
+                               double* sig) {
+  int out = 0;
+  int32_t chi[3] = {chil, 0, chir};
+  p_::ChainDev c = {};
+  c.W = W64;
+  c.V = V64;
+  c.sig = sig;
+  c.X = X;
+  c.chi = chi;
+  staged_probe<<<1, p_::NT, p_::kBlockSmem, nullptr>>>(theta, chil, chir, &c, polish, &out);
+  return out;
+}
+
+// Whether a block's wave layout, and its layout without padding, fit the kernel's buffer.
+extern "C" int hm_probe_layouts(int q, int p, int64_t bytes) {
+  const int64_t n = bytes / 4;
+  return (p_::block_floats(q, p) <= n ? 1 : 0) + (p_::tight_floats(q, p) <= n ? 2 : 0);
+}

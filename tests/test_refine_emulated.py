@@ -82,3 +82,37 @@ def test_overlaps_end_below_the_bar(emu, case):
     assert np.abs(W - A @ V).max() <= 3e-5 * np.abs(A).max()
     ref = np.linalg.svd(A, compute_uv=False)
     assert np.abs(np.sort(d)[::-1] - ref).max() <= 3e-6 * ref[0]
+
+
+# Blocks around the edge of the buffers (218 KB with one chain per SM, 109 KB with two): 1 = the
+# wave layout fits, 2 = the unpadded one does, which keeps the sweeps in shared memory too.
+@pytest.mark.parametrize("q,p,kb,want", [(163, 163, 218, 3), (169, 160, 218, 3), (165, 162, 218, 3), (166, 166, 218, 2),
+                                         (168, 168, 218, 0), (118, 116, 109, 2), (126, 113, 109, 2), (117, 114, 109, 3),
+                                         (120, 117, 109, 0)])
+def test_layouts_at_the_edge_of_the_buffers(emu, q, p, kb, want):
+    assert emu.hm_probe_layouts(q, p, ctypes.c_int64(kb * 1024)) == want
+
+
+@pytest.mark.parametrize("chil,chir,polish", [(39, 38, 1), (38, 39, 1), (39, 38, 0), (40, 39, 1)])
+def test_a_block_at_the_edge_of_the_buffer(emu, chil, chir, polish):
+    """117 x 114 fits 109 KB without padding: no use of the scratch in global memory.  120 x 117 does not."""
+    rng = np.random.default_rng(chil)
+    theta = (rng.standard_normal((3 * chil, 3 * chir)) * np.logspace(0, -3, 3 * chir)).astype(np.float32)
+    q, p = max(theta.shape), min(theta.shape)
+    fits = q < 120
+    X = None if fits else np.zeros(2 * q * p, dtype=np.float32)
+    W, V, sig = np.zeros((p, q)), np.zeros((p, p)), np.zeros(p)
+    emu.hm_probe_staged.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_void_p, ctypes.c_int] + \
+        [ctypes.c_void_p] * 3
+    code = emu.hm_probe_staged(_ptr(theta), chil, chir, None if fits else _ptr(X), polish, _ptr(W), _ptr(V), _ptr(sig))
+    assert code > 0 and (code >= 1000) == bool(polish)
+    # rows (l a) of theta against the block's order (a l), columns alike; W holds the transpose of a wide block
+    A = theta.astype(np.float64).reshape(chil, 3, 3 * chir).transpose(1, 0, 2).reshape(3 * chil, 3 * chir)
+    A = A.T if chir > chil else A
+    W, V = W.T, V.T
+    assert np.abs(W - A @ V).max() <= 3e-5 * np.abs(A).max()
+    assert np.abs(np.linalg.norm(V, axis=0) - 1).max() <= (1e-9 if polish else 3e-7)
+    d = np.linalg.norm(W, axis=0)
+    G = np.abs(W.T @ W - np.diag(d * d)) / np.outer(d, d)
+    assert G.max() <= 3e-6
+    assert np.abs(np.sort(d)[::-1] - np.linalg.svd(A, compute_uv=False)).max() <= 3e-6 * d.max()
