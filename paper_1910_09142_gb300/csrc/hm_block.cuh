@@ -1350,8 +1350,11 @@ __device__ int jacobi_regs(float* __restrict__ W, int q, int ldw, int p, float* 
 // One-sided Jacobi of one block by a warp group: jacobi_regs for binary32
 // blocks of up to 128 rows; above, the block ordering in shared memory for 16
 // columns or more; otherwise (binary64) the round-robin ordering with 8 lanes a
-// pair.  None of them depends on the number of warps, nor does anything else a block goes through, so a chain's results are
-// the same bits whatever batch or team it runs in.
+// pair.  None of them depends on the number of warps, nor does anything else a
+// block goes through that fits the kernel's buffer.  So a chain's results are the
+// same bits in every batch and team while all its blocks fit half an SM (104 KB in
+// binary64: 79 x 79; 109 KB in the mixed kernel: 116 x 116).  A wider block takes a path of
+// its own in the build for two chains per SM, and its bits depend on the build.
 // TV: element type of V.  A binary64 polish of a binary32 result may keep V
 // in binary32: V carries binary32 accuracy from the preconditioning sweeps
 // anyway, and the polish's rotations are tiny (angles ~1e-6).

@@ -127,14 +127,14 @@ int device_sm_count();
 void set_global_error(const char* msg);
 
 // Mixed-precision evolve (hm_mixed.cu); chi_cap = largest bond cap in the
-// batch; polish != 0 finishes every SVD with binary64 sweeps (HM_MIXED).
+// batch; polish != 0 finishes every SVD in binary64 (HM_MIXED).
 // A batch of more chains than SMs with chi_cap <= kPairChiCap goes to
 // launch_evolve_mixed_pair (hm_mixed_pair.cu): two CTAs of 256 threads per
 // SM with kPairBlockSmem of shared memory each.  kPairChiCap: on the S=1
-// ladder at chi = 256 the largest charge block measured needs 106 KB in the
-// binary32 layout (p (q + 1) + p (p + 1) + p values; oracle U(1) chain,
-// Lx = 16, 2W = 8, beta = 1, three samples); a larger block takes the
-// staged global-memory path of the same kernel.
+// ladder at chi = 256 (oracle U(1) chain, Lx = 16, 2W = 8, beta = 1, cutoff 1e-7,
+// eight samples) the widest charge block has 97 to 109 columns, 89 to 114 KB in
+// the kernel's layout (block_floats), and 2 of 170,000 blocks need more than
+// 109 KB; those take decompose_staged.
 int launch_evolve_mixed(const BatchArg& b, const OutArg& o, int chi_cap, int polish, void* stream);
 int launch_evolve_mixed_pair(const BatchArg& b, const OutArg& o, int chi_cap, int polish, void* stream);
 constexpr int kPairChiCap = 256;
