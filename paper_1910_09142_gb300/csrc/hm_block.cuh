@@ -528,10 +528,11 @@ __device__ void theta_direct(const ChainDev* c, int k, const SplitSh& s, T* __re
   team_sync(tm);
 }
 
-template <int NT, int TM, int TN, int TK, typename T>
-__device__ void theta_blocks(const ChainDev* c, int k, const SplitSh& s, T* __restrict__ theta, T* smem,
+template <int NT, int TM, int TN, int TK>
+__device__ void theta_blocks(const ChainDev* c, int k, const SplitSh& s, float* __restrict__ theta, float* smem,
                              const Team& tm) {
-  if (sizeof(T) == sizeof(double) || s.k1 <= kThetaDirect) return theta_direct<NT, T>(c, k, s, theta, tm);
+  using T = float;
+  if (s.k1 <= kThetaDirect) return theta_direct<NT, T>(c, k, s, theta, tm);
   const int tid = threadIdx.x;
   const int chim = c->chi[k + 1], chir = c->chi[k + 2];
   const int n = 3 * chir;
@@ -1490,7 +1491,8 @@ __device__ __forceinline__ double warp_sum64(double v) {
 
 // Truncation rule (Sec. II): smallest k >= 1 whose discarded weight
 // sum_{q>=k} s_q^2 / sum s^2 <= cutoff, then min(k, chi_max), then lowered to
-// the nearest gap s_k < s_{k-1} (1 - 1e-8).  s sorted descending; one thread.
+// the nearest gap s_k < s_{k-1} (1 - 1e-8).  s sorted descending; one thread (the
+// allocation-free update; the evolve kernels take warp_trunc_rank).
 __device__ inline int trunc_rank(const double* s, int n, int chi_max, double cutoff, double* tail, double* total_out) {
   tail[n] = 0.0;
   for (int q = n - 1; q >= 0; --q) tail[q] = tail[q + 1] + s[q] * s[q];

@@ -234,27 +234,6 @@ __device__ int cta_jacobi(double* __restrict__ W, int q, int p, double* __restri
   return converged ? done : -1;
 }
 
-// Truncation rule (Sec. II): smallest k >= 1 whose discarded weight
-// sum_{q>=k} s_q^2 / sum s^2 <= cutoff, then min(k, chi_max), then lowered to
-// the nearest gap s_{k} < s_{k-1} (1 - 1e-8).  Runs on thread 0.
-__device__ int truncation_rank(const double* s, int n, int chi_max, double cutoff, double* tail,
-                               double* total_out) {
-  tail[n] = 0.0;
-  for (int q = n - 1; q >= 0; --q) tail[q] = tail[q + 1] + s[q] * s[q];
-  const double total = tail[0];
-  *total_out = total;
-  int k = n;
-  for (int kk = 1; kk <= n; ++kk) {
-    if (tail[kk] <= cutoff * total) {
-      k = kk;
-      break;
-    }
-  }
-  if (k > chi_max) k = chi_max;
-  while (k > 1 && k < n && s[k] >= s[k - 1] * (1.0 - 1e-8)) --k;
-  return k;
-}
-
 __device__ void two_site_op(ChainDev* c, const OpDev op, int t, Shared& sh, int32_t* ctx_err) {
   const int tid = threadIdx.x;
   const int k = op.k;
@@ -330,7 +309,7 @@ __device__ void two_site_op(ChainDev* c, const OpDev op, int t, Shared& sh, int3
     int kk;
     double nrm = 1.0;
     if (!op.exact) {
-      kk = truncation_rank(s, p, c->chi_max, c->cutoff, tail, &total);
+      kk = blk::trunc_rank(s, p, c->chi_max, c->cutoff, tail, &total);
       if (!(total > 0.0) || !isfinite(total)) kk = -1;
       else {
         double kept = 0.0;
@@ -613,15 +592,15 @@ __device__ void evolve_chain(const BatchArg& b, const OutArg& o, double* buf, si
 }
 
 __global__ void __launch_bounds__(kWideNT, 1) evolve_fp64_wide_kernel(BatchArg b, OutArg o, int team) {
-  extern __shared__ double dsm[];
+  extern __shared__ double2 dsm[];                           // 16-byte aligned: 128-bit loads of the columns
   __shared__ EvolveSh sh;
-  evolve_chain<kWideNT>(b, o, dsm, kWideSmem, sh, team);
+  evolve_chain<kWideNT>(b, o, reinterpret_cast<double*>(dsm), kWideSmem, sh, team);
 }
 
 __global__ void __launch_bounds__(NT, 2) evolve_fp64_pair_kernel(BatchArg b, OutArg o) {
-  extern __shared__ double dsm[];
+  extern __shared__ double2 dsm[];
   __shared__ EvolveSh sh;
-  evolve_chain<NT>(b, o, dsm, kPairSmem, sh, 1);
+  evolve_chain<NT>(b, o, reinterpret_cast<double*>(dsm), kPairSmem, sh, 1);
 }
 
 // Step 3 (Sec. I.C.1): <S_i.S_j> and <Sz_i Sz_j> on every measured bond.

@@ -46,8 +46,6 @@ constexpr int kMaxSweeps = 60;
 constexpr int GM = kMixedGM, GN = kMixedGN, GK = kMixedGK;   // binary32 GEMM tile (2x4 or 4x4 outputs a thread)
 
 struct Scal {
-  double red[NT / 32][2];
-  double dval[4];
   int32_t ival[4];
 };
 
@@ -220,8 +218,7 @@ __device__ void cross_phase_reg(float* W, float* V, int q, int p, int b, int nb,
 
 // Block one-sided Jacobi on W (q x p column-major, q >= p) with V (p x p).
 // smem holds two blocks of b columns of W and of V.  Returns sweeps or -1.
-// tmp: q p + p p floats of scratch (used once, to order the columns).
-__device__ int cta_jacobi_f32(float* W, int q, int p, float* V, int b, float* smem, Scal& sc, float* tmp) {
+__device__ int cta_jacobi_f32(float* W, int q, int p, float* V, int b, float* smem, Scal& sc) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int nwarps = NT / 32;
   for (int e = tid; e < p * p; e += NT) V[e] = (e % (p + 1) == 0) ? 1.f : 0.f;
@@ -234,36 +231,6 @@ __device__ int cta_jacobi_f32(float* W, int q, int p, float* V, int b, float* sm
   const int nb = (p + b - 1) / b;
   int done = 0;
   bool converged = false;
-  if (tmp) {
-    // order the columns by decreasing norm before the first sweep (W and V
-    // permuted together, so W = X V still holds): the graded two-site
-    // matrices converge in ~1 sweep fewer (12.3 -> 11.3 for 256 < p <= 512)
-    float* nrm = svJ + (size_t)b * p;
-    int* rk = reinterpret_cast<int*>(swI);
-    for (int j = warp; j < p; j += nwarps) {
-      const float* cj = W + (size_t)j * q;
-      float s2 = 0.f;
-      for (int i = lane; i < q; i += 32) s2 = fmaf(cj[i], cj[i], s2);
-      s2 = warp_sumf(s2);
-      if (lane == 0) nrm[j] = s2;
-    }
-    __syncthreads();
-    for (int j = tid; j < p; j += NT) {
-      const float nj = nrm[j];
-      int r = 0;
-      for (int i = 0; i < p; ++i) r += (nrm[i] > nj) || (nrm[i] == nj && i < j);
-      rk[j] = r;
-    }
-    __syncthreads();
-    float* tW = tmp;
-    float* tV = tmp + (size_t)q * p;
-    for (int e = tid; e < q * p; e += NT) tW[(size_t)rk[e / q] * q + e % q] = W[e];
-    for (int e = tid; e < p * p; e += NT) tV[(size_t)rk[e / p] * p + e % p] = V[e];
-    __syncthreads();
-    for (int e = tid; e < q * p; e += NT) W[e] = tW[e];
-    for (int e = tid; e < p * p; e += NT) V[e] = tV[e];
-    __syncthreads();
-  }
   while (done < kMaxSweeps) {
     if (tid == 0) {
       sc.ival[0] = 0;
@@ -518,7 +485,7 @@ __device__ HM_COLD int decompose_staged(ChainDev* c, int k, const blk::SplitSh& 
   __syncthreads();
   const int sw = fits ? blk::jacobi_group<float>(W32, q, ldw, p, V32, ldv, V32 + (size_t)p * ldv, warp, NT / 32, 1, 0,
                                                  gs, polish ? kStop32Polished : kStop32, kMaxSweeps)
-                      : cta_jacobi_f32(W32, q, p, V32, bcols, smem, sc, nullptr);
+                      : cta_jacobi_f32(W32, q, p, V32, bcols, smem, sc);
   if (sw < 0) return -1;
   double* W64 = c->W + r.woff;
   double* V64 = c->V + r.voff;
@@ -548,7 +515,7 @@ __device__ void two_site_op_mixed(ChainDev* c, const OpDev op, int t, int bcols,
   blk::PrepTab& tab = *reinterpret_cast<blk::PrepTab*>(smem);
   if (!blk::prepare<NT>(c, op, ss, tab, tm)) blk::prepare<NT>(c, op, ss, tab, tm);
   float* theta = reinterpret_cast<float*>(c->theta);
-  blk::theta_blocks<NT, GM, GN, GK, float>(c, op.k, ss, theta, smem, tm);
+  blk::theta_blocks<NT, GM, GN, GK>(c, op.k, ss, theta, smem, tm);
   int sw32 = 0, sw64 = 0;
   int64_t cost = -1;
   constexpr int64_t cap = kWaveFloats;
@@ -649,7 +616,8 @@ __device__ __forceinline__ bool check_range(const BatchArg& b, const ChainDev* c
 // team: CTAs of a cluster that share one chain (1: no cluster).
 __global__ void __launch_bounds__(NT, kCtasPerSm) evolve_mixed_kernel(BatchArg b, OutArg o, int bcols, int polish,
                                                                       int team) {
-  extern __shared__ float smem[];
+  extern __shared__ float4 dsm[];                            // 16-byte aligned: 128-bit loads of the columns
+  float* smem = reinterpret_cast<float*>(dsm);
   __shared__ Scal sc;
   __shared__ blk::SplitSh ss;
   __shared__ blk::WaveSh wv;
