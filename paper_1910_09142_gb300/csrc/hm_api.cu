@@ -872,6 +872,7 @@ static int evolve_launches(hm_ctx* ctx, const std::vector<Chain*>& cs, int budge
     // Equal costs keep the caller's order.
     std::stable_sort(group.begin(), group.end(), [](const Chain* a, const Chain* b) { return a->cost > b->cost; });
     const int rc = for_batches(group, [&](BatchArg& b, int s) {
+      b.chi_cap = chi_cap;
       auto launch = [&]() {
         return prec == HM_FP64 ? launch_evolve_fp64(b, o, ctx->stream)
                                : launch_evolve_mixed(b, o, chi_cap, prec == HM_MIXED, ctx->stream);
@@ -1252,6 +1253,7 @@ int hm_apply_ops(hm_ctx* ctx, hm_chain chain, const int32_t* ops, int32_t n_ops)
   BatchArg b{};
   b.n = 1;
   b.c[0] = c->dev;
+  b.chi_cap = c->mp.chi_cap;
   b.t0 = 0;
   b.t1 = n_ops;
   b.ops_override = (const OpDev*)sc.ptr;

@@ -1127,7 +1127,7 @@ int launch_evolve_fp64(const BatchArg& b, const OutArg& o, void* stream) {
     evolve_fp64_pair_kernel<<<b.n, NT, kPairSmem, (cudaStream_t)stream>>>(b, o);
   } else {
 #if !defined(HM_HOST_EMULATION)
-    const int team = team_size((const void*)evolve_fp64_wide_kernel, kWideNT, kWideSmem, b.n);
+    const int team = team_size((const void*)evolve_fp64_wide_kernel, kWideNT, kWideSmem, b.n, b.chi_cap);
     if (team > 1) return launch_team(evolve_fp64_wide_kernel, b, o, team, kWideNT, kWideSmem, stream, team);
 #endif
     evolve_fp64_wide_kernel<<<b.n, kWideNT, kWideSmem, (cudaStream_t)stream>>>(b, o, 1);

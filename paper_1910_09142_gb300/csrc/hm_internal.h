@@ -100,6 +100,7 @@ struct BatchArg {
   int32_t n_override;            // op count of ops_override
   int32_t budget;                // > 0: each chain runs ops [cursor, cursor + budget) of its own
                                  // list from its counters[4] and advances it (t0, t1 unused)
+  int32_t chi_cap;               // largest bond cap in the batch (evolve launches)
   const OpDev* ops_override;     // explicit op list (debug / kernel parity) or nullptr
   ChainDev* c[kMaxBatch];
 };

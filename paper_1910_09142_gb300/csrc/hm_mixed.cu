@@ -674,7 +674,7 @@ int launch_kernel(const BatchArg& b, const OutArg& o, int chi_cap, int polish, v
     }
   }
 #if HM_MIXED_CTAS_PER_SM == 1 && !defined(HM_HOST_EMULATION)
-  const int team = team_size((const void*)evolve_mixed_kernel, NT, smem, b.n);
+  const int team = team_size((const void*)evolve_mixed_kernel, NT, smem, b.n, chi_cap);
   if (team > 1) return launch_team(evolve_mixed_kernel, b, o, team, NT, smem, stream, bcols, polish, team);
 #endif
   evolve_mixed_kernel<<<b.n, NT, smem, (cudaStream_t)stream>>>(b, o, bcols, polish, 1);

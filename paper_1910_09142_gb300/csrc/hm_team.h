@@ -3,8 +3,9 @@
 //
 // A chain's ops are serial, but the charge blocks of one split are not: a team
 // shares out theta's tiles, the blocks (each decomposed by one CTA, the
-// costliest first) and the absorb, and meets at three cluster barriers an op.  Everything a CTA needs from another goes through the chain's
-// own buffers in global memory.  A Markov step, one CTA -> a team: 4 chains of Lx = 4, 2W =
+// costliest first) and the absorb, and meets at three cluster barriers an op.
+// Everything a CTA needs from another goes through the chain's own buffers in
+// global memory.  A Markov step, one CTA -> a team: 4 chains of Lx = 4, 2W =
 // 4, binary64, 206 -> 113 ms (8 CTAs); 8 mixed chains of Lx = 4, 30.4 -> 22.4
 // ms (8); one METTS chain of small blocks, 22.1 -> 20.4 ms (8).
 #pragma once
@@ -17,11 +18,26 @@
 
 namespace hm {
 
+// Bond caps up to here get one CTA a chain in every batch: a split has a few blocks
+// of a few columns, and three cluster barriers cost more than they share out.
+// us an op, one CTA and a team of 8 (1 to 70 chains): HM_FP64 cap 3 25 and 30, cap 9
+// 37 and 41, cap 27 51 and 51, cap 64 97 to 119 and 88 to 108; HM_MIXED 37 and 40, 39 and 41,
+// 46 and 46, 67 to 74 and 60 to 69.
+constexpr int kTeamChiCap = 27;
+
+// Largest cluster size of 8, 4 or 2 of which n are resident at once (most[e]:
+// clusters of 2^e that fit), else 1.
+inline int pick_team(const int (&most)[4], int n, int chi_cap) {
+  if (chi_cap <= kTeamChiCap) return 1;
+  for (int e = 3; e >= 1; --e)
+    if (most[e] >= n) return 1 << e;
+  return 1;
+}
+
 #if !defined(HM_HOST_EMULATION)
-// Largest cluster size of 8, 4 or 2 for which n clusters of `kernel` are
-// resident at once, else 1.  The occupancy answers are kept per device and
-// kernel (at most four kernels).
-inline int team_size(const void* kernel, int threads, size_t smem, int n) {
+// Cluster size for n chains with bond caps up to chi_cap.  The occupancy answers
+// are kept per device and kernel (at most four kernels).
+inline int team_size(const void* kernel, int threads, size_t smem, int n, int chi_cap) {
   struct Known {
     const void* kernel;
     int dev, most[4];                       // clusters of 2, 4 and 8 that fit
@@ -29,7 +45,7 @@ inline int team_size(const void* kernel, int threads, size_t smem, int n) {
   static std::mutex mu;
   static Known known[16] = {};
   static int n_known = 0;
-  if (2 * n > device_sm_count()) return 1;
+  if (2 * n > device_sm_count() || chi_cap <= kTeamChiCap) return 1;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 1;
   std::lock_guard<std::mutex> lock(mu);
@@ -60,9 +76,7 @@ inline int team_size(const void* kernel, int threads, size_t smem, int n) {
       k = &known[n_known++];
     }
   }
-  for (int e = 3; e >= 1; --e)
-    if (k->most[e] >= n) return 1 << e;
-  return 1;
+  return pick_team(k->most, n, chi_cap);
 }
 
 template <typename... P, typename... A>

@@ -98,3 +98,9 @@ extern "C" int hm_probe_layouts(int q, int p, int64_t bytes) {
   const int64_t n = bytes / 4;
   return (p_::block_floats(q, p) <= n ? 1 : 0) + (p_::tight_floats(q, p) <= n ? 2 : 0);
 }
+
+// Cluster size for n chains when 75, 37 and 18 clusters of 2, 4 and 8 CTAs fit.
+extern "C" int hm_probe_team(int n, int chi_cap) {
+  const int most[4] = {0, 75, 37, 18};
+  return p_::pick_team(most, n, chi_cap);
+}

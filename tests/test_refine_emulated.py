@@ -116,3 +116,9 @@ def test_a_block_at_the_edge_of_the_buffer(emu, chil, chir, polish):
     G = np.abs(W.T @ W - np.diag(d * d)) / np.outer(d, d)
     assert G.max() <= 3e-6
     assert np.abs(np.sort(d)[::-1] - np.linalg.svd(A, compute_uv=False)).max() <= 3e-6 * d.max()
+
+
+@pytest.mark.parametrize("n,chi,want", [(1, 3, 1), (1, 27, 1), (70, 27, 1), (1, 28, 8), (18, 64, 8), (19, 64, 4), (37, 256, 4),
+                                        (38, 256, 2), (75, 256, 2), (76, 256, 1)])
+def test_cluster_size_of_a_batch(emu, n, chi, want):
+    assert emu.hm_probe_team(n, chi) == want
