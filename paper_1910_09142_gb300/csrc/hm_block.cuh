@@ -1236,7 +1236,7 @@ __device__ __forceinline__ void intra_rows(float2 (&x)[2 * U], float2 (&v)[2 * U
 // rotation: ~300 clocks).  Super-columns of eight (4 lanes a pair) measured 3 %
 // faster on blocks of up to 32 rows and 10 % slower above.
 // Lx = 9, 2W = 8, chi = 256, binary32, 152 chains: 269 ms a Markov step with
-// jacobi_blocks, 208 ms with this.
+// jacobi_blocks, 208 ms with this (170 ms with the steps after it).
 //
 // Two copies, U = 2 and 4, for every size.  The groups of a CTA work on blocks of
 // different sizes at once, and four copies (and the shared-memory pass for the pairs
@@ -1385,8 +1385,9 @@ __device__ __forceinline__ int block_cost(int q, int p) { return p * p * (q + 48
 // worth a warp or more does, and smaller ones are put together, one after
 // another, until they are worth one: with one warp at least for every block,
 // a split of eight blocks on eight warps took 2.6 times as long as its work
-// (Lx = 16, chi = 256, 256 chains: 808 -> 750 ms a step; but 16 chains of Lx = 5,
-// where the warps are plenty, 77 -> 84 ms, hence the first case).  Then the
+// (Lx = 16, chi = 256, 256 chains: 808 -> 750 ms a step when it was made, 392 ms with
+// the steps after it; but 16 chains of Lx = 5, where the warps are plenty, 77 -> 84 ms, hence
+// the first case).  Then the
 // warps go one at a time to the group that takes longest, at most p / 2 to
 // one.  Writes every block's group and every group's first warp and warp
 // count; returns the groups.  One thread.

@@ -14,8 +14,9 @@
 // constant larger than every partial sum splits exactly too: dot2 below spends
 // seven binary32 instructions a term (64 x the rate of the binary64 pipe) and
 // returns the Gram entry to about 2^-45 of the columns' norms.  Measured on Lx =
-// 16, 2W = 8, chi = 256 (256 chains, beta = 0.3): the evolution 1043 -> 800 ms,
-// sweep, promotion to binary64 and the scales together 37 -> about 15 % of it.
+// 16, 2W = 8, chi = 256 (256 chains, beta = 0.3) when it was made: the evolution
+// 1043 -> 800 ms, sweep, promotion to binary64 and the scales together 37 -> about
+// 15 % of it (the whole step is 392 ms with the steps after it).
 //
 // Two columns of nearly the same norm have a large angle whatever their
 // overlap; their pairs (|b - a| < kNear max(a, b)) are left out of K and
